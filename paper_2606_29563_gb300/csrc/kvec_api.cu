@@ -618,6 +618,7 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
     if (e == cudaSuccess) e = configure_score(G);
     if (e == cudaSuccess) e = configure_window(G);
     if (e == cudaSuccess) e = configure_select();
+    if (e == cudaSuccess) e = configure_decode();
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&h->prio_lo, &h->prio_hi);
     for (cudaStream_t* st : {&h->s_score, &h->s_gather, &h->s_cap})
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(st, cudaStreamNonBlocking, h->prio_lo);
@@ -1021,7 +1022,7 @@ kvec_status kvec_decode_attention(kvec_handle* h, int batch, const void* q, cons
     io.Hkv = p.num_kv_heads;
     io.cap = cap;
     io.scale = p.softmax_scale > 0.f ? p.softmax_scale : (float)(1.0 / sqrt((double)p.head_dim));
-    cudaError_t e = launch_decode(io, reinterpret_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_decode(io, h->num_sms, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "decode attention launch");
     return KVEC_OK;
 }

@@ -198,8 +198,8 @@ cudaError_t launch_finalize(const Geometry& g, const LayerIO& io, const Scratch&
 // the layer's selection (it waits for it).
 cudaError_t launch_ada(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl, cudaStream_t st,
                        int priority, int ncall);
+cudaError_t launch_decode(const DecodeIO& io, int num_sms, cudaStream_t st);
 // out_idx from the slot's kept-position bits, then the K/V rows.
-cudaError_t launch_decode(const DecodeIO& io, cudaStream_t st);
 void launch_gather(const Geometry& g, const LayerIO& io, const Slot& sl, cudaStream_t st);
 
 // Fault injected by kvec_set_test_fault (0: none), read when a kernel is launched.
@@ -210,5 +210,6 @@ size_t window_smem_bytes(const Geometry& g);
 cudaError_t configure_score(const Geometry& g);
 cudaError_t configure_window(const Geometry& g);
 cudaError_t configure_select();
+cudaError_t configure_decode();
 
 }  // namespace kvec

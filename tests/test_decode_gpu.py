@@ -96,6 +96,24 @@ def test_long_caches_span_several_tiles_per_split(cap, n):
     _check(sel, q, k, v, [n])
 
 
+@pytest.mark.parametrize("Hq,Hkv", [(8, 8), (8, 4), (32, 8), (40, 8), (64, 8)])
+@pytest.mark.parametrize("batch", [10, 20, 40, 80])
+def test_batches_over_every_cluster_size(batch, Hq, Hkv):
+    # batch * Hkv pairs take clusters of 8, 4, 2 or 1 CTAs; lengths around the
+    # eight-row blocks, the eight warps' first round and the ring's depth, empty
+    # caches between them, and NaN in every row past a sequence's length.
+    cap = 530
+    gen = torch.Generator().manual_seed(batch * 7 + Hq)
+    lens = [(0, 1, 7, 8, 9, 63, 64, 65, 129, 191, 193, 255, 257, 511, 513, 530)[(3 * b + b // 16) % 16] for b in range(batch)]
+    q = _rand((batch, Hq, 128), gen)
+    k = torch.randn((batch, Hkv, cap, 128), generator=gen).to(torch.bfloat16)
+    v = torch.randn((batch, Hkv, cap, 128), generator=gen).to(torch.bfloat16)
+    for b, n in enumerate(lens):
+        k[b, :, n:] = float("nan")
+        v[b, :, n:] = float("nan")
+    _check(_selector(Hq, Hkv, max_batch=batch), q, k.cuda(), v.cuda(), lens)
+
+
 def test_peaked_softmax_and_garbage_past_lens():
     gen = torch.Generator().manual_seed(7)
     sel = _selector(8, 2)
