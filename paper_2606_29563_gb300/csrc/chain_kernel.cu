@@ -1,0 +1,427 @@
+// Section 4.2 over a run of consecutive layers: P' = P + lambda * I * (1 - n_t /
+// (l + 1)), the preserved tokens stay, the rest of B - w goes to the largest P',
+// the last w tokens are kept, and the layer's union moves the coverage counts.
+//
+// Only this step is serial across layers, so one launch walks all the layers
+// whose scores are ready.  A cluster of Hkv CTAs serves a sequence, a CTA per KV
+// head: every thread keeps the counts n_t of its positions in registers, builds
+// their keys in registers, and the heads' kept bits meet over distributed shared
+// memory behind one cluster barrier per layer, under which the next layer's
+// scores are already being loaded.  Per-layer launches instead pass the union
+// and the counts through L2 and stage the keys in shared memory: 14 to 17 us per
+// layer of one 8192-token sequence where this takes about 4.
+#include <cooperative_groups.h>
+
+#include "hist_select.cuh"
+
+namespace kvec {
+
+namespace {
+
+namespace cg = cooperative_groups;
+
+struct ChainArgs {
+    Geometry G;
+    const int* cu;
+    uint8_t* state;
+    int* refused;      // [batch] 1: the call would take this state past 255 layers (set by its first launch)
+    int* err;
+    int l0, nl, ncall; // layers [l0, l0 + nl) of a call of ncall
+    Slot sl[kMaxGroup];
+};
+
+// What the CTAs of a cluster read from each other in a joint selection.
+struct JointShared {
+    uint32_t kmin, kmax;
+    int total;                            // keys in this CTA's slice of the buckets
+    int bin, above, count;                // the bucket of the k-th key, in the CTA whose slice holds it
+    int fill;                             // list entries, or equal keys
+    unsigned long long list[kSelList];    // this head's keys in that bucket: key << 32 | ~(head, position)
+};
+
+// The k largest of the keys in `active` over every CTA of the cluster (a KV head
+// each), ORed into their heads' bits; ties go to the lower head, then to the lower
+// position.  HistSelect's buckets, over the cluster's range of keys: each CTA
+// counts its own keys, CTA r adds up the r-th slice of the buckets from the top,
+// and the one whose slice holds the k-th key names its bucket.  At least k keys
+// are active.  The bits are complete after the next block barrier.
+template <int NT, int KPT>
+__device__ __noinline__ void joint_select(const uint32_t* keys, uint32_t active, int k, HistSelectShared& sm,
+                                          JointShared& js, uint32_t* bits) {
+    using HS = HistSelect<NT, KPT>;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nc = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t key[KPT];
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        key[i] = keys[i];
+        if ((active >> i) & 1u) {
+            kmin = min(kmin, key[i]);
+            kmax = max(kmax, key[i]);
+        }
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+        sm.wmin[warp] = kmin;
+        sm.wmax[warp] = kmax;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < HS::kWarps; ++w) {
+            kmin = min(kmin, sm.wmin[w]);
+            kmax = max(kmax, sm.wmax[w]);
+        }
+        js.kmin = kmin;
+        js.kmax = kmax;
+        js.fill = 0;
+    }
+    cluster.sync();
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    if (lane < nc) {
+        lo = *cluster.map_shared_rank(&js.kmin, lane);
+        hi = *cluster.map_shared_rank(&js.kmax, lane);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    int shift = max(32 - kSelBits - __clz(hi - lo), 0);
+    const int slice = (kSelBins + nc - 1) / nc, per = (slice + NT - 1) / NT;   // buckets of a CTA, of a thread
+    uint32_t sure = 0u, match = 0u;
+    int kk = k, m = 0;
+    for (;;) {
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if ((active >> i) & 1u) atomicAdd(&sm.hist[(key[i] - lo) >> shift], 1u);
+        cluster.sync();
+        // Buckets from the top: this CTA's slice, this thread's `per` of it.
+        int own = 0;
+        for (int b = 0; b < per; ++b) {
+            const int i = tid * per + b, bin = kSelBins - 1 - (rank * slice + i);
+            if (i >= slice || bin < 0) break;
+            for (int r = 0; r < nc; ++r) own += (int)*cluster.map_shared_rank(&sm.hist[bin], r);
+        }
+        int incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) sm.wsum[warp] = incl;
+        __syncthreads();
+        const int ws = lane < HS::kWarps ? sm.wsum[lane] : 0;
+        const int total = __reduce_add_sync(0xffffffffu, ws);
+        int before = __reduce_add_sync(0xffffffffu, lane < warp ? ws : 0) + incl - own;
+        if (tid == 0) js.total = total;
+        cluster.sync();
+        int owner = 0, above = 0;   // the CTA whose slice holds the kk-th key, and the keys in the slices above it
+        for (; owner + 1 < nc; ++owner) {
+            const int t = *cluster.map_shared_rank(&js.total, owner);
+            if (kk <= above + t) break;
+            above += t;
+        }
+        if (owner == rank && above + before < kk && kk <= above + before + own) {
+            int at = above + before;
+            for (int b = 0; b < per; ++b) {
+                const int bin = kSelBins - 1 - (rank * slice + tid * per + b);
+                if (tid * per + b >= slice || bin < 0) break;
+                int c = 0;
+                for (int r = 0; r < nc; ++r) c += (int)*cluster.map_shared_rank(&sm.hist[bin], r);
+                if (at < kk && kk <= at + c) {
+                    js.bin = bin;
+                    js.above = at;
+                    js.count = c;
+                }
+                at += c;
+            }
+        }
+        cluster.sync();
+        HS::clear(sm);   // every count has been read
+        const uint32_t bin = (uint32_t)*cluster.map_shared_rank(&js.bin, owner);
+        kk -= *cluster.map_shared_rank(&js.above, owner);
+        m = *cluster.map_shared_rank(&js.count, owner);
+        match = 0u;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) {
+            const uint32_t on = (active >> i) & 1u, d = (key[i] - lo) >> shift;
+            sure |= (on & (d > bin ? 1u : 0u)) << i;
+            match |= (on & (d == bin ? 1u : 0u)) << i;
+        }
+        if (m == kk || m <= kSelList || shift == 0) break;
+        active = match;
+        lo += bin << shift;
+        shift = max(shift - kSelBits, 0);
+        __syncthreads();   // the counters are clear
+    }
+    if (m == kk) {   // the bucket is taken whole
+        HS::store_or(sure | match, bits);
+        return;
+    }
+    HS::store_or(sure, bits);
+    if (m <= kSelList) {
+        // The heads' entries of the bucket side by side, ranked against each other.
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if ((match >> i) & 1u)
+                js.list[atomicAdd(&js.fill, 1)] =
+                    ((unsigned long long)key[i] << 32) | (uint32_t)~(((uint32_t)rank << 24) | (uint32_t)HS::position(i));
+        cluster.sync();
+        int at = 0;
+        for (int r = 0; r < nc; ++r) {
+            const int n = *cluster.map_shared_rank(&js.fill, r);
+            for (int e = tid; e < n; e += NT) sm.list[at + e] = *cluster.map_shared_rank(&js.list[e], r);
+            at += n;
+        }
+        __syncthreads();
+        if (tid < m) {
+            const unsigned long long mine = sm.list[tid];
+            const uint32_t where = ~(uint32_t)mine;
+            if ((int)(where >> 24) == rank) {
+                int better = 0;
+                for (int j = 0; j < m; ++j) better += sm.list[j] > mine ? 1 : 0;
+                const uint32_t pos = where & 0xffffffu;
+                if (better < kk) atomicOr(&bits[pos >> 5], 1u << (pos & 31));
+            }
+        }
+        return;
+    }
+    // More than kSelList equal keys: the lower heads', then the lower positions'.
+    const int c = __reduce_add_sync(0xffffffffu, __popc(match));
+    if (lane == 0 && c) atomicAdd(&js.fill, c);
+    cluster.sync();
+    for (int r = 0; r < rank; ++r) kk -= *cluster.map_shared_rank(&js.fill, r);
+    HS::store_or(HS::lowest(sm, match, max(kk, 0)), bits);
+}
+
+template <int NT, int KPT, bool ADA>
+__global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ ChainArgs A) {
+    using HS = HistSelect<NT, KPT>;
+    __shared__ HistSelectShared sm;
+    __shared__ __align__(16) uint32_t bits[2][HS::kWords];   // this head's kept positions, by layer parity
+    __shared__ __align__(16) uint32_t uni[HS::kWords];       // the last layer's union
+    __shared__ JointShared js[1];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int h = (int)cluster.block_rank(), s = blockIdx.y;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int Hkv = A.G.Hkv, words = A.G.words, budget = A.G.budget;
+    const int L = __ldg(&A.cu[s + 1]) - __ldg(&A.cu[s]);
+    const int Lc = L - A.G.wk;
+    const int wordsL = (L + 31) >> 5;
+    const bool select = L > budget;
+    const size_t row = (size_t)s * Hkv + h;
+    uint8_t* st = A.state + (size_t)s * A.G.state_stride;
+    uint8_t* nst = st + A.G.state_n_off;
+    const uint32_t ell0 = __ldcg(reinterpret_cast<const uint32_t*>(st));   // layers before this launch
+    // n_t is 8-bit: a state may count at most 255 layers.  Every launch of a
+    // refused call leaves the state as it was.
+    const bool refuse = A.l0 == 0 ? ell0 + (uint32_t)A.ncall > 255u : __ldcg(&A.refused[s]) != 0;
+    if (A.l0 == 0 && h == 0 && tid == 0) A.refused[s] = refuse ? 1 : 0;
+    if (refuse) {   // the same for the whole cluster
+        if (tid == 0) atomicExch(A.err, 2);
+        return;
+    }
+    uint32_t n4[KPT / 4];   // counts of this thread's positions, four bytes a word
+#pragma unroll
+    for (int g = 0; g < KPT / 4; ++g) {
+        const int t = HS::position(4 * g);
+        n4[g] = t < L ? __ldcg(reinterpret_cast<const uint32_t*>(nst + t)) : 0u;
+    }
+    HS::clear(sm);
+    // Sixteen values of a thread at a time: its scores, and the preserved bits.
+    float4 p[4], im[4];
+    uint32_t pw[4];
+    auto load = [&](int l, int part) {
+        const Slot& sl = A.sl[l];
+        const float* P = (__ldg(&sl.htop[row]) ? sl.POe : sl.PO) + row * A.G.ML;
+        const float* I = sl.I + (size_t)s * A.G.ML;
+        const uint32_t* pres = sl.pres + row * words;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int t = HS::position(16 * part + 4 * g);
+            if (t < Lc) {
+                p[g] = __ldg(reinterpret_cast<const float4*>(P + t));
+                im[g] = __ldg(reinterpret_cast<const float4*>(I + t));
+                pw[g] = __ldg(&pres[t >> 5]) >> (t & 31);
+            }
+        }
+    };
+    // With 64 registers a thread (NT = 1024) there is no room for the next layer's
+    // scores while this one's are ranked.
+    constexpr bool kAhead = NT < 1024;
+    if (kAhead && select) load(0, 0);
+    __syncthreads();
+    for (int l = 0; l < A.nl; ++l) {
+        uint32_t* b = bits[l & 1];
+        uint32_t keep = 0u;   // positions kept without ranking: preserved tokens and the kept tail
+        if (select) {
+            const float inv_l1 = __frcp_rn((float)(ell0 + (uint32_t)l + 1u));
+            // P' of the last layer of a call is kept for inspection (kvec_debug_scores).
+            float* Pp = A.l0 + l + 1 == A.ncall ? A.sl[l].Pprime + row * A.G.ML : nullptr;
+            uint32_t key[KPT];
+#pragma unroll
+            for (int part = 0; part < KPT / 16; ++part) {
+                if (!kAhead || part > 0) load(l, part);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const int i0 = 16 * part + 4 * g, t0 = HS::position(i0);
+                    const float p4[4] = {p[g].x, p[g].y, p[g].z, p[g].w};
+                    const float i4[4] = {im[g].x, im[g].y, im[g].z, im[g].w};
+                    float out[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int t = t0 + e;
+                        key[i0 + e] = 0u;
+                        if (t < Lc) {
+                            // coverage = n_t / (l + 1), by the rounded reciprocal
+                            const float coverage = (float)((n4[i0 / 4] >> (8 * e)) & 255u) * inv_l1;
+                            const float pp = p4[e] + A.G.lambda * (i4[e] * (1.f - coverage));
+                            out[e] = pp;
+                            const uint32_t kept = (pw[g] >> e) & 1u;
+                            keep |= kept << (i0 + e);
+                            if (!kept) key[i0 + e] = float_order_key(pp);
+                        } else {
+                            out[e] = 0.f;
+                            keep |= (t < L ? 1u : 0u) << (i0 + e);
+                        }
+                    }
+                    if (Pp && t0 < Lc) *reinterpret_cast<float4*>(Pp + t0) = make_float4(out[0], out[1], out[2], out[3]);
+                }
+            }
+            if (A.G.f0 > 0) {
+                HS hs{sm, A.G.f0};
+                uint32_t match;
+                keep |= hs.begin(key, match);
+                HS::store(keep, b);
+                hs.finish(key, match, b);
+            } else {
+                HS::store(keep, b);
+            }
+            if constexpr (ADA) {
+                // Head-wise adaptive fill: the sequence's other extras = Hkv * (k2 - f0)
+                // slots go to the best of all heads' remaining candidates.  (Preserved
+                // tokens are exactly Kp of the Lc candidates, so there are enough.)
+                if (A.G.extras > 0) {
+                    __syncthreads();
+                    uint32_t rest = 0u;
+#pragma unroll
+                    for (int i = 0; i < KPT; ++i) {
+                        const int t = HS::position(i);
+                        rest |= (key[i] != 0u && !((b[t >> 5] >> (t & 31)) & 1u) ? 1u : 0u) << i;
+                    }
+                    __syncthreads();   // the bits have been read
+                    joint_select<NT, KPT>(key, rest, A.G.extras, sm, js[0], b);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) keep |= (HS::position(i) < L ? 1u : 0u) << i;
+            HS::store(keep, b);
+        }
+        // The heads' kept bits: written above, read below by every CTA of the
+        // cluster.  A buffer is written again two layers on, after the next
+        // barrier, which every reader passes first.
+        auto token = cluster.barrier_arrive();
+        if (kAhead && select && l + 1 < A.nl) load(l + 1, 0);
+        cluster.barrier_wait(std::move(token));
+        // A warp's union words: lane (4 hh + c) takes four words of head hh.
+#pragma unroll
+        for (int part = 0; part < KPT / 16; ++part) {
+            const int w0 = warp * KPT + part * 16;
+            const int hh = lane >> 2;
+            uint4 u = make_uint4(0u, 0u, 0u, 0u);
+            if (hh < Hkv) u = *reinterpret_cast<const uint4*>(cluster.map_shared_rank(&b[w0 + (lane & 3) * 4], hh));
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {
+                u.x |= __shfl_xor_sync(0xffffffffu, u.x, o);
+                u.y |= __shfl_xor_sync(0xffffffffu, u.y, o);
+                u.z |= __shfl_xor_sync(0xffffffffu, u.z, o);
+                u.w |= __shfl_xor_sync(0xffffffffu, u.w, o);
+            }
+            __syncwarp();   // the last layer's words have been read
+            if (lane < 4) *reinterpret_cast<uint4*>(&uni[w0 + lane * 4]) = u;
+            __syncwarp();
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const uint32_t nib = (uni[w0 + g * 4 + (lane >> 3)] >> ((lane & 7) * 4)) & 15u;
+                n4[part * 4 + g] += (nib * 0x00204081u) & 0x01010101u;   // a byte per position: no count passes 255
+            }
+            // The head's kept positions, for the gather.
+            if (lane < 16 && w0 + lane < wordsL) A.sl[l].sel[row * words + w0 + lane] = b[w0 + lane];
+        }
+    }
+    // Counts, union and header for the next launch or call; the CTAs take slices
+    // of the positions (all counts were read before the first barrier).
+    const int fper = (((L + Hkv - 1) / Hkv) + 31) & ~31;
+    const int f0 = min(h * fper, L), f1 = min(f0 + fper, L);
+#pragma unroll
+    for (int g = 0; g < KPT / 4; ++g) {
+        const int t = HS::position(4 * g);
+        if (t < f0 || t >= f1) continue;
+        if (t + 4 <= L) {
+            *reinterpret_cast<uint32_t*>(nst + t) = n4[g];
+        } else {
+            for (int e = 0; t + e < L; ++e) nst[t + e] = (uint8_t)(n4[g] >> (8 * e));
+        }
+    }
+    if (h == 0) {
+        uint32_t* last_union = reinterpret_cast<uint32_t*>(st + A.G.state_union_off);
+        for (int w = lane; w < KPT; w += 32) {
+            const int wd = warp * KPT + w;
+            if (wd < words) last_union[wd] = wd < wordsL ? uni[wd] : 0u;
+        }
+        for (int wd = HS::kWords + tid; wd < words; wd += NT) last_union[wd] = 0u;
+        if (tid == 0) {
+            reinterpret_cast<uint32_t*>(st)[0] = ell0 + (uint32_t)A.nl;
+            reinterpret_cast<uint32_t*>(st)[1] = (uint32_t)L;
+        }
+    }
+    cluster.sync();   // no CTA leaves while another still reads its bits
+}
+
+template <int NT, int KPT, bool ADA>
+cudaError_t launch_one(const ChainArgs& a, cudaStream_t st, int priority) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.G.Hkv, a.G.batch);
+    cfg.blockDim = dim3(NT);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = a.G.Hkv;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributePriority;
+    attr[1].val.priority = priority;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, chain_kernel<NT, KPT, ADA>, a);
+}
+
+template <bool ADA>
+cudaError_t launch_for(const Geometry& g, const ChainArgs& a, cudaStream_t st, int priority) {
+    if (g.max_len <= 256 * 16) return launch_one<256, 16, ADA>(a, st, priority);
+    if (g.max_len <= 512 * 16) return launch_one<512, 16, ADA>(a, st, priority);
+    if (g.max_len <= 512 * 32) return launch_one<512, 32, ADA>(a, st, priority);
+    return launch_one<1024, 32, ADA>(a, st, priority);
+}
+
+}  // namespace
+
+bool chain_fits(const Geometry& g) { return g.Hkv <= kMaxClusterHeads && g.max_len <= kMaxRegisterRow; }
+
+cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, int l0, int ncall, cudaStream_t st,
+                         int priority) {
+    ChainArgs a{};
+    a.G = g;
+    a.cu = gr.io[0].cu;
+    a.state = gr.io[0].state;
+    a.refused = sc.refused;
+    a.err = sc.err;
+    a.l0 = l0;
+    a.nl = gr.nl;
+    a.ncall = ncall;
+    for (int l = 0; l < gr.nl; ++l) a.sl[l] = gr.sl[l];
+    return g.ada ? launch_for<true>(g, a, st, priority) : launch_for<false>(g, a, st, priority);
+}
+
+}  // namespace kvec

@@ -62,8 +62,11 @@ struct TimedLaunch {
 
 int kvec::test_fault() { return g_test_fault.load(std::memory_order_relaxed); }
 
-constexpr int kSlots = 8;   // per-layer score arrays in flight between the score and select stages
-constexpr int kScoreBufs = 2;   // segment-partial buffers in flight between the score and row-statistics stages
+constexpr int kSlots = 4 * kMaxGroup;   // per-layer score arrays in flight between the score and select stages
+constexpr int kPartials = 2 * kMaxGroup;   // layers whose segment partials are in flight
+constexpr int kSelRing = 32;               // layers whose kept-position bits are in flight to the gather
+constexpr size_t kSlotBytes = size_t(8) << 30;
+constexpr size_t kPartialsBytes = size_t(128) << 20;   // for the segment partials of the layers in flight
 constexpr size_t kGraphCache = 16;  // captured multi-layer calls kept per handle
 
 struct kvec_handle {
@@ -74,11 +77,12 @@ struct kvec_handle {
     size_t state_stride = 0, n_off = 16, union_off = 0;
     void* ws = nullptr;
     size_t ws_bytes = 0;
-    int* claims = nullptr;   // [max_layers] the score launches' chunk counters (zero between launches)
+    int* claims = nullptr;   // [max_layers][2] the score and window launches' work counters (zero between launches)
     Scratch sc{};
-    Scratch score_buf[kScoreBufs]{};   // segment partials, one per layer in flight
-    Slot slots[kSlots]{};
-    float2* rowstat_slot[kSlots]{};    // row statistics of the layer in slot k (read by its window grid)
+    float2* segpart[kPartials]{};      // segment partials of the layers in flight, layer l in l % nsegpart
+    uint32_t* sel[kSelRing]{};         // kept positions, layer l in l % nsel
+    int nsegpart = 0, nslots = 0, nsel = 0;
+    Slot slots[kSlots]{};              // layer l in l % nslots (its sel pointer is set per call)
     int last_slot = 0;
     int last_batch = 0;
     bool profiling = false;
@@ -99,6 +103,7 @@ struct kvec_handle {
     struct CachedGraph {
         std::vector<uint64_t> key;
         cudaGraphExec_t exec;
+        int last_slot;
     };
     std::vector<CachedGraph> graphs;
     std::vector<std::vector<uint64_t>> seen_keys;
@@ -210,7 +215,7 @@ struct DeviceGuard {
 };
 
 kvec_status validate_call(kvec_handle* h, int batch, const int32_t* cu_host, const int32_t* cu_dev, int budget,
-                          int* total_tiles, int* total_win_tiles) {
+                          int* total_tiles, int* total_win_tiles, int* max_len) {
     if (!h) return fail(KVEC_ERR_INVALID_ARG, "handle is NULL");
     if (batch < 1 || batch > h->p.max_batch)
         return fail(KVEC_ERR_INVALID_ARG, "batch %d outside [1, max_batch=%d]", batch, h->p.max_batch);
@@ -219,17 +224,19 @@ kvec_status validate_call(kvec_handle* h, int batch, const int32_t* cu_host, con
     const int wk = h->p.all_positions ? 0 : h->p.window;   // the tail kept unconditionally
     if (budget < 1) return fail(KVEC_ERR_INVALID_ARG, "budget %d < 1", budget);
     if (budget < wk) return fail(KVEC_ERR_INVALID_ARG, "budget %d < window %d", budget, wk);
-    int tiles = 0, chunks = 0;
+    int tiles = 0, chunks = 0, longest = 0;
     for (int b = 0; b < batch; ++b) {
         const int L = cu_host[b + 1] - cu_host[b];
         if (L < h->p.window || L > h->p.max_seqlen)
             return fail(KVEC_ERR_INVALID_ARG, "sequence %d has length %d outside [window=%d, max_seqlen=%d]", b, L,
                         h->p.window, h->p.max_seqlen);
         tiles += (L + kTileT - 1) / kTileT;
+        longest = std::max(longest, L);
         chunks += (L - wk + kTileT - 1) / kTileT;   // candidate tiles of the window kernel
     }
     *total_tiles = tiles;
     *total_win_tiles = chunks;
+    *max_len = longest;
     return KVEC_OK;
 }
 
@@ -237,7 +244,8 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 constexpr int kDecodeMaxCap = 1 << 20;   // cached rows per (sequence, KV head) a decode call may pass
 
-Geometry make_geometry(const kvec_handle* h, int batch, int budget, int tiles, int chunks, int total_tokens) {
+Geometry make_geometry(const kvec_handle* h, int batch, int budget, int tiles, int chunks, int total_tokens,
+                       int max_len) {
     const kvec_params& p = h->p;
     Geometry G{};
     G.Hq = p.num_q_heads;
@@ -270,9 +278,11 @@ Geometry make_geometry(const kvec_handle* h, int batch, int budget, int tiles, i
     G.HG = p.num_kv_heads < kWinHeadsPerCta ? p.num_kv_heads : kWinHeadsPerCta;
     G.NG = (p.num_kv_heads + G.HG - 1) / G.HG;
     G.total_tokens = total_tokens;
+    G.max_len = max_len;
     G.state_stride = h->state_stride;
     G.state_n_off = h->n_off;
     G.state_union_off = h->union_off;
+    G.jm = tile_variant_fits(G) ? 1 : 0;
     G.nlen = (int)round_up((size_t)p.max_seqlen, 16);
     return G;
 }
@@ -280,23 +290,34 @@ Geometry make_geometry(const kvec_handle* h, int batch, int budget, int tiles, i
 // One layer, every kernel on one stream with one slot (used without a handle).
 kvec_status run_layer_sequential(kvec_handle* h, const Geometry& G, const LayerIO& io, cudaStream_t st) {
     ScorePlan plan;
-    cudaError_t se = plan_score(G, io, h->sc, h->num_sms, &plan);
+    Group gr{};
+    gr.nl = 1;
+    gr.io[0] = io;
+    gr.sl[0] = h->slots[0];
+    gr.segpart[0] = h->segpart[0];
+    cudaError_t se = plan_score(G, gr, h->num_sms, &plan);
     if (se != cudaSuccess) return cuda_fail(se, "score kernel tensor maps");
-    se = launch_score(plan, h->claims, st, false);
+    se = launch_score(plan, G, gr, h->sc, h->claims, st, false);
     if (se != cudaSuccess) return cuda_fail(se, "score kernel launch");
-    se = launch_rowstat(plan, G, io, h->sc, h->claims, st, /*programmatic=*/true, /*after_score=*/true);
+    se = launch_rowstat(plan, G, gr, h->claims, st, /*programmatic=*/true, /*after_score=*/true);
     if (se != cudaSuccess) return cuda_fail(se, "row statistics launch");
-    se = launch_window(plan, G, io, h->sc, h->slots[0], st, false);
+    se = launch_window(plan, G, gr, h->sc, h->claims, st, false);
     if (se != cudaSuccess) return cuda_fail(se, "window kernel launch");
-    se = launch_heads(G, io, h->sc, h->slots[0], st, h->prio_hi);
+    se = launch_heads(G, gr, h->sc, h->claims, st, h->prio_hi);
     if (se != cudaSuccess) return cuda_fail(se, "heads kernel launch");
-    se = launch_select(G, io, h->sc, h->slots[0], nullptr, st, h->prio_hi, 0, 1, /*programmatic=*/false);
-    if (se != cudaSuccess) return cuda_fail(se, "select kernel launch");
-    launch_gather(G, io, h->slots[0], st);
-    se = launch_finalize(G, io, h->sc, h->slots[0], st, h->prio_hi, 1);
-    if (se != cudaSuccess) return cuda_fail(se, "finalize kernel launch");
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+    if (chain_fits(G)) {
+        se = launch_chain(G, gr, h->sc, 0, 1, st, h->prio_hi);
+        if (se != cudaSuccess) return cuda_fail(se, "chain kernel launch");
+    } else {
+        se = launch_select(G, io, h->sc, h->slots[0], nullptr, st, h->prio_hi, 0, 1, /*programmatic=*/false);
+        if (se != cudaSuccess) return cuda_fail(se, "select kernel launch");
+    }
+    se = launch_gather(G, gr, st);
+    if (se != cudaSuccess) return cuda_fail(se, "gather kernel launch");
+    if (!chain_fits(G)) {
+        se = launch_finalize(G, io, h->sc, h->slots[0], st, h->prio_hi, 1);
+        if (se != cudaSuccess) return cuda_fail(se, "finalize kernel launch");
+    }
     return KVEC_OK;
 }
 
@@ -348,99 +369,129 @@ cudaError_t restore_full_edges(cudaGraph_t graph, const std::vector<std::pair<cu
         if (e_ != cudaSuccess) return cuda_fail(e_, #call);   \
     } while (0)
 
-// Layers 0..n-1 as a five-stream pipeline.  Only the coverage-adjusted select
-// is serial across layers (it carries n_t); the score, window and heads work of
-// later layers runs ahead of it, bounded by the double-buffered score scratch
-// and by the kSlots ring of per-layer score arrays.  The row statistics live
-// with the slot (for the window grid); a layer's score grid reuses the segment
-// partials of layer l - kScoreBufs after that layer's window grid, or, when the
-// score and window grids fit on the SMs together, as soon as its row
-// statistics are done with them (else an early score grid only takes SMs that
-// the window and heads kernels of the layers ahead need: measured slower).
-// With the caller's log-sum-exp there is no score grid, and the same wait
-// keeps at most two layers' window grids in flight.
+// Layers that share a launch: the persistent grids' start and end (about 10 us)
+// weigh less on more layers, so as many as the ring of slots and partials leaves
+// room for two groups of, and four groups or more of a long call.  The last groups
+// halve, as nothing overlaps the last one's selection.  (32 layers in us with 1 / 2
+// / 4 / 8 layers a launch: ragged batch of 8 prompts 2896 / 2624 / 2436 / 2327, one
+// prompt of 8192 tokens 816 / 571 / 452 / 421.)
+int group_layers(const kvec_handle* h, const Geometry& G, int n, int l0) {
+    if (G.max_len > kMaxRegisterRow) return 1;   // the heads kernels' key rows are one layer's
+    const int left = n - l0;
+    int gs = std::min({kMaxGroup, h->nslots / 2, h->nsegpart / 2, (n + 3) / 4, std::max((left + 1) / 2, 2), left});
+    return std::max(1, std::min(gs, 65535 / G.batch));
+}
+
+// Layers 0..n-1 as a pipeline of layer groups over five stages, each on a stream
+// (the heads stage on two, alternating).  Only the coverage-adjusted selection is
+// serial across layers (it carries n_t); the score, window and heads work of later
+// groups runs ahead of it, bounded by the ring of per-layer score arrays.  A
+// group's score grid reuses the segment partials of an earlier one after that
+// group's window grid, or, when the score and window grids fit on the SMs
+// together, as soon as its row statistics are done with them (else an early
+// score grid only takes SMs that the window and heads kernels of the layers
+// ahead need: measured slower).  With the caller's log-sum-exp there is no score
+// grid, and the same wait keeps at most two groups' window grids in flight.
 kvec_status launch_pipeline(kvec_handle* h, const Geometry& G, const LayerIO* ios, int n, cudaStream_t origin) {
     KV_CHECK(cudaEventRecord(h->ev_fork, origin));
     for (cudaStream_t st : {h->s_score, h->s_win, h->s_heads, h->s_heads2, h->s_chain, h->s_gather})
         KV_CHECK(cudaStreamWaitEvent(st, h->ev_fork, 0));
     cudaGraphNode_t prev_score = nullptr, prev_window = nullptr, prev_select = nullptr;   // captured (h->capturing)
-    for (int l = 0; l < n; ++l) {
-        const Slot& sl = h->slots[l % kSlots];
-        Scratch sc = h->score_buf[l % kScoreBufs];
-        sc.rowstat = h->rowstat_slot[l % kSlots];
-        const LayerIO& io = ios[l];
-        ScorePlan plan;
-        cudaError_t se = plan_score(G, io, sc, h->num_sms, &plan);
-        if (se != cudaSuccess) return cuda_fail(se, "score kernel tensor maps");
-        // Partials buffer reuse (window stream).
-        if (l >= kScoreBufs) {
-            const bool early = !io.lse && plan.grid + window_grid_size(plan, G, false) <= h->num_sms;
-            KV_CHECK(cudaStreamWaitEvent(h->s_score, early ? h->ev_rs[l - kScoreBufs] : h->ev_win[l - kScoreBufs], 0));
+    const bool chain = chain_fits(G), lse = ios[0].lse != nullptr;
+    cudaError_t se;
+    std::vector<int> group_of(n);   // group of every layer so far
+    for (int k = 0, l0 = 0, nl; l0 < n; ++k, l0 += nl) {
+        nl = group_layers(h, G, n, l0);
+        Group gr{};
+        gr.nl = nl;
+        for (int i = 0; i < nl; ++i) {
+            const int l = l0 + i;
+            group_of[l] = k;
+            gr.io[i] = ios[l];
+            h->slots[l % h->nslots].sel = h->sel[l % h->nsel];
+            gr.sl[i] = h->slots[l % h->nslots];
+            gr.segpart[i] = h->segpart[l % h->nsegpart];
         }
-        // The score grid of layer l > 0 is a programmatic dependent of layer
-        // l - 1's (it reads none of its results); the event wait above stays a
+        const int last = l0 + nl - 1;
+        ScorePlan plan;
+        se = plan_score(G, gr, h->num_sms, &plan);
+        if (se != cudaSuccess) return cuda_fail(se, "score kernel tensor maps");
+        // Partials buffer reuse, and at most two groups' score and window grids in flight.
+        if (k >= 2) {
+            const bool early = !lse && plan.grid + window_grid_size(plan, G, nl) <= h->num_sms;
+            KV_CHECK(cudaStreamWaitEvent(h->s_score, early ? h->ev_rs[k - 2] : h->ev_win[k - 2], 0));
+        }
+        if (!lse && last >= h->nsegpart) KV_CHECK(cudaStreamWaitEvent(h->s_score, h->ev_rs[group_of[last - h->nsegpart]], 0));
+        // The score grid of group k > 0 is a programmatic dependent of group
+        // k - 1's (it reads none of its results); the event wait above stays a
         // full dependency (restore_full_edges when captured).
-        if (!io.lse) {
-            timed_launch(h, 0, h->s_score, [&] { se = launch_score(plan, h->claims + l, h->s_score, l > 0); });
+        if (!lse) {
+            timed_launch(h, 0, h->s_score, [&] { se = launch_score(plan, G, gr, h->sc, h->claims + 2 * k, h->s_score, k > 0); });
             if (se != cudaSuccess) return cuda_fail(se, "score kernel launch");
             if (h->capturing) {
                 cudaGraphNode_t node = captured_tail(h->s_score);
                 if (!node) return fail(KVEC_ERR_CUDA, "score kernel: no captured node");
-                if (l > 0) h->prog_nodes.emplace_back(node, prev_score);
+                if (k > 0) h->prog_nodes.emplace_back(node, prev_score);
                 prev_score = node;
             }
         }
-        KV_CHECK(cudaEventRecord(h->ev_score[l], h->s_score));
+        KV_CHECK(cudaEventRecord(h->ev_score[k], h->s_score));
         // Window stream: the row statistics (after the score grid and, for slot
-        // reuse, after layer l - kSlots's selection and gather), then the window
+        // reuse, after an earlier group's selection), then the window
         // sums as their programmatic dependent (it waits before reading them).
-        KV_CHECK(cudaStreamWaitEvent(h->s_win, h->ev_score[l], 0));
-        if (l >= kSlots) {
-            KV_CHECK(cudaStreamWaitEvent(h->s_win, h->ev_sel[l - kSlots], 0));
-            KV_CHECK(cudaStreamWaitEvent(h->s_win, h->ev_gather[l - kSlots], 0));
-        }
-        // The row statistics are a programmatic dependent of the previous layer's
-        // window grid, which they do not wait for: they read only this layer's
-        // partials (full dependency above), and the statistics buffer they
-        // overwrite belongs to this layer's slot, last read by layer l - kSlots's
+        KV_CHECK(cudaStreamWaitEvent(h->s_win, h->ev_score[k], 0));
+        if (last >= h->nslots) KV_CHECK(cudaStreamWaitEvent(h->s_win, h->ev_sel[group_of[last - h->nslots]], 0));
+        // The row statistics are a programmatic dependent of the previous group's
+        // window grid, which they do not wait for: they read only this group's
+        // partials (full dependency above), and the statistics buffers they
+        // overwrite belong to this group's slots, last read by an earlier group's
         // window grid (the waits above).  So consecutive window grids overlap.
-        se = io.lse ? launch_rowstat_lse(G, io, sc, h->s_win, l > 0)
-                    : launch_rowstat(plan, G, io, sc, h->claims + l, h->s_win, l > 0, /*after_score=*/false);
+        se = lse ? launch_rowstat_lse(G, gr, h->s_win, k > 0)
+                 : launch_rowstat(plan, G, gr, h->claims + 2 * k, h->s_win, k > 0, /*after_score=*/false);
         if (se != cudaSuccess) return cuda_fail(se, "row statistics launch");
         if (h->capturing) {
             cudaGraphNode_t node = captured_tail(h->s_win);
             if (!node) return fail(KVEC_ERR_CUDA, "row statistics: no captured node");
-            if (l > 0) h->prog_nodes.emplace_back(node, prev_window);
+            if (k > 0) h->prog_nodes.emplace_back(node, prev_window);
         }
-        KV_CHECK(cudaEventRecord(h->ev_rs[l], h->s_win));
-        timed_launch(h, 1, h->s_win, [&] { se = launch_window(plan, G, io, sc, sl, h->s_win, true); });
+        KV_CHECK(cudaEventRecord(h->ev_rs[k], h->s_win));
+        timed_launch(h, 1, h->s_win, [&] { se = launch_window(plan, G, gr, h->sc, h->claims + 2 * k, h->s_win, true); });
         if (se != cudaSuccess) return cuda_fail(se, "window kernel launch");
         if (h->capturing) {
             prev_window = captured_tail(h->s_win);
             if (!prev_window) return fail(KVEC_ERR_CUDA, "window kernel: no captured node");
         }
-        KV_CHECK(cudaEventRecord(h->ev_win[l], h->s_win));
-        cudaStream_t s_h = (l & 1) ? h->s_heads2 : h->s_heads;
-        KV_CHECK(cudaStreamWaitEvent(s_h, h->ev_win[l], 0));
-        timed_launch(h, 2, s_h, [&] { se = launch_heads(G, io, sc, sl, s_h, h->prio_hi); });
+        KV_CHECK(cudaEventRecord(h->ev_win[k], h->s_win));
+        // (Rows beyond kMaxRegisterRow rank in key rows that every layer shares: one stream.)
+        cudaStream_t s_h = (k & 1) && G.max_len <= kMaxRegisterRow ? h->s_heads2 : h->s_heads;
+        KV_CHECK(cudaStreamWaitEvent(s_h, h->ev_win[k], 0));
+        timed_launch(h, 2, s_h, [&] { se = launch_heads(G, gr, h->sc, h->claims + 2 * k, s_h, h->prio_hi); });
         if (se != cudaSuccess) return cuda_fail(se, "heads kernel launch");
-        KV_CHECK(cudaEventRecord(h->ev_heads[l], s_h));
-        KV_CHECK(cudaStreamWaitEvent(h->s_chain, h->ev_heads[l], 0));
-        const Slot* prev = l > 0 ? &h->slots[(l - 1) % kSlots] : nullptr;
-        // The selection is a programmatic dependent of the previous layer's: it
-        // stages this layer's scores (behind the full dependency on the heads
-        // kernels) while that one drains.
-        timed_launch(h, 3, h->s_chain,
-                     [&] { se = launch_select(G, io, sc, sl, prev, h->s_chain, h->prio_hi, l, n, /*programmatic=*/true); });
-        if (se != cudaSuccess) return cuda_fail(se, "select kernel launch");
-        if (h->capturing) {
-            cudaGraphNode_t node = captured_tail(h->s_chain);
-            if (!node) return fail(KVEC_ERR_CUDA, "select kernel: no captured node");
-            h->prog_nodes.emplace_back(node, prev_select);
-            prev_select = node;
+        KV_CHECK(cudaEventRecord(h->ev_heads[k], s_h));
+        KV_CHECK(cudaStreamWaitEvent(h->s_chain, h->ev_heads[k], 0));
+        if (last >= h->nsel) KV_CHECK(cudaStreamWaitEvent(h->s_chain, h->ev_gather[group_of[last - h->nsel]], 0));
+        if (chain) {
+            timed_launch(h, 3, h->s_chain, [&] { se = launch_chain(G, gr, h->sc, l0, n, h->s_chain, h->prio_hi); });
+            if (se != cudaSuccess) return cuda_fail(se, "chain kernel launch");
         }
-        if (G.ada) {
-            se = launch_ada(G, io, sc, sl, h->s_chain, h->prio_hi, n);
+        for (int l = l0; !chain && l < l0 + gr.nl; ++l) {
+            // The selection is a programmatic dependent of the previous layer's: it
+            // stages this layer's scores (behind the full dependency on the heads
+            // kernels) while that one drains.
+            const Slot* prev = l > 0 ? &h->slots[(l - 1) % h->nslots] : nullptr;
+            const Slot& sl = gr.sl[l - l0];
+            timed_launch(h, 3, h->s_chain, [&] {
+                se = launch_select(G, ios[l], h->sc, sl, prev, h->s_chain, h->prio_hi, l, n, /*programmatic=*/true);
+            });
+            if (se != cudaSuccess) return cuda_fail(se, "select kernel launch");
+            if (h->capturing) {
+                cudaGraphNode_t node = captured_tail(h->s_chain);
+                if (!node) return fail(KVEC_ERR_CUDA, "select kernel: no captured node");
+                h->prog_nodes.emplace_back(node, prev_select);
+                prev_select = node;
+            }
+            if (!G.ada) continue;
+            se = launch_ada(G, ios[l], h->sc, sl, h->s_chain, h->prio_hi, n);
             if (se != cudaSuccess) return cuda_fail(se, "adaptive fill launch");
             if (h->capturing) {
                 cudaGraphNode_t node = captured_tail(h->s_chain);
@@ -449,15 +500,16 @@ kvec_status launch_pipeline(kvec_handle* h, const Geometry& G, const LayerIO* io
                 prev_select = node;
             }
         }
-        KV_CHECK(cudaEventRecord(h->ev_sel[l], h->s_chain));
-        KV_CHECK(cudaStreamWaitEvent(h->s_gather, h->ev_sel[l], 0));
-        timed_launch(h, 4, h->s_gather, [&] { launch_gather(G, io, sl, h->s_gather); });
-        KV_CHECK(cudaEventRecord(h->ev_gather[l], h->s_gather));
+        KV_CHECK(cudaEventRecord(h->ev_sel[k], h->s_chain));
+        KV_CHECK(cudaStreamWaitEvent(h->s_gather, h->ev_sel[k], 0));
+        timed_launch(h, 4, h->s_gather, [&] { se = launch_gather(G, gr, h->s_gather); });
+        if (se != cudaSuccess) return cuda_fail(se, "gather kernel launch");
+        KV_CHECK(cudaEventRecord(h->ev_gather[k], h->s_gather));
     }
+    h->last_slot = (n - 1) % h->nslots;
     // The last layer's union goes into the state.
-    {
-        cudaError_t se = launch_finalize(G, ios[n - 1], h->score_buf[(n - 1) % kScoreBufs], h->slots[(n - 1) % kSlots], h->s_chain,
-                                         h->prio_hi, n);
+    if (!chain) {
+        se = launch_finalize(G, ios[n - 1], h->sc, h->slots[h->last_slot], h->s_chain, h->prio_hi, n);
         if (se != cudaSuccess) return cuda_fail(se, "finalize kernel launch");
     }
     KV_CHECK(cudaGetLastError());
@@ -469,7 +521,6 @@ kvec_status launch_pipeline(kvec_handle* h, const Geometry& G, const LayerIO* io
     KV_CHECK(cudaEventRecord(h->ev_fork, h->s_chain));   // reused: the end of the chain stream
     KV_CHECK(cudaStreamWaitEvent(origin, h->ev_fork, 0));
     for (cudaEvent_t e : h->ev_join) KV_CHECK(cudaStreamWaitEvent(origin, e, 0));
-    h->last_slot = (n - 1) % kSlots;
     return KVEC_OK;
 }
 
@@ -562,20 +613,26 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
         {(void**)&h->sc.keys, MB * Hkv * ML * sizeof(uint32_t)},
         {(void**)&h->sc.nbuf, MB * round_up((size_t)p.max_seqlen, 16)},
         {(void**)&h->sc.err, sizeof(int)},
+        {(void**)&h->sc.refused, MB * sizeof(int)},
         {(void**)&h->sc.keys_sel, MB * Hkv * ML * sizeof(uint32_t)},
         {(void**)&h->sc.jkeys, p.head_budget ? MB * (Hkv * ML + 32) * sizeof(uint32_t) : 0},
         {(void**)&h->sc.jpos, p.head_budget ? MB * (Hkv * ML + 32) * sizeof(int32_t) : 0},
         {(void**)&h->sc.jbits, p.head_budget ? MB * (Hkv * ML + 32) / 32 * sizeof(uint32_t) : 0},
-        {(void**)&h->claims, (size_t)p.max_layers * sizeof(int)},
+        {(void**)&h->claims, 2 * (size_t)p.max_layers * sizeof(int)},
     };
-    for (int k = 0; k < kScoreBufs; ++k) {
-        Scratch& b = h->score_buf[k];
-        std::vector<Part> sp = {
-            {(void**)&b.segpart, max_tiles * Hkv * R * sizeof(float2)},
-        };
-        parts.insert(parts.end(), sp.begin(), sp.end());
-    }
-    for (int k = 0; k < kSlots; ++k) {
+    // Partials of as many layers as kPartialsBytes holds, of two at least.
+    Geometry Gmax = make_geometry(h, p.max_batch, p.window, 1, 1, p.window, p.window);
+    const size_t part_bytes = score_partial_bytes(Gmax, max_tiles);
+    h->nsegpart = (int)std::min<size_t>(kPartials, std::max<size_t>(2, kPartialsBytes / part_bytes));
+    h->nsel = std::min(p.max_layers, kSelRing);
+    for (int k = 0; k < h->nsel; ++k) parts.push_back({(void**)&h->sel[k], MB * Hkv * W * sizeof(uint32_t)});
+    for (int k = 0; k < h->nsegpart; ++k) parts.push_back({(void**)&h->segpart[k], part_bytes});
+    // Fewer slots (still a ring of groups) where all of them would take over kSlotBytes,
+    // and no more than a call has layers.
+    const size_t slot_bytes = (5 * MB * Hkv * ML + 2 * MB * ML + max_tiles * NGmax * p.obs_window * kTileT) * sizeof(float);
+    h->nslots = kSlots;
+    while (h->nslots > kMaxGroup && (slot_bytes * h->nslots > kSlotBytes || h->nslots / 2 >= p.max_layers)) h->nslots /= 2;
+    for (int k = 0; k < h->nslots; ++k) {
         Slot& sl = h->slots[k];
         std::vector<Part> sp = {
             {(void**)&sl.rawO, MB * Hkv * ML * sizeof(float)},  {(void**)&sl.rawOe, MB * Hkv * ML * sizeof(float)},
@@ -583,9 +640,8 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
             {(void**)&sl.POe, MB * Hkv * ML * sizeof(float)},   {(void**)&sl.I, MB * ML * sizeof(float)},
             {(void**)&sl.sigma, MB * Hkv * sizeof(float)},      {(void**)&sl.htop, MB * Hkv * sizeof(int)},
             {(void**)&sl.pres, MB * Hkv * W * sizeof(uint32_t)}, {(void**)&sl.Pprime, MB * Hkv * ML * sizeof(float)},
-            {(void**)&sl.sel, MB * Hkv * W * sizeof(uint32_t)},
             {(void**)&sl.wpart, max_tiles * NGmax * p.obs_window * kTileT * sizeof(float)},
-            {(void**)&h->rowstat_slot[k], MB * Hkv * R * sizeof(float2)},
+            {(void**)&sl.rowstat, MB * Hkv * R * sizeof(float2)},
         };
         parts.insert(parts.end(), sp.begin(), sp.end());
     }
@@ -604,16 +660,7 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
         *pt.dst = static_cast<char*>(h->ws) + off;
         off += round_up(pt.bytes, 256);
     }
-    for (Scratch& b : h->score_buf) {
-        b.keys = h->sc.keys;
-        b.keys_sel = h->sc.keys_sel;
-        b.jkeys = h->sc.jkeys;
-        b.jpos = h->sc.jpos;
-        b.jbits = h->sc.jbits;
-        b.nbuf = h->sc.nbuf;
-        b.err = h->sc.err;
-    }
-    Geometry G = make_geometry(h, 1, p.window, 1, 1, p.window);
+    Geometry G = make_geometry(h, 1, p.window, 1, 1, p.window, p.window);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess) e = configure_score(G);
     if (e == cudaSuccess) e = configure_window(G);
@@ -696,8 +743,8 @@ kvec_status select_layers_impl(kvec_handle* h, int num_layers, int batch, const 
                                const void* const* v, const float* const* lse, void* coverage_state, int budget,
                                int32_t* const* out_idx, void* const* out_k, void* const* out_v,
                                kvec_stream_t stream) {
-    int tiles = 0, chunks = 0;
-    kvec_status s = validate_call(h, batch, cu_seqlens_host, cu_seqlens_dev, budget, &tiles, &chunks);
+    int tiles = 0, chunks = 0, max_len = 0;
+    kvec_status s = validate_call(h, batch, cu_seqlens_host, cu_seqlens_dev, budget, &tiles, &chunks, &max_len);
     if (s != KVEC_OK) return s;
     if (num_layers < 1 || num_layers > h->p.max_layers)
         return fail(KVEC_ERR_INVALID_ARG, "num_layers %d outside [1, max_layers=%d]", num_layers, h->p.max_layers);
@@ -717,7 +764,7 @@ kvec_status select_layers_impl(kvec_handle* h, int num_layers, int batch, const 
     s = set_device(h, &prev);
     if (s != KVEC_OK) return s;
     DeviceGuard guard{prev, h->device};
-    Geometry G = make_geometry(h, batch, budget, tiles, chunks, cu_seqlens_host[batch]);
+    Geometry G = make_geometry(h, batch, budget, tiles, chunks, cu_seqlens_host[batch], max_len);
     G.cu_host = cu_seqlens_host;
     cudaStream_t st = (cudaStream_t)stream;
     std::vector<LayerIO> ios(num_layers);
@@ -741,7 +788,7 @@ kvec_status select_layers_impl(kvec_handle* h, int num_layers, int batch, const 
         for (size_t i = 0; i < h->graphs.size(); ++i) {
             if (h->graphs[i].key != key) continue;
             KV_CHECK(cudaGraphLaunch(h->graphs[i].exec, st));
-            h->last_slot = (num_layers - 1) % kSlots;
+            h->last_slot = h->graphs[i].last_slot;
             h->last_batch = batch;
             return KVEC_OK;
         }
@@ -773,7 +820,7 @@ kvec_status select_layers_impl(kvec_handle* h, int num_layers, int batch, const 
                 cudaGraphExecDestroy(h->graphs.front().exec);
                 h->graphs.erase(h->graphs.begin());
             }
-            h->graphs.push_back({key, exec});
+            h->graphs.push_back({key, exec, h->last_slot});
             KV_CHECK(cudaGraphLaunch(exec, st));
             h->last_batch = batch;
             return KVEC_OK;
@@ -892,8 +939,8 @@ kvec_status kvec_select_layer_noalloc(const kvec_params* params, int batch, cons
     tmp.state_stride = kvec_state_bytes(params->max_seqlen);
     tmp.n_off = 16;
     tmp.union_off = 16 + round_up((size_t)params->max_seqlen, 16);
-    int tiles = 0, chunks = 0;
-    s = validate_call(&tmp, batch, cu_seqlens_host, cu_seqlens_dev, budget, &tiles, &chunks);
+    int tiles = 0, chunks = 0, max_len = 0;
+    s = validate_call(&tmp, batch, cu_seqlens_host, cu_seqlens_dev, budget, &tiles, &chunks, &max_len);
     if (s != KVEC_OK) return s;
     if (!q_obs || !k || !v || !out_idx || !out_k || !out_v || !coverage_state)
         return fail(KVEC_ERR_INVALID_ARG, "NULL pointer argument");
@@ -913,11 +960,12 @@ kvec_status kvec_select_layer_noalloc(const kvec_params* params, int batch, cons
     const size_t NGv = (Hkv + HGv - 1) / HGv;
     Part parts[] = {
         {(void**)&tmp.sc.err, sizeof(int)},                   // error word, first: see noalloc_setup
-        {(void**)&tmp.claims, sizeof(int)},
+        {(void**)&tmp.claims, 2 * sizeof(int)},
+        {(void**)&tmp.sc.refused, nb * sizeof(int)},
         {(void**)&tmp.sc.nbuf, nb * round_up((size_t)params->max_seqlen, 16)},
-        {(void**)&tmp.sc.segpart, nt * Hkv * R * sizeof(float2)},
+        {(void**)&tmp.segpart[0], score_partial_bytes(make_geometry(&tmp, batch, budget, tiles, chunks, cu_seqlens_host[batch], max_len), nt)},
         {(void**)&tmp.slots[0].wpart, nt * NGv * (size_t)params->obs_window * kTileT * sizeof(float)},
-        {(void**)&tmp.sc.rowstat, nb * Hkv * R * sizeof(float2)},
+        {(void**)&tmp.slots[0].rowstat, nb * Hkv * R * sizeof(float2)},
         {(void**)&tmp.sc.keys, nb * Hkv * ML * sizeof(uint32_t)},
         {(void**)&tmp.sc.keys_sel, nb * Hkv * ML * sizeof(uint32_t)},
         {(void**)&tmp.slots[0].rawO, nb * Hkv * ML * sizeof(float)},
@@ -946,7 +994,7 @@ kvec_status kvec_select_layer_noalloc(const kvec_params* params, int batch, cons
     tmp.device = prev;
     e = cudaDeviceGetAttribute(&tmp.num_sms, cudaDevAttrMultiProcessorCount, prev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
-    Geometry G = make_geometry(&tmp, batch, budget, tiles, chunks, cu_seqlens_host[batch]);
+    Geometry G = make_geometry(&tmp, batch, budget, tiles, chunks, cu_seqlens_host[batch], max_len);
     G.cu_host = cu_seqlens_host;
     void* base = nullptr;
     s = noalloc_setup(prev, &base, G);
@@ -1037,7 +1085,7 @@ kvec_status kvec_debug_scores(kvec_handle* h, kvec_debug_view* out) {
     out->htop = sl.htop;
     out->pres_bits = sl.pres;
     out->Pprime = sl.Pprime;
-    out->row_stats = reinterpret_cast<const float*>(h->rowstat_slot[h->last_slot]);
+    out->row_stats = reinterpret_cast<const float*>(sl.rowstat);
     out->max_seqlen = (int)row_stride(h->p.max_seqlen);
     out->words_per_row = h->words;
     return KVEC_OK;

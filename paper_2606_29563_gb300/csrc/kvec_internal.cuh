@@ -15,6 +15,9 @@ constexpr int kMaxPool = 15;       // largest pool kernel (halo 7)
 constexpr int kSelectThreads = 512;
 constexpr int kMaxObsWindow = 64;  // largest O: the window kernel keeps O x 128 head maxima in shared memory
 constexpr int kWinHeadsPerCta = 8; // KV heads one window CTA processes
+constexpr int kMaxGroup = 8;       // consecutive layers one launch may serve
+constexpr int kMaxClusterHeads = 8;      // KV heads of a sequence that one (portable) cluster serves
+constexpr int kMaxRegisterRow = 32768;   // positions whose keys a block's registers hold
 
 // Sizes and hyper-parameters shared by every kernel of one call.
 struct Geometry {
@@ -22,7 +25,8 @@ struct Geometry {
     int wk;            // kept tail: w, or 0 when every position is a candidate; candidates [0, L - wk)
     int pool_avg;      // 1: average pool instead of max-pool
     int head_entropy;  // 1: rank heads by minus the entropy of pooled P_O instead of its std
-    int R;             // rows per KV head = g * w, ordered r = q * g + j
+    int R;             // rows per KV head = g * w; row statistics are ordered r = q * g + j
+    int jm;            // 1: a query tile's rows are ordered j * w + q (by query head), 0: q * g + j
     float lambda;
     float sl2;         // softmax scale * log2(e)
     int ML;            // max_seqlen: row stride of per-position workspace arrays
@@ -38,6 +42,7 @@ struct Geometry {
     int win_tiles;     // sum over sequences of ceil((L_s - wk) / kTileT): candidate tiles
     int HG, NG;        // KV heads per window CTA, window CTAs per candidate tile
     int total_tokens;  // cu_seqlens[batch]
+    int max_len;       // longest sequence of the call
     const int* cu_host;  // host copy of cu_seqlens (host-side planning only; not for device code)
     size_t state_stride;
     size_t state_n_off, state_union_off;
@@ -58,17 +63,17 @@ struct Slot {
     float* Pprime;        // [max_batch][Hkv][ML]
     float* wpart;         // [win_tiles][NG][O][kTileT] per-group head maxima of G_h[q][t] (NG > 1)
     uint32_t* sel;        // [max_batch][Hkv][words]  kept positions of the layer, one bit each
+    float2* rowstat;      // [max_batch][Hkv][R]    (row max in log2 units, softmax denominator)
 };
 
 struct Scratch {
-    float2* segpart;      // [total_tiles * Hkv][R] per-CTA segment (max, sum), keyed by the segment's first item
-    float2* rowstat;      // [max_batch][Hkv][R]    (row max in log2 units, softmax denominator), for inspection
     uint32_t* keys;       // [max_batch][Hkv][ML]   radix-select keys of the heads kernel
     uint32_t* keys_sel;   // [max_batch][Hkv][ML]   radix-select keys of the select kernel
     uint32_t* jkeys;      // [max_batch][jstride]   adaptive fill: the heads' joint candidates' keys (a key row)
     int32_t* jpos;        // [max_batch][jstride]   their positions (candidate i belongs to head i / jpool)
     uint32_t* jbits;      // [max_batch][jstride / 32] winners of the joint ranking, one bit per candidate
     uint8_t* nbuf;        // [max_batch][nlen]      second copy of n_t (the coverage counts alternate)
+    int* refused;         // [max_batch] the running call's refusal of a state (chain_kernel)
     int* err;             // device error word
 };
 
@@ -82,6 +87,15 @@ struct LayerIO {
     __nv_bfloat16* out_k;
     __nv_bfloat16* out_v;
     const float* lse;         // [batch][w][Hq] natural-log softmax denominators of the window rows, or null
+};
+
+// Consecutive layers that one launch serves: same sequences, their own inputs,
+// outputs and score arrays.
+struct Group {
+    int nl;
+    LayerIO io[kMaxGroup];
+    Slot sl[kMaxGroup];
+    float2* segpart[kMaxGroup];   // score kernel's partials: [segments][accumulators][R] (max, sum)
 };
 
 // One decoding step over a compacted cache (decode_kernel.cu).
@@ -120,40 +134,46 @@ __host__ __device__ __forceinline__ int tiles_of(int L) { return (L + kTileT - 1
 
 // ---------------------------------------------------------------- launchers
 
-// Host-side launch description of the score kernel (tensor maps encoded ahead of the launch).
+// Whether the tile-owning window kernel takes this geometry (its query tiles are
+// ordered by query head, Geometry::jm).
+bool tile_variant_fits(const Geometry& g);
+
+// Host-side launch description of a group's score and window kernels: tensor maps
+// of every layer's keys and window queries, encoded ahead of the launches.
 struct ScorePlan {
-    CUtensorMap kmap, qmap;
-    alignas(16) unsigned char args[512];
+    CUtensorMap kmap[kMaxGroup], qmap[kMaxGroup];
     int grid, threads, mb;   // mb: 128-row M-blocks per KV head
+    int items;               // (sequence, head, tile) work items of a layer
     int chunk;               // work items per claim of the score kernel (segment boundaries of its partials)
     size_t smem;
     int num_sms;             // SMs of the device (persistent grids are sized from it)
 };
-cudaError_t plan_score(const Geometry& g, const LayerIO& io, const Scratch& sc, int num_sms, ScorePlan* plan);
-// after_own_launch: the stream's previous kernel is the previous layer's launch
+cudaError_t plan_score(const Geometry& g, const Group& gr, int num_sms, ScorePlan* plan);
+// after_own_launch: the stream's previous kernel is the previous group's launch
 // of the same kernel (the multi-stream layer pipeline); the launch may then
 // overlap it (programmatic stream serialization), as it reads none of its results.
-// claim: an int in device memory, zero before the launch (the CTAs count the
-// work chunks they claim on it; the layer's launch_rowstat sets it back to
-// zero once the score grid has completed); a distinct one for every launch in flight.
-cudaError_t launch_score(const ScorePlan& plan, int* claim, cudaStream_t st, bool after_own_launch);
+// claim: two ints in device memory, zero before the launch (the CTAs of the score
+// and window grids count the work they claim on them; the group's launch_rowstat
+// sets the first back to zero once the score grid has completed, launch_heads the
+// second after the window grid); a distinct pair for every group in flight.
+cudaError_t launch_score(const ScorePlan& plan, const Geometry& g, const Group& gr, const Scratch& sc, int* claim,
+                         cudaStream_t st, bool after_own_launch);
 // (m_r, Z_r) from the score launch's partials.  programmatic: a programmatic
 // dependent of the stream's previous kernel.  after_score: that kernel is this
-// layer's score launch, waited for (griddepcontrol.wait) before the partials
+// group's score launch, waited for (griddepcontrol.wait) before the partials
 // are read; without it the partials must come through a full dependency and the
 // previous kernel (the layer pipeline's previous window grid) is not waited for.
-cudaError_t launch_rowstat(const ScorePlan& plan, const Geometry& g, const LayerIO& io, const Scratch& sc,
-                           int* claim, cudaStream_t st, bool programmatic, bool after_score);
+cudaError_t launch_rowstat(const ScorePlan& plan, const Geometry& g, const Group& gr, int* claim, cudaStream_t st,
+                           bool programmatic, bool after_score);
 // (m_r, Z_r) = (lse * log2(e), 1) from the caller's log-sum-exp (io.lse), in place
 // of the score and row-statistics launches.  programmatic: as for launch_rowstat
 // without after_score (it reads only the caller's input).
-cudaError_t launch_rowstat_lse(const Geometry& g, const LayerIO& io, const Scratch& sc, cudaStream_t st,
-                               bool programmatic);
-cudaError_t launch_window(const ScorePlan& sp, const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl,
+cudaError_t launch_rowstat_lse(const Geometry& g, const Group& gr, cudaStream_t st, bool programmatic);
+cudaError_t launch_window(const ScorePlan& sp, const Geometry& g, const Group& gr, const Scratch& sc, int* claim,
                           cudaStream_t st, bool after_own_launch);
-// CTAs of the grid launch_window starts for this layer (0 without candidates);
-// lse: the layer comes with the caller's log-sum-exp (io.lse).
-int window_grid_size(const ScorePlan& sp, const Geometry& g, bool lse);
+// CTAs of the grid launch_window starts for a group of nl layers (0 without
+// candidates).
+int window_grid_size(const ScorePlan& sp, const Geometry& g, int nl);
 // Launches kernel<<<grid, block, smem, st>>> with a scheduling priority (lower
 // numbers first; the range comes from cudaDeviceGetStreamPriorityRange) and,
 // with `programmatic`, as a programmatic dependent of the stream's previous
@@ -177,7 +197,7 @@ cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t 
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-cudaError_t launch_heads(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl, cudaStream_t st,
+cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, int* claim, cudaStream_t st,
                          int priority);
 // lcall: the layer's index within a call of ncall layers (0 for the first);
 // prev: the previous layer's slot (null for lcall = 0), whose kept-position
@@ -191,6 +211,11 @@ cudaError_t launch_heads(const Geometry& g, const LayerIO& io, const Scratch& sc
 // the stream's previous kernel wrote this layer's scores.
 cudaError_t launch_select(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl, const Slot* prev,
                           cudaStream_t st, int priority, int lcall, int ncall, bool programmatic);
+// The same for a group whose first layer is layer l0 of a call of ncall, in one
+// launch, state and header included; needs chain_fits(g).
+bool chain_fits(const Geometry& g);
+cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, int l0, int ncall, cudaStream_t st,
+                         int priority);
 cudaError_t launch_finalize(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& last, cudaStream_t st,
                             int priority, int ncall);
 // Adaptive fill: the layer's extra fill slots over every head of a sequence,
@@ -200,12 +225,14 @@ cudaError_t launch_ada(const Geometry& g, const LayerIO& io, const Scratch& sc, 
                        int priority, int ncall);
 cudaError_t launch_decode(const DecodeIO& io, int num_sms, cudaStream_t st);
 // out_idx from the slot's kept-position bits, then the K/V rows.
-void launch_gather(const Geometry& g, const LayerIO& io, const Slot& sl, cudaStream_t st);
+cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st);
 
 // Fault injected by kvec_set_test_fault (0: none), read when a kernel is launched.
 int test_fault();
 
 size_t score_smem_bytes(const Geometry& g);
+// Bytes of a layer's partials for `tiles` 128-token tiles in g.batch sequences.
+size_t score_partial_bytes(const Geometry& g, size_t tiles);
 size_t window_smem_bytes(const Geometry& g);
 cudaError_t configure_score(const Geometry& g);
 cudaError_t configure_window(const Geometry& g);

@@ -3,48 +3,56 @@
 // row r of KV head h, the row max m_r of s = <q_r, k_t> * scale (log2 units)
 // and Z_r = sum_t 2^(s_rt - m_r), causal on the window part.
 //
-// Persistent, warp-specialised, one CTA per SM; CTAs claim chunks of
-// consecutive work items (sequence s, KV head h, 128-token tile j)
-// from a per-launch counter, so a CTA that starts late (its SM held by other
-// kernels) takes fewer chunks instead of delaying the launch:
-//   warp 0      TMA producer: the KV head's g*w query rows (once per (s,h)) and
-//               a ring of 128-token K tiles, both 128-byte swizzled;
+// Persistent, warp-specialised, one CTA per SM; a launch serves a group of
+// layers, and its CTAs claim chunks of a layer's consecutive work items
+// (sequence s, KV head h, 128-token tile j) from a per-launch counter, so a CTA
+// that starts late (its SM held by other kernels) takes fewer chunks instead of
+// delaying the launch:
+//   warp 0      TMA producer: the KV head's g*w query rows (once per (s,h) of a
+//               chunk, two buffers) and a ring of 128-token K tiles, both
+//               128-byte swizzled;
 //   warp 1      one thread issues tcgen05.mma (M = 128 query rows per M-block,
 //               N = 128 tokens, K = 128 = d) into TMEM accumulators;
 //   warps 2..17 epilogue: groups of warps, one per TMEM accumulator, each
-//               taking every NB-th item; one thread per query row and all
-//               128 columns of the item: tcgen05.ld of its logits, their sum
+//               taking every NB-th item of a chunk; one thread per query row and
+//               all 128 columns of the item: tcgen05.ld of its logits, their sum
 //               of 2^(s - max), merged online into the thread's running
-//               (max, sum) of the CTA's contiguous segment of (s, h).
-// At the end of a segment (a run of one (s, h) inside a chunk) the groups merge
-// in shared memory and the CTA writes one (max, sum) partial per row, keyed by
-// the segment's first item; rowstat_kernel then merges the partials of a (s, h)
-// into (m_r, Z_r).  The segments are fixed by the chunk boundaries, not by which
+//               (max, sum) of the group's items of one (s, h) inside the chunk.
+// No stage waits for a chunk's end: the producer claims the next chunk while it
+// loads this one, its K tiles follow each other through the ring whatever chunk
+// they belong to, and every warp of the epilogue takes the chunks from the hand-
+// over slots by itself.  At the end of a segment (a run of one (s, h) inside a
+// chunk) each group writes one (max, sum) partial per row; rowstat_kernel merges
+// the groups' and then the segments' partials of a (s, h) into (m_r, Z_r).  The
+// segments and the groups' shares are fixed by the chunk boundaries, not by which
 // CTA claimed a chunk, so the results do not depend on the schedule.
 // The window kernel recomputes the logits with these statistics.
 #include <cudaTypedefs.h>
 
 #include "kvec_internal.cuh"
 #include "sm100_ptx.cuh"
+#include "tile_loads.cuh"
 
 namespace kvec {
 
 namespace {
 
-constexpr int kKStages = 4;                           // deepest K ring (fewer when shared memory is short)
+constexpr int kKStages = 6;                           // deepest K ring (fewer when shared memory is short)
 constexpr int kMaxSmem = 232448;                      // opt-in shared memory per CTA on sm_103
 constexpr int kKStageBytes = kTileT * kHeadDim * 2;   // 32 KB: two 64-column swizzled halves
 constexpr int kKHalfBytes = kTileT * 128;             // 16 KB
 constexpr uint32_t kTmemCols = 512;
 
-// Position of work item i: sequence s, KV head h, tile j.  Items are ordered
-// (s, h, j); sequence s owns ntiles(s) * Hkv consecutive items.  A CTA walks its
-// items in order, so the walker decodes once and then steps, reading the
-// sequence offsets (device memory) only when the sequence changes.
+constexpr int kSeqCache = 64;   // sequences whose first items the CTA keeps in shared memory
+
+// Position of work item i of a layer: sequence s, KV head h, tile j.  Items are
+// ordered (s, h, j); sequence s owns ntiles(s) * Hkv consecutive items.  A role
+// walks a chunk's items in order, so the walker decodes once and then steps.
 struct ItemWalker {
     const int* cu;
+    const int* first;             // [batch] first item of every sequence, or null (batch > kSeqCache)
     int batch, Hkv;
-    int s, h, j, ibase, ntiles;   // ibase: first item of (s, h)
+    int s, h, j, ntiles;
     int row0, L;                  // cu[s], L_s
 
     __device__ __forceinline__ void enter_sequence() {
@@ -52,26 +60,28 @@ struct ItemWalker {
         L = __ldg(&cu[s + 1]) - row0;
         ntiles = tiles_of(L);
     }
-    __device__ __forceinline__ void init(const int* cu_, int batch_, int Hkv_, int i) {
-        cu = cu_;
-        batch = batch_;
-        Hkv = Hkv_;
+    __device__ __forceinline__ void init(int i) {
         int base = 0;
-        for (s = 0; s < batch; ++s) {
+        if (first) {
+            for (s = 0; s + 1 < batch && i >= first[s + 1]; ++s) {}
+            base = first[s];
             enter_sequence();
-            if (i < base + ntiles * Hkv) break;
-            base += ntiles * Hkv;
+        } else {
+            for (s = 0; s < batch; ++s) {
+                enter_sequence();
+                if (i < base + ntiles * Hkv) break;
+                base += ntiles * Hkv;
+            }
         }
         const int local = i - base;
         h = local / ntiles;
         j = local - h * ntiles;
-        ibase = base + h * ntiles;
     }
     __device__ __forceinline__ bool last_of_head() const { return j + 1 == ntiles; }
+    __device__ __forceinline__ int head() const { return s * Hkv + h; }
     __device__ __forceinline__ void next() {
         if (++j < ntiles) return;
         j = 0;
-        ibase += ntiles;
         if (++h < Hkv) return;
         h = 0;
         if (++s < batch) enter_sequence();
@@ -84,13 +94,16 @@ constexpr int kChunkSmall = 8;           // items per claim otherwise
 constexpr int kChunkSlots = 4;           // claimed chunks in flight inside a CTA
 
 struct ScoreArgs {
+    CUtensorMap kmap[kMaxGroup], qmap[kMaxGroup];
     Geometry G;
     const int* cu;                 // device cu_seqlens
-    Scratch sc;
-    int W;        // total work items
+    int* err;
+    int nl;       // layers
+    int W;        // work items of a layer
     int kst;      // K ring depth
     int* claim;   // the launch's chunk counter, zero before the launch
     int chunk;    // items per claim
+    float2* segpart[kMaxGroup];
 };
 
 constexpr int kEpiWarps = 16;
@@ -99,15 +112,14 @@ constexpr int kScoreThreads = 64 + kEpiThreads;
 
 struct __align__(8) Barriers {
     uint64_t k_full[kKStages], k_empty[kKStages];
-    uint64_t q_full, q_empty;
+    uint64_t q_full[2], q_empty[2];
     uint64_t acc_full[4], acc_empty[4];
     uint64_t c_full[kChunkSlots], c_empty[kChunkSlots];
     uint64_t mma_done;
     uint32_t tmem_base;
     volatile int abort_flag;
     volatile int chunk[kChunkSlots];   // claimed chunk (-1: no more work)
-    volatile int cur_chunk[2];         // the epilogue's current chunk (-2: gave up), double-buffered
-    float2 xf[512];            // a segment's (max, sum) per epilogue group and row, merged at its end
+    int first[kSeqCache];              // first item of every sequence
 };
 
 __device__ __forceinline__ void raise_abort(Barriers* bars, int* err) {
@@ -115,36 +127,45 @@ __device__ __forceinline__ void raise_abort(Barriers* bars, int* err) {
     atomicExch(err, 3);
 }
 
+__device__ __forceinline__ void merge_partial(float& M, float& Z, float2 o) {
+    if (o.x == -INFINITY) return;
+    if (o.x > M) {
+        Z = Z * ptx::ex2(M - o.x) + o.y;
+        M = o.x;
+    } else {
+        Z += o.y * ptx::ex2(o.x - M);
+    }
+}
+
 // MB: 128-row M-blocks per KV head (R <= 128 * MB).  The 16 epilogue warps form
 // NB = 4 / MB groups of 4 * MB warps, one group per TMEM accumulator.
 template <int MB>
-__global__ void __launch_bounds__(kScoreThreads, 1)
-    score_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap,
-                 const __grid_constant__ ScoreArgs A) {
+__global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_constant__ ScoreArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // 1024-byte alignment for the swizzled operand tiles.
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     // Scalars and pointers in registers: values read through a reference to the
     // parameter block would be re-read after every asm statement that clobbers memory.
     const Geometry G = A.G;
-    const Scratch sc = A.sc;
+    int* const err = A.err;
     const int W = A.W, kst = A.kst;
     const int chunk_items = A.chunk;
-    const int nchunks = (W + chunk_items - 1) / chunk_items;
+    const int per_layer = (W + chunk_items - 1) / chunk_items;   // chunks of a layer
+    const int nchunks = A.nl * per_layer;
     int* const claim = A.claim;
-    const int* const cu_dev = A.cu;
-    const int Rpad = 128 * MB, R = G.R;
-    uint8_t* sQ = smem;                                   // 2 halves x Rpad rows x 128 B
-    uint8_t* sK = sQ + 2 * Rpad * 128;                    // kst x 32 KB
+    const int R = G.R;
+    const uint32_t qhalf = (uint32_t)R * 128u;            // bytes of a query buffer's half (64 columns)
+    uint8_t* sQ = smem;                                   // 2 buffers x 2 halves x R rows x 128 B
+    uint8_t* sK = sQ + 4 * qhalf;                         // kst x 32 KB
     Barriers* bars = reinterpret_cast<Barriers*>(sK + kst * kKStageBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int NB = 4 / MB;                             // TMEM accumulator buffers
 
     if (warp == 0 && lane == 0) {
-        ptx::prefetch_tensormap(&kmap);
-        ptx::prefetch_tensormap(&qmap);
-        // The next launch on this stream (the next layer's statistics) reads
+        ptx::prefetch_tensormap(&A.kmap[0]);
+        ptx::prefetch_tensormap(&A.qmap[0]);
+        // The next launch on this stream (the next group's statistics) reads
         // nothing this grid writes: let it be scheduled as SMs free up.
         asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     }
@@ -153,19 +174,27 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
             ptx::mbar_init(&bars->k_full[s], 1);
             ptx::mbar_init(&bars->k_empty[s], 1);
         }
-        ptx::mbar_init(&bars->q_full, 1);
-        ptx::mbar_init(&bars->q_empty, 1);
+        for (int b = 0; b < 2; ++b) {
+            ptx::mbar_init(&bars->q_full[b], 1);
+            ptx::mbar_init(&bars->q_empty[b], 1);
+        }
         for (int b = 0; b < 4; ++b) {
             ptx::mbar_init(&bars->acc_full[b], 1);
             ptx::mbar_init(&bars->acc_empty[b], 4 * MB);  // one arrival per warp of the group
         }
         for (int c = 0; c < kChunkSlots; ++c) {
             ptx::mbar_init(&bars->c_full[c], 1);
-            ptx::mbar_init(&bars->c_empty[c], 2);         // the MMA issuer and the epilogue's leader
+            ptx::mbar_init(&bars->c_empty[c], 1 + kEpiWarps);   // the MMA issuer and every epilogue warp
         }
         ptx::mbar_init(&bars->mma_done, 1);
         bars->abort_flag = 0;
         ptx::fence_barrier_init();
+    }
+    if (threadIdx.x >= 64 && threadIdx.x - 64 < min(G.batch, kSeqCache)) {
+        const int s = threadIdx.x - 64;
+        int base = 0;
+        for (int b = 0; b < s; ++b) base += tiles_of(__ldg(&A.cu[b + 1]) - __ldg(&A.cu[b])) * G.Hkv;
+        bars->first[s] = base;
     }
     if (warp == 1) {
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
@@ -175,182 +204,210 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
+    ItemWalker p;
+    p.cu = A.cu;
+    p.first = G.batch <= kSeqCache ? bars->first : nullptr;
+    p.batch = G.batch;
+    p.Hkv = G.Hkv;
 
+    // The producer and the MMA issuer run as whole warps, so that what they compute
+    // stays uniform, and elect a lane for the instructions that one thread issues.
+    // (Run by lane 0 alone, each tcgen05.mma and TMA instruction had its operands
+    // moved to uniform registers one by one: 1,700 cycles an item for the MMA issuer.)
+    auto uniform_init = [&](int i0) {
+        p.init(i0);
+        p.s = ptx::warp_uniform(p.s);
+        p.h = ptx::warp_uniform(p.h);
+        p.j = ptx::warp_uniform(p.j);
+        p.ntiles = ptx::warp_uniform(p.ntiles);
+        p.row0 = ptx::warp_uniform(p.row0);
+    };
+    auto uniform_next = [&]() {
+        if (++p.j < p.ntiles) return;
+        p.j = 0;
+        if (++p.h < p.Hkv) return;
+        p.h = 0;
+        if (++p.s < p.batch) {
+            p.enter_sequence();
+            p.ntiles = ptx::warp_uniform(p.ntiles);
+            p.row0 = ptx::warp_uniform(p.row0);
+        }
+    };
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            const uint64_t policy = ptx::policy_evict_normal();   // the window kernel reads K again
-            int qloads = 0, issued = 0, it = 0, di = 0;
-            for (;;) {
-                // Claim a chunk and hand it to the MMA issuer and the epilogue.
-                const int c = bars->abort_flag ? nchunks : atomicAdd(claim, 1);
-                const int ds = di % kChunkSlots, nd = di / kChunkSlots;
-                if (nd > 0 && !ptx::mbar_wait(&bars->c_empty[ds], (nd - 1) & 1)) {
-                    raise_abort(bars, sc.err);
-                    break;
-                }
+        const uint64_t policy = ptx::policy_evict_normal();   // the window kernel reads K again
+        int qloads = 0, issued = 0, st = 0, di = 0;
+        uint32_t kphase = 0u;   // bit st: the stage has been filled an odd number of times
+        int next = 0;
+        if (lane == 0) next = atomicAdd(claim, 1);
+        bool stop = false;
+        while (!stop) {
+            // Hand the claimed chunk to the MMA issuer and the epilogue, and claim
+            // the next one: its number arrives while this one is loaded.
+            const int ds = di % kChunkSlots, nd = di / kChunkSlots;
+            if (nd > 0 && !ptx::warp_wait(&bars->c_empty[ds], (nd - 1) & 1, &bars->abort_flag)) {
+                if (lane == 0) raise_abort(bars, err);
+                break;
+            }
+            const int c = ptx::warp_uniform(bars->abort_flag ? nchunks : next);
+            if (lane == 0) {
                 bars->chunk[ds] = c < nchunks ? c : -1;
                 ptx::mbar_arrive(&bars->c_full[ds]);
-                ++di;
-                if (c >= nchunks) break;
-                const int i0 = c * chunk_items, i1 = min(W, i0 + chunk_items);
-                int prev_sh = -1;   // the query rows are loaded again at every chunk's start
-                ItemWalker p;
-                p.init(cu_dev, G.batch, G.Hkv, i0);
-                bool stop = false;
-                for (int i = i0; i < i1; ++i, ++it, p.next()) {
-                    const int sh = p.s * G.Hkv + p.h;
-                    if (sh != prev_sh) {
-                        if (qloads > 0 && !ptx::mbar_wait(&bars->q_empty, (qloads - 1) & 1)) {
-                            stop = true;
-                            break;
-                        }
-                        ptx::mbar_arrive_expect_tx(&bars->q_full, 2u * R * 128u);
-                        ptx::tma_load_4d(sQ, &qmap, &bars->q_full, 0, p.h * G.g, 0, p.s);
-                        ptx::tma_load_4d(sQ + Rpad * 128, &qmap, &bars->q_full, 64, p.h * G.g, 0, p.s);
-                        ++qloads;
-                        prev_sh = sh;
-                    }
-                    const int st = it % kst, n = it / kst;
-                    if (n > 0 && !ptx::mbar_wait(&bars->k_empty[st], (n - 1) & 1)) {
+            }
+            ++di;
+            if (c >= nchunks) break;
+            if (lane == 0) next = atomicAdd(claim, 1);
+            const int lay = c / per_layer, i0 = (c - lay * per_layer) * chunk_items, i1 = min(W, i0 + chunk_items);
+            const CUtensorMap* kmap = &A.kmap[lay];
+            const CUtensorMap* qmap = &A.qmap[lay];
+            int prev_sh = -1;   // the query rows are loaded again at every chunk's start
+            uniform_init(i0);
+            for (int i = i0; i < i1; ++i) {
+                if (p.head() != prev_sh) {
+                    const int qs = qloads & 1, nq = qloads >> 1;
+                    if (nq > 0 && !ptx::warp_wait(&bars->q_empty[qs], (nq - 1) & 1, &bars->abort_flag)) {
                         stop = true;
                         break;
                     }
+                    if (ptx::elect_one()) {
+                        ptx::mbar_arrive_expect_tx(&bars->q_full[qs], 2u * qhalf);
+                        load_queries(sQ + qs * 2 * qhalf, qhalf, qmap, &bars->q_full[qs], G, p.h, p.s);
+                    }
+                    __syncwarp();
+                    ++qloads;
+                    prev_sh = p.head();
+                }
+                if (issued >= kst && !ptx::warp_wait(&bars->k_empty[st], ((kphase >> st) & 1u) ^ 1u, &bars->abort_flag)) {
+                    stop = true;
+                    break;
+                }
+                if (ptx::elect_one()) {
                     uint8_t* dst = sK + st * kKStageBytes;
                     const int row = p.row0 + p.j * kTileT;
                     ptx::mbar_arrive_expect_tx(&bars->k_full[st], (uint32_t)kKStageBytes);
-                    ptx::tma_load_3d(dst, &kmap, &bars->k_full[st], 0, p.h, row, policy);
-                    ptx::tma_load_3d(dst + kKHalfBytes, &kmap, &bars->k_full[st], 64, p.h, row, policy);
-                    ++issued;
+                    ptx::tma_load_3d(dst, kmap, &bars->k_full[st], 0, p.h, row, policy);
+                    ptx::tma_load_3d(dst + kKHalfBytes, kmap, &bars->k_full[st], 64, p.h, row, policy);
                 }
-                if (stop) {
-                    raise_abort(bars, sc.err);
-                    break;
-                }
+                __syncwarp();
+                kphase ^= 1u << st;
+                ++issued;
+                st = st + 1 == kst ? 0 : st + 1;
+                uniform_next();
             }
-            // Drain: every issued copy lands before the CTA may exit (stage st was
-            // filled ceil((issued - st) / kst) times).
-            for (int st = 0; st < kst && st < issued; ++st) {
-                const int fills = (issued - st + kst - 1) / kst;
-                ptx::mbar_wait(&bars->k_full[st], (fills - 1) & 1, 50000000ull);
-            }
-            if (qloads > 0) ptx::mbar_wait(&bars->q_full, (qloads - 1) & 1, 50000000ull);
+            if (stop && lane == 0) raise_abort(bars, err);
         }
+        // Drain: every issued copy lands before the CTA may exit (stage b was
+        // filled ceil((issued - b) / kst) times, query buffer b ceil((qloads - b) / 2)).
+        for (int b = 0; b < kst && b < issued; ++b)
+            ptx::mbar_wait(&bars->k_full[b], ((issued - b + kst - 1) / kst - 1) & 1, 50000000ull);
+        for (int b = 0; b < 2 && b < qloads; ++b)
+            ptx::mbar_wait(&bars->q_full[b], ((qloads - b + 1) / 2 - 1) & 1, 50000000ull);
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = ptx::idesc_bf16_f32(128, kTileT);
-            const uint32_t sQa = ptx::smem_u32(sQ), sKa = ptx::smem_u32(sK);
-            int qk = 0, it = 0, di = 0;
-            bool stop = false;
-            while (!stop && !bars->abort_flag) {
-                const int ds = di % kChunkSlots;
-                if (!ptx::mbar_wait(&bars->c_full[ds], (di / kChunkSlots) & 1)) {
-                    raise_abort(bars, sc.err);
-                    break;
-                }
-                const int c = bars->chunk[ds];
-                ptx::mbar_arrive(&bars->c_empty[ds]);
-                ++di;
-                if (c < 0) break;
-                const int i0 = c * chunk_items, i1 = min(W, i0 + chunk_items);
-                int prev_sh = -1;
-                ItemWalker p;
-                p.init(cu_dev, G.batch, G.Hkv, i0);
-                for (int i = i0; i < i1 && !bars->abort_flag; ++i, ++it, p.next()) {
-                    const int sh = p.s * G.Hkv + p.h;
-                    if (sh != prev_sh) {
-                        if (!ptx::mbar_wait(&bars->q_full, qk & 1)) {
-                            raise_abort(bars, sc.err);
-                            stop = true;
-                            break;
-                        }
-                        ++qk;
-                        prev_sh = sh;
-                    }
-                    const int st = it % kst, n = it / kst;
-                    const int buf = it % NB, nb = it / NB;
-                    if (!ptx::mbar_wait(&bars->k_full[st], n & 1) ||
-                        (nb > 0 && !ptx::mbar_wait(&bars->acc_empty[buf], (nb - 1) & 1))) {
-                        raise_abort(bars, sc.err);
+        const uint32_t idesc = ptx::idesc_bf16_f32(128, kTileT);
+        const uint64_t qdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sQ)), kdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sK));
+        int qk = 0, st = 0, di = 0;
+        uint32_t kphase = 0u, used = 0u, aphase = 0u;   // per stage / accumulator
+        bool stop = false;
+        while (!stop) {
+            const int ds = di % kChunkSlots;
+            if (!ptx::warp_wait(&bars->c_full[ds], (di / kChunkSlots) & 1, &bars->abort_flag)) {
+                stop = true;
+                break;
+            }
+            const int c = ptx::warp_uniform(bars->chunk[ds]);
+            if (lane == 0) ptx::mbar_arrive(&bars->c_empty[ds]);
+            ++di;
+            if (c < 0) break;
+            const int i0 = (c % per_layer) * chunk_items, i1 = min(W, i0 + chunk_items);
+            int prev_sh = -1, qs = 0, buf = 0;
+            uniform_init(i0);
+            for (int i = i0; i < i1; ++i) {
+                if (p.head() != prev_sh) {
+                    qs = qk & 1;
+                    if (!ptx::warp_wait(&bars->q_full[qs], (qk >> 1) & 1, &bars->abort_flag)) {
                         stop = true;
                         break;
                     }
-                    ptx::tc_fence_after();
-                    const uint32_t kst = sKa + st * kKStageBytes;
+                    ++qk;
+                    prev_sh = p.head();
+                }
+                // Giving up on a stage in flight is safe: the producer drains its own loads.
+                if (!ptx::warp_wait(&bars->k_full[st], (kphase >> st) & 1u, &bars->abort_flag) ||
+                    (((used >> buf) & 1u) != 0u &&
+                     !ptx::warp_wait(&bars->acc_empty[buf], ((aphase >> buf) & 1u) ^ 1u, &bars->abort_flag))) {
+                    stop = true;
+                    break;
+                }
+                ptx::tc_fence_after();
+                const bool seg_end = i + 1 >= i1 || p.last_of_head();
+                if (ptx::elect_one()) {
+                    const uint64_t kd = kdesc + (uint32_t)(st * (kKStageBytes >> 4)), qd = qdesc + (uint32_t)qs * (qhalf >> 3);
+#pragma unroll
                     for (int m = 0; m < MB; ++m) {
                         const uint32_t d = tmem + (uint32_t)(buf * 128 * MB + m * 128);
-    #pragma unroll
+#pragma unroll
                         for (int kk = 0; kk < 8; ++kk) {
-                            const int half = kk >> 2, kin = kk & 3;
-                            const uint64_t ad = ptx::smem_desc_k_sw128(sQa + half * Rpad * 128 + m * 16384 + kin * 32);
-                            const uint64_t bd = ptx::smem_desc_k_sw128(kst + half * kKHalfBytes + kin * 32);
-                            ptx::mma_bf16(d, ad, bd, idesc, kk > 0 ? 1u : 0u);
+                            const uint32_t half = kk >> 2, kin = kk & 3;
+                            ptx::mma_bf16(d, qd + half * (qhalf >> 4) + m * 1024 + kin * 2,
+                                          kd + half * (kKHalfBytes >> 4) + kin * 2, idesc, kk > 0 ? 1u : 0u);
                         }
                     }
                     ptx::mma_commit(&bars->k_empty[st]);
                     ptx::mma_commit(&bars->acc_full[buf]);
-                    if (i + 1 >= i1 || p.last_of_head()) ptx::mma_commit(&bars->q_empty);
+                    if (seg_end) ptx::mma_commit(&bars->q_empty[qs]);
                 }
+                __syncwarp();
+                kphase ^= 1u << st;
+                used |= 1u << buf;
+                aphase ^= 1u << buf;
+                st = st + 1 == kst ? 0 : st + 1;
+                buf = buf + 1 == NB ? 0 : buf + 1;
+                uniform_next();
             }
-            ptx::mma_commit(&bars->mma_done);
         }
+        if (stop && lane == 0) raise_abort(bars, err);
+        if (ptx::elect_one()) ptx::mma_commit(&bars->mma_done);
+        __syncwarp();
     } else {
         // ------------------------------------------------------------ epilogue
-        // NB groups of GW = 4 * MB warps; group a takes the CTA's items a, a + NB,
-        // ... from its own accumulator, so the groups work on different items at
-        // once (one group's TMEM loads and barrier waits overlap the others' ex2).
-        // Warp k of a group reads TMEM lanes 32*(warp % 4) .. +31 (the lane
-        // quadrant its warp id allows) of M-block k / 4: one thread per query row,
-        // all 128 columns of the item.
+        // NB groups of GW = 4 * MB warps; group a takes the items a, a + NB, ... of
+        // every chunk from its own accumulator, so the groups work on different
+        // items at once (one group's TMEM loads and barrier waits overlap the
+        // others' ex2).  Warp k of a group reads TMEM lanes 32*(warp % 4) .. +31
+        // (the lane quadrant its warp id allows) of M-block k / 4: one thread per
+        // query row, all 128 columns of the item.
         constexpr int GW = 4 * MB;
         const int ew = warp - 2;
         const int grp = ew / GW;
         const int m = (ew % GW) >> 2;
         const int quad = warp & 3;
-        const int row = m * 128 + quad * 32 + lane;
+        const int row = m * 128 + quad * 32 + lane;   // query head j of the group at window position q
         const bool vrow = row < R;
-        const int q = vrow ? row / G.g : 0;
-        bool aborted = false;
+        const int q = !vrow ? 0 : G.jm ? row % G.w : row / G.g;
         float seg_m = -INFINITY, seg_z = 0.f;
-        int cur_sh = -1, seg_first = 0;
-
-        auto merge = [](float& M, float& Z, float2 o) {
-            if (o.x == -INFINITY) return;
-            if (o.x > M) {
-                Z = Z * ptx::ex2(M - o.x) + o.y;
-                M = o.x;
-            } else {
-                Z += o.y * ptx::ex2(o.x - M);
-            }
-        };
-        // Every epilogue thread calls this at the same segment boundaries (aborted
-        // warps included), so the named barriers always complete.  The groups'
-        // partials merge here; rowstat_kernel merges the CTAs' partials of a
-        // (sequence, head) into (m_r, Z_r).
-        auto flush_segment = [&]() {
-            bars->xf[grp * Rpad + row] = make_float2(seg_m, seg_z);
-            ptx::named_bar_sync(1, kEpiThreads);
-            if (grp == 0) {
-                float M = seg_m, Z = seg_z;
+        // Relative to the segment's running reference seg_m, 2^(s - seg_m) sums the
+        // same mass as an online max/rescale without a max pass.  32 columns of the
+        // row, four sums of every fourth.
+        auto sum32 = [&](const float* v) {
+            const uint64_t sl2 = ptx::pack_f32x2(G.sl2, G.sl2), ref = ptx::pack_f32x2(-seg_m, -seg_m);
+            uint64_t z01 = 0ull, z23 = 0ull;   // packed pairs: the roundings are the scalar operations'
 #pragma unroll
-                for (int c = 1; c < NB; ++c) merge(M, Z, bars->xf[c * Rpad + row]);
-                if (vrow) sc.segpart[(size_t)seg_first * R + row] = make_float2(M, Z);
+            for (int c = 0; c < 32; c += 4) {
+                const uint64_t a = ptx::fma_f32x2(ptx::pack_f32x2(v[c], v[c + 1]), sl2, ref);
+                const uint64_t b = ptx::fma_f32x2(ptx::pack_f32x2(v[c + 2], v[c + 3]), sl2, ref);
+                z01 = ptx::add_f32x2(z01, ptx::pack_f32x2(ptx::ex2(ptx::lo_f32(a)), ptx::ex2(ptx::hi_f32(a))));
+                z23 = ptx::add_f32x2(z23, ptx::pack_f32x2(ptx::ex2(ptx::lo_f32(b)), ptx::ex2(ptx::hi_f32(b))));
             }
-            ptx::named_bar_sync(1, kEpiThreads);   // xf is free for the next segment
+            return (ptx::lo_f32(z01) + ptx::hi_f32(z01)) + (ptx::lo_f32(z23) + ptx::hi_f32(z23));
         };
-        // 32 columns of the row, `lim` of them visible (<= 0: none).  Relative to
-        // the segment's running reference seg_m, 2^(s - seg_m) sums the same mass
-        // as an online max/rescale without a max pass; a chunk far above the
-        // reference (sum not below 2^64) and the segment's first chunk take the
-        // exact path.
+        // The same, `lim` of the columns visible (<= 0: none), for any of them: a sum
+        // far above the reference (not below 2^64) and the segment's first columns
+        // take the exact path.
         auto chunk = [&](const float* v, int lim) {
             if (lim <= 0) return;
             if (lim >= 32 && seg_m != -INFINITY) {
-                float z4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int c = 0; c < 32; ++c) z4[c & 3] += ptx::ex2(fmaf(v[c], G.sl2, -seg_m));
-                const float z = (z4[0] + z4[1]) + (z4[2] + z4[3]);
+                const float z = sum32(v);
                 if (z < 0x1p64f) {
                     seg_z += z;
                     if (seg_z >= 0x1p40f) {
@@ -371,79 +428,100 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 #pragma unroll
             for (int c = 0; c < 32; ++c)
                 if (c < lim) z4[c & 3] += ptx::ex2(fmaf(v[c], G.sl2, -mu));
-            merge(seg_m, seg_z, make_float2(mu, (z4[0] + z4[1]) + (z4[2] + z4[3])));
+            merge_partial(seg_m, seg_z, make_float2(mu, (z4[0] + z4[1]) + (z4[2] + z4[3])));
         };
 
-        int it = 0, di = 0;
-        for (;;) {
-            // The epilogue's leader takes the next claimed chunk; the barrier
-            // hands it to every epilogue thread (-1: no more work, -2: gave up).
+        int di = 0;
+        uint32_t nb = 0u;   // items of this group so far
+        bool aborted = false;
+        while (!aborted) {
+            // Each warp takes the next claimed chunk by itself (-1: no more work).
             const int ds = di % kChunkSlots;
-            if (threadIdx.x == 64) {
-                int c = -2;
-                if (ptx::mbar_wait(&bars->c_full[ds], (di / kChunkSlots) & 1)) {
+            int c = -1;
+            if (lane == 0) {
+                if (ptx::mbar_wait_abortable(&bars->c_full[ds], (di / kChunkSlots) & 1, &bars->abort_flag)) {
                     c = bars->chunk[ds];
                     ptx::mbar_arrive(&bars->c_empty[ds]);
                 } else {
-                    raise_abort(bars, sc.err);
+                    raise_abort(bars, err);
                 }
-                bars->cur_chunk[di & 1] = c;
             }
-            ptx::named_bar_sync(1, kEpiThreads);
-            const int c = bars->cur_chunk[di & 1];
+            c = __shfl_sync(0xffffffffu, c, 0);
             ++di;
             if (c < 0) break;
-            const int i0 = c * chunk_items, i1 = min(W, i0 + chunk_items);
-            ItemWalker p;
-            p.init(cu_dev, G.batch, G.Hkv, i0);
-            for (int i = i0; i < i1; ++i, ++it, p.next()) {
-                const int sh = p.s * G.Hkv + p.h;
-                if (sh != cur_sh) {
-                    if (cur_sh >= 0) flush_segment();
-                    cur_sh = sh;
+            const int lay = c / per_layer, cl = c - lay * per_layer;
+            const int i0 = cl * chunk_items, i1 = min(W, i0 + chunk_items);
+            // The segment of chunk cl and head sh is number cl + sh of the layer: one of
+            // the two grows from a segment to the next.
+            float2* const segpart = A.segpart[lay];
+            p.init(i0);
+            for (int i = i0; i < i1; ++i) {
+                if ((i - i0) % NB == grp) {
+                    // One warp of the group polls, the others wait in the barrier (a
+                    // polling warp takes issue slots from those that compute).
+                    bool ok = true;
+                    if (ew % GW == 0) {
+                        ok = ptx::warp_wait(&bars->acc_full[grp], nb & 1u, &bars->abort_flag);
+                        if (!ok && lane == 0) raise_abort(bars, err);
+                    }
+                    if (ptx::named_bar_or(1 + grp, 32 * GW, !ok)) {
+                        aborted = true;
+                        break;
+                    }
+                    ++nb;
+                    ptx::tc_fence_after();
+                    const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(grp * 128 * MB + m * 128);
+                    const int t0 = p.j * kTileT;
+                    const int last = vrow ? min(p.L - 1, p.L - G.w + q) : -1;   // causal on the window part
+                    const int nvalid = max(0, min(kTileT, last - t0 + 1));
+                    // Four times 32 columns, straight through: the next columns' TMEM load
+                    // is in flight while these are summed.  The sums count when every
+                    // row of the warp has a reference that they stay near (all but a
+                    // segment's first item and its last tile); else the columns are
+                    // read again and taken one by one.
+                    bool plain = nvalid == kTileT && seg_m != -INFINITY;
+                    if (__all_sync(0xffffffffu, plain || !vrow)) {
+                        float va[32], vb[32], z[4];
+                        ptx::tmem_ld32(taddr, va);
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_ld32(taddr + 32, vb);
+                        z[0] = sum32(va);
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_ld32(taddr + 64, va);
+                        z[1] = sum32(vb);
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_ld32(taddr + 96, vb);
+                        z[2] = sum32(va);
+                        ptx::tmem_wait_ld();
+                        z[3] = sum32(vb);
+                        const float s0 = seg_z + z[0], s1 = s0 + z[1], s2 = s1 + z[2], s3 = s2 + z[3];
+                        plain = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])) < 0x1p64f &&
+                                fmaxf(fmaxf(s0, s1), fmaxf(s2, s3)) < 0x1p40f && s3 == s3;
+                        plain = __all_sync(0xffffffffu, plain || !vrow);
+                        if (plain) seg_z = s3;
+                    } else {
+                        plain = false;
+                    }
+                    if (!plain) {
+#pragma unroll 1
+                        for (int c = 0; c < kTileT; c += 32) {
+                            float v[32];
+                            ptx::tmem_ld32(taddr + (uint32_t)c, v);
+                            ptx::tmem_wait_ld();
+                            chunk(v, nvalid - c);
+                        }
+                    }
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&bars->acc_empty[grp]);
+                }
+                if (i + 1 >= i1 || p.last_of_head()) {   // the segment ends
+                    if (vrow) segpart[((size_t)(cl + p.head()) * NB + grp) * R + row] = make_float2(seg_m, seg_z);
                     seg_m = -INFINITY;
                     seg_z = 0.f;
-                    seg_first = i;
                 }
-                if (it % NB != grp || aborted) continue;   // another group's item (or keep walking for the barriers)
-                const int nb = it / NB;
-                int ok = 1;
-                if (lane == 0) {
-                    ok = !bars->abort_flag && ptx::mbar_wait(&bars->acc_full[grp], nb & 1);
-                    if (!ok) raise_abort(bars, sc.err);
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) {
-                    aborted = true;
-                    continue;
-                }
-                ptx::tc_fence_after();
-                const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(grp * 128 * MB + m * 128);
-                const int L = p.L;
-                const int t0 = p.j * kTileT;
-                const int last = vrow ? min(L - 1, L - G.w + q) : -1;   // causal on the window part
-                const int nvalid = max(0, min(kTileT, last - t0 + 1));
-                // Four 32-column chunks; the next chunk's TMEM load is in flight while
-                // this one is reduced.
-                float va[32], vb[32];
-                ptx::tmem_ld32(taddr, va);
-                ptx::tmem_wait_ld();
-                ptx::tmem_ld32(taddr + 32, vb);
-                chunk(va, nvalid);
-                ptx::tmem_wait_ld();
-                ptx::tmem_ld32(taddr + 64, va);
-                chunk(vb, nvalid - 32);
-                ptx::tmem_wait_ld();
-                ptx::tmem_ld32(taddr + 96, vb);
-                chunk(va, nvalid - 64);
-                ptx::tmem_wait_ld();
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bars->acc_empty[grp]);   // the accumulator is in registers
-                chunk(vb, nvalid - 96);
+                p.next();
             }
-            if (cur_sh >= 0) flush_segment();   // a chunk's end closes its last segment
-            cur_sh = -1;
         }
     }
 
@@ -455,11 +533,12 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
     if (warp == 1) ptx::tmem_dealloc(tmem, kTmemCols);
 }
 
-// (m_r, Z_r) of every row of (s, h) from the score kernel's segment partials:
-// one at the head's first item, then one at every chunk boundary inside the
-// head's range of items, merged in item order.  Grid (Hkv, batch), one thread
-// per row.
-__global__ void __launch_bounds__(256) rowstat_kernel(Geometry G, Scratch sc, const int* __restrict__ cu,
+// (m_r, Z_r) of every row of (s, h) from the score kernel's partials: its
+// segments lie in the consecutive chunks that hold its items, the groups' partials
+// of a segment merge first, then the segments in item order.  Grid (Hkv, batch,
+// layers), one thread per row, as the score kernel orders them.
+template <int NB>
+__global__ void __launch_bounds__(256) rowstat_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A,
                                                       int chunk, int* claim, int wait_prev) {
     // The window launch that follows may start; it waits for this grid.
     if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -468,55 +547,51 @@ __global__ void __launch_bounds__(256) rowstat_kernel(Geometry G, Scratch sc, co
     // Otherwise the partials come through a full dependency and the stream's
     // previous kernel (if a programmatic predecessor at all) is not waited for.
     if (wait_prev) asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    const int h = blockIdx.x, s = blockIdx.y, r = threadIdx.x;
+    const int h = blockIdx.x, s = blockIdx.y, lay = blockIdx.z, r = threadIdx.x;
     // The score grid has completed: its chunk counter is free for the next launch.
-    if (h == 0 && s == 0 && r == 0) *claim = 0;
+    if (h == 0 && s == 0 && lay == 0 && r == 0) *claim = 0;
     if (r >= G.R) return;
+    const int* __restrict__ cu = A.io[0].cu;
     int ib = 0;
     for (int b = 0; b < s; ++b) ib += tiles_of(__ldg(&cu[b + 1]) - __ldg(&cu[b])) * G.Hkv;
     const int nt = tiles_of(__ldg(&cu[s + 1]) - __ldg(&cu[s]));
+    const int sh = s * G.Hkv + h;
     ib += h * nt;
-    const int iend = ib + nt;
+    const int seg0 = ib / chunk + sh, seg1 = (ib + nt - 1) / chunk + sh;
+    const float2* src = A.segpart[lay] + r;
     float M = -INFINITY, Z = 0.f;
-    // Segment starts: the head's first item, then every chunk boundary inside it.
-    int next = ib, bnd = (ib / chunk + 1) * chunk;
-    while (next < iend) {
-        float2 pz[16];
+    constexpr int kSegs = 16 / NB;   // segments whose loads are issued together
+    for (int g0 = seg0; g0 <= seg1; g0 += kSegs) {
+        float2 pz[kSegs][NB];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            pz[k] = make_float2(-INFINITY, 0.f);
-            if (next < iend) {
-                pz[k] = __ldcg(&sc.segpart[(size_t)next * G.R + r]);
-                next = bnd;
-                bnd += chunk;
-            }
-        }
+        for (int k = 0; k < kSegs; ++k)
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const float2 o = pz[k];
-            if (o.x == -INFINITY) continue;
-            if (o.x > M) {
-                Z = Z * ptx::ex2(M - o.x) + o.y;
-                M = o.x;
-            } else {
-                Z += o.y * ptx::ex2(o.x - M);
-            }
+            for (int a = 0; a < NB; ++a)
+                pz[k][a] = g0 + k <= seg1 ? __ldcg(&src[((size_t)(g0 + k) * NB + a) * G.R]) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int k = 0; k < kSegs; ++k) {
+            float ms = pz[k][0].x, zs = pz[k][0].y;
+#pragma unroll
+            for (int a = 1; a < NB; ++a) merge_partial(ms, zs, pz[k][a]);
+            merge_partial(M, Z, make_float2(ms, zs));
         }
     }
-    sc.rowstat[((size_t)s * G.Hkv + h) * G.R + r] = make_float2(M, Z);
+    const int q = G.jm ? r % G.w : r / G.g, j = G.jm ? r / G.w : r - q * G.g;
+    A.sl[lay].rowstat[(size_t)sh * G.R + q * G.g + j] = make_float2(M, Z);
 }
 
 // Row statistics from the caller's log-sum-exp of each window query row (the
 // denominator its prefill attention already computed): row r = q * g + j of KV
-// head h is query head h * g + j at window position q.  Grid (Hkv, batch).
-__global__ void __launch_bounds__(256) rowstat_lse_kernel(Geometry G, Scratch sc, const float* __restrict__ lse) {
+// head h is query head h * g + j at window position q.  Grid (Hkv, batch, layers).
+__global__ void __launch_bounds__(256) rowstat_lse_kernel(const __grid_constant__ Geometry G,
+                                                          const __grid_constant__ Group A) {
     // The window launch that follows may start; it waits for this grid before reading.
     if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    const int h = blockIdx.x, s = blockIdx.y, r = threadIdx.x;
+    const int h = blockIdx.x, s = blockIdx.y, lay = blockIdx.z, r = threadIdx.x;
     if (r >= G.R) return;
     const int q = r / G.g, j = r - q * G.g;
-    const float v = __ldg(&lse[((size_t)s * G.w + q) * G.Hq + h * G.g + j]);
-    sc.rowstat[((size_t)s * G.Hkv + h) * G.R + r] = make_float2(v * 1.4426950408889634f, 1.f);
+    const float v = __ldg(&A.io[lay].lse[((size_t)s * G.w + q) * G.Hq + h * G.g + j]);
+    A.sl[lay].rowstat[((size_t)s * G.Hkv + h) * G.R + r] = make_float2(v * 1.4426950408889634f, 1.f);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -534,9 +609,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 int mblocks(const Geometry& g) { return g.R > 128 ? 2 : 1; }
 
+// Two query buffers of R rows, the K ring, the barriers.  (An M-block's rows past R
+// are whatever follows the buffer; their accumulator rows are not read.)
 size_t smem_bytes_with(const Geometry& g, int kst) {
-    const int MB = mblocks(g);
-    return 1024 + 2 * (size_t)MB * 128 * 128 + (size_t)kst * kKStageBytes + sizeof(Barriers);
+    return 1024 + 4 * (size_t)g.R * 128 + (size_t)kst * kKStageBytes + sizeof(Barriers);
 }
 
 int kstages_for(const Geometry& g) {
@@ -551,6 +627,10 @@ size_t smem_bytes_for(const Geometry& g) { return smem_bytes_with(g, kstages_for
 
 size_t score_smem_bytes(const Geometry& g) { return smem_bytes_for(g); }
 
+size_t score_partial_bytes(const Geometry& g, size_t tiles) {
+    return (tiles * g.Hkv / kChunkSmall + 1 + (size_t)g.batch * g.Hkv) * (4 / mblocks(g)) * g.R * sizeof(float2);
+}
+
 cudaError_t configure_score(const Geometry& g) {
     // Per-function attribute shared by every handle: the largest supported geometry.
     size_t need = 0;
@@ -564,51 +644,46 @@ cudaError_t configure_score(const Geometry& g) {
     return e;
 }
 
-cudaError_t plan_score(const Geometry& g, const LayerIO& io, const Scratch& sc, int num_sms, ScorePlan* plan) {
+cudaError_t plan_score(const Geometry& g, const Group& gr, int num_sms, ScorePlan* plan) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    CUtensorMap& kmap = plan->kmap;
-    CUtensorMap& qmap = plan->qmap;
-    {
-        cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.Hkv, (cuuint64_t)g.total_tokens};
-        cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)g.Hkv * kHeadDim * 2};
-        cuuint32_t box[3] = {64, 1, (cuuint32_t)kTileT};
-        cuuint32_t es[3] = {1, 1, 1};
-        if (enc(&kmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(io.k), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
+    for (int l = 0; l < gr.nl; ++l) {
+        {
+            cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.Hkv, (cuuint64_t)g.total_tokens};
+            cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)g.Hkv * kHeadDim * 2};
+            cuuint32_t box[3] = {64, 1, (cuuint32_t)kTileT};
+            cuuint32_t es[3] = {1, 1, 1};
+            if (enc(&plan->kmap[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(gr.io[l].k), dims,
+                    strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return cudaErrorInvalidValue;
+        }
+        {
+            // A KV head's rows in one box, or a box for each query head (load_queries).
+            cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.Hq, (cuuint64_t)g.w, (cuuint64_t)g.batch};
+            cuuint64_t strides[3] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)g.Hq * kHeadDim * 2,
+                                     (cuuint64_t)g.w * g.Hq * kHeadDim * 2};
+            cuuint32_t box[4] = {64, (cuuint32_t)(g.jm ? 1 : g.g), (cuuint32_t)g.w, 1};
+            cuuint32_t es[4] = {1, 1, 1, 1};
+            if (enc(&plan->qmap[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(gr.io[l].q), dims,
+                    strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return cudaErrorInvalidValue;
+        }
     }
-    {
-        cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)g.Hq, (cuuint64_t)g.w, (cuuint64_t)g.batch};
-        cuuint64_t strides[3] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)g.Hq * kHeadDim * 2,
-                                 (cuuint64_t)g.w * g.Hq * kHeadDim * 2};
-        cuuint32_t box[4] = {64, (cuuint32_t)g.g, (cuuint32_t)g.w, 1};
-        cuuint32_t es[4] = {1, 1, 1, 1};
-        if (enc(&qmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(io.q), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
-    ScoreArgs& a = *reinterpret_cast<ScoreArgs*>(plan->args);
-    static_assert(sizeof(ScoreArgs) <= sizeof(plan->args), "ScorePlan::args too small");
-    a = ScoreArgs{};
-    a.G = g;
-    a.cu = io.cu;
-    a.sc = sc;
-    a.W = g.total_tiles * g.Hkv;
-    a.kst = kstages_for(g);
+    plan->items = g.total_tiles * g.Hkv;
     // At most all but kScoreReserveSms SMs (the rest run the window, heads and
     // selection kernels of neighbouring layers, which cannot share an SM with a
     // score CTA) and at most one CTA per chunk.
     const int usable = num_sms > 2 * kScoreReserveSms ? num_sms - kScoreReserveSms : num_sms;
-    // Chunks of kChunkLarge items when that still gives every usable SM one, else
-    // of kChunkSmall (measured: larger chunks reload the query rows less often,
-    // smaller ones leave fewer SMs idle on small layers).
-    a.chunk = a.W / kChunkLarge >= usable ? kChunkLarge : kChunkSmall;
-    const int nchunks = (a.W + a.chunk - 1) / a.chunk;
+    // Chunks of kChunkLarge items when one layer's still give every usable SM one,
+    // else of kChunkSmall (measured: larger chunks reload the query rows less
+    // often, smaller ones leave fewer SMs idle on small layers).  The rule looks at
+    // one layer, so that a row's statistics do not depend on how many layers
+    // share a launch.
+    plan->chunk = plan->items / kChunkLarge >= usable ? kChunkLarge : kChunkSmall;
+    const int nchunks = (plan->items + plan->chunk - 1) / plan->chunk * gr.nl;
     plan->grid = nchunks < usable ? nchunks : usable;
-    plan->chunk = a.chunk;
     plan->threads = kScoreThreads;
     plan->mb = mblocks(g);
     plan->smem = smem_bytes_for(g);
@@ -616,53 +691,61 @@ cudaError_t plan_score(const Geometry& g, const LayerIO& io, const Scratch& sc, 
     return cudaSuccess;
 }
 
-cudaError_t launch_rowstat(const ScorePlan& plan, const Geometry& g, const LayerIO& io, const Scratch& sc,
-                           int* claim, cudaStream_t st, bool programmatic, bool after_score) {
-    (void)plan;
+namespace {
+
+cudaLaunchConfig_t launch_config(dim3 grid, int threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr,
+                                 bool programmatic) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.Hkv, g.batch);
-    cfg.blockDim = dim3(256);
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = programmatic ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, rowstat_kernel, g, sc, io.cu, plan.chunk, claim, after_score ? 1 : 0);
+    return cfg;
 }
 
-cudaError_t launch_rowstat_lse(const Geometry& g, const LayerIO& io, const Scratch& sc, cudaStream_t st,
-                               bool programmatic) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.Hkv, g.batch);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = programmatic ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, rowstat_lse_kernel, g, sc, io.lse);
+}  // namespace
+
+cudaError_t launch_rowstat(const ScorePlan& plan, const Geometry& g, const Group& gr, int* claim, cudaStream_t st,
+                           bool programmatic, bool after_score) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = launch_config(dim3(g.Hkv, g.batch, gr.nl), 256, 0, st, &attr, programmatic);
+    if (plan.mb == 2) return cudaLaunchKernelEx(&cfg, rowstat_kernel<2>, g, gr, plan.chunk, claim, after_score ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, rowstat_kernel<4>, g, gr, plan.chunk, claim, after_score ? 1 : 0);
 }
 
-cudaError_t launch_score(const ScorePlan& plan, int* claim, cudaStream_t st, bool after_own_launch) {
-    ScoreArgs a = *reinterpret_cast<const ScoreArgs*>(plan.args);
+cudaError_t launch_rowstat_lse(const Geometry& g, const Group& gr, cudaStream_t st, bool programmatic) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = launch_config(dim3(g.Hkv, g.batch, gr.nl), 256, 0, st, &attr, programmatic);
+    return cudaLaunchKernelEx(&cfg, rowstat_lse_kernel, g, gr);
+}
+
+cudaError_t launch_score(const ScorePlan& plan, const Geometry& g, const Group& gr, const Scratch& sc, int* claim,
+                         cudaStream_t st, bool after_own_launch) {
+    ScoreArgs a{};
+    for (int l = 0; l < gr.nl; ++l) {
+        a.kmap[l] = plan.kmap[l];
+        a.qmap[l] = plan.qmap[l];
+        a.segpart[l] = gr.segpart[l];
+    }
+    a.G = g;
+    a.cu = gr.io[0].cu;
+    a.err = sc.err;
+    a.nl = gr.nl;
+    a.W = plan.items;
+    a.kst = kstages_for(g);
     a.claim = claim;
+    a.chunk = plan.chunk;
     // after_own_launch: the previous kernel on the stream is the previous
-    // layer's launch, whose results this grid does not read; the launch is then
+    // group's launch, whose results this grid does not read; the launch is then
     // its programmatic dependent and never executes griddepcontrol.wait.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(plan.grid);
-    cfg.blockDim = dim3(plan.threads);
-    cfg.dynamicSmemBytes = plan.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = after_own_launch ? 1 : 0;
-    if (plan.mb == 2) return cudaLaunchKernelEx(&cfg, score_kernel<2>, plan.kmap, plan.qmap, a);
-    return cudaLaunchKernelEx(&cfg, score_kernel<1>, plan.kmap, plan.qmap, a);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = launch_config(dim3(plan.grid), plan.threads, plan.smem, st, &attr, after_own_launch);
+    if (plan.mb == 2) return cudaLaunchKernelEx(&cfg, score_kernel<2>, a);
+    return cudaLaunchKernelEx(&cfg, score_kernel<1>, a);
 }
 
 }  // namespace kvec

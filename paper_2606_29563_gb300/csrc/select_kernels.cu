@@ -6,6 +6,7 @@
 // shared by all keys skipped, 4-bit digits counted in registers, one barrier
 // per digit, small threshold buckets compacted and ranked directly).  Ties at
 // the threshold go to the lower position.
+#include "hist_select.cuh"
 #include "kvec_internal.cuh"
 
 namespace kvec {
@@ -849,13 +850,18 @@ __device__ Moments block_moments(Moments v, float3* red) {
     return t;
 }
 
-// Section 4.1, first half.  One CTA per (KV head, sequence): pool the head's
+// Section 4.1, first half.  One CTA per (KV head, sequence, layer): pool the head's
 // P_O and P_O' rows and a slice of I (max-pool, inherited from SnapKV; or the
 // average variant) and the head's ranking key: sigma_h = sample std of pooled
 // P_O over the candidates (Welford/Chan moments in fp32), or, for the entropy
 // criterion of the Section 5.4 ablation, minus the entropy of pooled P_O
 // normalised over the candidates, sum(x ln x)/S - ln S with S = sum(x).
-__global__ void __launch_bounds__(kSelectThreads) heads_pool_kernel(Geometry G, LayerIO io, Scratch sc, Slot sl) {
+__global__ void __launch_bounds__(kSelectThreads) heads_pool_kernel(const __grid_constant__ Geometry G,
+                                                                     const __grid_constant__ Group A, int* claim) {
+    // The window grid has completed: its work counter is free for the next launch.
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) claim[1] = 0;
+    const LayerIO& io = A.io[blockIdx.z];
+    const Slot& sl = A.sl[blockIdx.z];
     __shared__ float3 red[32];
     extern __shared__ float mbuf[];   // raw I of a chunk, per window row (several head groups only)
     const int h = blockIdx.x, s = blockIdx.y;
@@ -975,10 +981,14 @@ __global__ void __launch_bounds__(kSelectThreads) heads_pool_kernel(Geometry G, 
 }
 
 // Section 4.1, second half, and the preserved tokens of Section 4.2.  One CTA
-// per (KV head, sequence), launched after heads_pool_kernel: every CTA ranks the
+// per (KV head, sequence, layer), launched after heads_pool_kernel: every CTA ranks the
 // sequence's sigmas the same way, the delta lowest-sigma heads take the O'
 // scores, then the top-K preserved tokens of the chosen row by radix select.
-__global__ void __launch_bounds__(kSelectThreads, 2) heads_topk_kernel(Geometry G, LayerIO io, Scratch sc, Slot sl) {
+__global__ void __launch_bounds__(kSelectThreads, 2) heads_topk_kernel(const __grid_constant__ Geometry G,
+                                                                        const __grid_constant__ Group A,
+                                                                        uint32_t* key_rows) {
+    const LayerIO& io = A.io[blockIdx.z];
+    const Slot& sl = A.sl[blockIdx.z];
     __shared__ TopkShared sm;
     __shared__ int top_flag;
     extern __shared__ __align__(16) uint32_t bits[];
@@ -1005,7 +1015,8 @@ __global__ void __launch_bounds__(kSelectThreads, 2) heads_topk_kernel(Geometry 
     const int top = top_flag;
     if (L > G.budget && G.Kp > 0) {
         const float* __restrict__ P = (top ? sl.POe : sl.PO) + row * G.ML;
-        uint32_t* keys = keys_in_smem(G.ML) ? bits + ((G.words + 3) & ~3) : sc.keys + row * G.ML;
+        uint32_t* keys = keys_in_smem(G.ML) ? bits + ((G.words + 3) & ~3)
+                                            : key_rows + ((size_t)blockIdx.z * G.batch * G.Hkv + row) * G.ML;
         for (int b0 = 4 * tid; b0 < Lc; b0 += 16 * NT) {
             float4 pv[4];
 #pragma unroll
@@ -1030,6 +1041,55 @@ __global__ void __launch_bounds__(kSelectThreads, 2) heads_topk_kernel(Geometry 
     }
     uint32_t* pres = sl.pres + row * G.words;
     for (int wd = tid; wd < G.words; wd += NT) pres[wd] = bits[wd];
+}
+
+// heads_topk_kernel for rows whose keys fit in a block's registers.
+template <int NT, int KPT>
+__global__ void __launch_bounds__(NT) heads_topk_reg_kernel(const __grid_constant__ Geometry G,
+                                                          const __grid_constant__ Group A) {
+    const LayerIO& io = A.io[blockIdx.z];
+    const Slot& sl = A.sl[blockIdx.z];
+    using HS = HistSelect<NT, KPT>;
+    __shared__ HistSelectShared sm;
+    __shared__ __align__(16) uint32_t bits[HS::kWords];
+    const int h = blockIdx.x, s = blockIdx.y;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int L = io.cu[s + 1] - io.cu[s];
+    const int Lc = L - G.wk;
+    const size_t row = (size_t)s * G.Hkv + h;
+    HS::clear(sm);
+    // Programmatic dependent of the pooling kernel: its sigmas and pooled rows are
+    // read only after that grid has completed.
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    // Every warp ranks the sequence's sigmas the same way.
+    const float sigma = __ldcg(&sl.sigma[row]);
+    const float so = lane < G.Hkv ? __ldcg(&sl.sigma[(size_t)s * G.Hkv + lane]) : INFINITY;
+    const bool before = lane < G.Hkv && (so < sigma || (so == sigma && lane < h));
+    const bool top = __popc(__ballot_sync(0xffffffffu, before)) < G.delta;
+    if (tid == 0) sl.htop[row] = top;
+    uint32_t* pres = sl.pres + row * G.words;
+    if (L <= G.budget || G.Kp == 0) {
+        for (int wd = tid; wd < G.words; wd += NT) pres[wd] = 0u;
+        return;
+    }
+    const float* __restrict__ P = (top ? sl.POe : sl.PO) + row * G.ML;
+    uint32_t key[KPT];
+#pragma unroll
+    for (int g = 0; g < KPT / 4; ++g) {
+        const int t = HS::position(4 * g);
+        const float4 v = t < Lc ? __ldcg(reinterpret_cast<const float4*>(P + t)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) key[4 * g + e] = t + e < Lc ? float_order_key(x[e]) : 0u;
+    }
+    __syncthreads();
+    HS hs{sm, G.Kp};
+    uint32_t match;
+    const uint32_t sure = hs.begin(key, match);
+    HS::store(sure, bits);
+    hs.finish(key, match, bits);
+    __syncthreads();
+    for (int wd = tid; wd < G.words; wd += NT) pres[wd] = wd < HS::kWords ? bits[wd] : 0u;
 }
 
 // Section 4.2: P' = P + lambda * I * (1 - n_t / (l + 1)); the preserved tokens
@@ -1351,12 +1411,14 @@ __global__ void __launch_bounds__(kSelectThreads) finalize_kernel(Geometry G, La
 // out_idx[s,h,j] = position of the j-th kept bit of (s, h) (-1 past the last),
 // j < cap (the budget, or the head capacity of the adaptive fill);
 // out_k[s,h,j,:] = K[cu[s] + idx, h, :] (zeros for idx = -1); the same for V.
-// Grid (ceil(cap/16), Hkv, batch), 256 threads: the block finds its 16 ranks from
+// Grid (ceil(cap/16), Hkv, layers * batch), 256 threads: the block finds its 16 ranks from
 // a prefix count over the row's bits words, then a half-warp moves one 256-byte row.
-__global__ void __launch_bounds__(256) gather_kernel(Geometry G, LayerIO io, Slot sl) {
+__global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A) {
     __shared__ int wsum[32];
     __shared__ int spos[16];
-    const int s = blockIdx.z, h = blockIdx.y;
+    const int s = blockIdx.z % G.batch, h = blockIdx.y;
+    const LayerIO& io = A.io[blockIdx.z / G.batch];
+    const Slot& sl = A.sl[blockIdx.z / G.batch];
     const int tid = threadIdx.x, NT = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5;
     const int L = io.cu[s + 1] - io.cu[s];
@@ -1430,15 +1492,22 @@ cudaError_t configure_select() {
     return e;
 }
 
-cudaError_t launch_heads(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl, cudaStream_t st,
+cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, int* claim, cudaStream_t st,
                          int priority) {
-    const dim3 grid(g.Hkv, g.batch);
+    const dim3 grid(g.Hkv, g.batch, gr.nl);
     cudaError_t e = launch_prio(heads_pool_kernel, grid, dim3(kSelectThreads), g.NG > 1 ? (size_t)kPoolSmemBytes : 0, st,
-                                priority, false, g, io, sc, sl);
-    if (e == cudaSuccess)
-        e = launch_prio(heads_topk_kernel, grid, dim3(kSelectThreads), heads_smem_bytes(g), st, priority,
-                        /*programmatic=*/true, g, io, sc, sl);
-    return e;
+                                priority, false, g, gr, claim);
+    if (e != cudaSuccess) return e;
+    // Sixteen positions a thread while a block can hold the longest row so.
+    const auto reg = [&](auto kernel, int threads) {
+        return launch_prio(kernel, grid, dim3(threads), 0, st, priority, /*programmatic=*/true, g, gr);
+    };
+    if (g.max_len <= 256 * 16) return reg(heads_topk_reg_kernel<256, 16>, 256);
+    if (g.max_len <= 512 * 16) return reg(heads_topk_reg_kernel<512, 16>, 512);
+    if (g.max_len <= 1024 * 16) return reg(heads_topk_reg_kernel<1024, 16>, 1024);
+    if (g.max_len <= kMaxRegisterRow) return reg(heads_topk_reg_kernel<1024, 32>, 1024);
+    return launch_prio(heads_topk_kernel, grid, dim3(kSelectThreads), heads_smem_bytes(g), st, priority,
+                       /*programmatic=*/true, g, gr, sc.keys);
 }
 
 cudaError_t launch_select(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl, const Slot* prev,
@@ -1462,8 +1531,9 @@ cudaError_t launch_ada(const Geometry& g, const LayerIO& io, const Scratch& sc, 
                        io, sc, sl, ncall);
 }
 
-void launch_gather(const Geometry& g, const LayerIO& io, const Slot& sl, cudaStream_t st) {
-    gather_kernel<<<dim3((g.cap + 15) / 16, g.Hkv, g.batch), 256, 0, st>>>(g, io, sl);
+cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st) {
+    gather_kernel<<<dim3((g.cap + 15) / 16, g.Hkv, gr.nl * g.batch), 256, 0, st>>>(g, gr);
+    return cudaGetLastError();
 }
 
 }  // namespace kvec

@@ -30,6 +30,7 @@
 
 #include "kvec_internal.cuh"
 #include "sm100_ptx.cuh"
+#include "tile_loads.cuh"
 
 namespace kvec {
 
@@ -42,14 +43,16 @@ constexpr int kMaxStages = 3;                         // deepest operand ring
 constexpr int kWinReserveSms = 8;                     // SMs a window launch leaves to the other kernels
 
 struct WinArgs {
+    CUtensorMap kmap[kMaxGroup], qmap[kMaxGroup];
     Geometry G;
-    Scratch sc;
-    Slot sl;
+    int* err;
+    Slot sl[kMaxGroup];
     const int* cu;                  // device cu_seqlens
+    int upl;                        // units of a layer
     int Npad;                       // query rows padded to a multiple of 16 (MMA N)
     int kst;                        // operand stages
     int nacc;                       // accumulators = epilogue groups (4, or 2 when N > 128)
-    int units;                      // (sequence, candidate tile, head group) units of the launch
+    int units;                      // (layer, sequence, candidate tile, head group) units of the launch
     uint32_t tmem_cols;
     int fault;                      // test of the error path (kvec_set_test_fault): the first
                                     // accumulator is never signalled and its wait gives up early
@@ -82,7 +85,7 @@ __device__ __forceinline__ void win_abort(WinBars* bars, int* err) {
     atomicExch(err, 3);
 }
 
-// Unit u -> sequence s, candidate tile jt within it, head group ng, global
+// Unit u of a layer -> sequence s, candidate tile jt within it, head group ng, global
 // candidate tile tg; sequence s owns ceil(Lc / 128) * NG consecutive units.
 struct WinUnit {
     int s, jt, ng, tg, L, Lc, row0;
@@ -177,13 +180,12 @@ __device__ __forceinline__ void head_rows(uint32_t taddr, const float* __restric
 
 template <int GG>
 __global__ void __launch_bounds__(kWinThreads, 1)
-    window_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap,
-                  const __grid_constant__ WinArgs A) {
+    window_kernel(const __grid_constant__ WinArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if (threadIdx.x == 0) {
-        ptx::prefetch_tensormap(&kmap);
-        ptx::prefetch_tensormap(&qmap);
-        // The next launch on this stream (the next layer's row statistics) reads
+        ptx::prefetch_tensormap(&A.kmap[0]);
+        ptx::prefetch_tensormap(&A.qmap[0]);
+        // The next launch on this stream (the next group's row statistics) reads
         // nothing this grid writes and does not wait for it: let it be scheduled.
         asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     }
@@ -191,8 +193,8 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     // Scalars and pointers in registers: values read through a reference to the
     // parameter block would be re-read after every asm statement that clobbers memory.
     const Geometry G = A.G;
-    const Scratch sc = A.sc;
-    const Slot sl = A.sl;
+    int* const err = A.err;
+    const int upl = A.upl;
     const int* const cu_dev = A.cu;
     const int kst = A.kst, NA = A.nacc, units = A.units, fault = A.fault;
     const uint32_t tmem_cols = A.tmem_cols;
@@ -239,13 +241,14 @@ __global__ void __launch_bounds__(kWinThreads, 1)
             int fills[kMaxStages] = {0, 0, 0};
             for (int u = u0; u < units && !bars->abort_flag; u += ustep) {
                 WinUnit wu;
-                decode_unit(G, cu_dev, u, wu);
+                const int lay = u / upl;
+                decode_unit(G, cu_dev, u - lay * upl, wu);
                 const int h0 = wu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
                 bool stop = false;
                 for (int hh = 0; hh < nh; ++hh, ++it) {
                     const int st = it % kst, n = it / kst;
                     if (n > 0 && !ptx::mbar_wait_abortable(&bars->empty[st], (n - 1) & 1, &bars->abort_flag)) {
-                        win_abort(bars, sc.err);
+                        win_abort(bars, err);
                         stop = true;
                         break;
                     }
@@ -253,10 +256,9 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                     uint8_t* sq = sk + kKTileBytes;
                     const int h = h0 + hh;
                     ptx::mbar_arrive_expect_tx(&bars->full[st], (uint32_t)kKTileBytes + 2u * (uint32_t)R * 128u);
-                    ptx::tma_load_3d(sk, &kmap, &bars->full[st], 0, h, wu.row0, policy);
-                    ptx::tma_load_3d(sk + kKTileBytes / 2, &kmap, &bars->full[st], 64, h, wu.row0, policy);
-                    ptx::tma_load_4d(sq, &qmap, &bars->full[st], 0, h * G.g, 0, wu.s);
-                    ptx::tma_load_4d(sq + Npad * 128, &qmap, &bars->full[st], 64, h * G.g, 0, wu.s);
+                    ptx::tma_load_3d(sk, &A.kmap[lay], &bars->full[st], 0, h, wu.row0, policy);
+                    ptx::tma_load_3d(sk + kKTileBytes / 2, &A.kmap[lay], &bars->full[st], 64, h, wu.row0, policy);
+                    load_queries(sq, Npad * 128, &A.qmap[lay], &bars->full[st], G, h, wu.s);
                     ++fills[st];
                 }
                 if (stop) break;
@@ -273,7 +275,8 @@ __global__ void __launch_bounds__(kWinThreads, 1)
             bool stop = false;
             for (int u = u0; u < units && !stop; u += ustep) {
                 WinUnit wu;
-                decode_unit(G, cu_dev, u, wu);
+                const int lay = u / upl;
+                decode_unit(G, cu_dev, u - lay * upl, wu);
                 const int nh = min(G.HG, G.Hkv - wu.ng * G.HG);
                 for (int hh = 0; hh < nh; ++hh, ++it) {
                     const int st = it % kst, n = it / kst;
@@ -281,7 +284,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                     // Giving up on a stage in flight is safe: the producer drains its own loads.
                     if (bars->abort_flag || !ptx::mbar_wait_abortable(&bars->full[st], n & 1, &bars->abort_flag) ||
                         (ub > 0 && !ptx::mbar_wait_abortable(&bars->acc_empty[b], (ub - 1) & 1, &bars->abort_flag))) {
-                        win_abort(bars, sc.err);
+                        win_abort(bars, err);
                         stop = true;
                         break;
                     }
@@ -316,8 +319,8 @@ __global__ void __launch_bounds__(kWinThreads, 1)
         // dependent of: wait for it before the first read.
         asm volatile("griddepcontrol.wait;\n" ::: "memory");
         // This thread's rows (gtid, gtid + 128) of an item's statistics.
-        auto fetch = [&](int s, int h, float& a, float& b) {
-            const float2* src = sc.rowstat + ((size_t)s * G.Hkv + h) * R;
+        auto fetch = [&](const float2* rowstat, int s, int h, float& a, float& b) {
+            const float2* src = rowstat + ((size_t)s * G.Hkv + h) * R;
             a = b = 0.f;
             if (gtid < R) {
                 const float2 m = __ldcg(src + gtid);
@@ -332,7 +335,9 @@ __global__ void __launch_bounds__(kWinThreads, 1)
         bool failed = false;
         for (int u = u0, ul = 0; u < units; u += ustep, ++ul) {
             WinUnit wu;
-            decode_unit(G, cu_dev, u, wu);
+            const int lay = u / upl;
+                decode_unit(G, cu_dev, u - lay * upl, wu);
+            const Slot& sl = A.sl[lay];
             const int h0 = wu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
             const int t = wu.jt * kTileT + tok;                  // token within the sequence
             const int qmin = t - (wu.L - G.w);                   // > 0 only for tokens in the window part
@@ -353,14 +358,14 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                     }
                 }
                 if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                    if (lane == 0) win_abort(bars, sc.err);
+                    if (lane == 0) win_abort(bars, err);
                     failed = true;
                 }
                 __threadfence_block();
             }
             float pa = 0.f, pb = 0.f;
             int hh = (grp - it % NA + NA) % NA;   // the unit's first item for this group
-            if (!failed && hh < nh) fetch(wu.s, h0 + hh, pa, pb);
+            if (!failed && hh < nh) fetch(sl.rowstat, wu.s, h0 + hh, pa, pb);
             for (; hh < nh && !failed; hh += NA, ++k) {
                 // gtid 0 waits for the accumulator and publishes the outcome to the
                 // group with the statistics (one barrier per item).
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                     const bool ok = !bars->abort_flag &&
                                     ptx::mbar_wait_abortable(&bars->acc_full[grp], k & 1, &bars->abort_flag,
                                                              fault && it + hh == 0 ? kFaultWaitNs : 200000000ull);
-                    if (!ok) win_abort(bars, sc.err);
+                    if (!ok) win_abort(bars, err);
                     bars->gok[grp][k & 1] = ok ? 1 : 0;
                 }
                 float* rsb = rs_g + (k & 1) * 256;
@@ -379,7 +384,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                     failed = true;
                     break;
                 }
-                if (hh + NA < nh) fetch(wu.s, h0 + hh + NA, pa, pb);   // next item's rows, in flight
+                if (hh + NA < nh) fetch(sl.rowstat, wu.s, h0 + hh + NA, pa, pb);   // next item's rows, in flight
                 ptx::tc_fence_after();
                 float po = 0.f, poe = 0.f;
                 head_rows<GG>(tbase, rsb, G.g, G.w, qmin, G.sl2, qO, qOe, mg + tok, po, poe);
@@ -433,40 +438,53 @@ __global__ void __launch_bounds__(kWinThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// Tile-owning variant for O <= 16 and a group size with a straight-line epilogue
-// (g in {1, 2, 4, 7, 8}): a unit is T = 4 (or, with N > 128, 2) consecutive
-// candidate tiles of one sequence and one head group, and epilogue group j owns
-// tile j of the unit for every head.  The query block Q_h is loaded once per
-// (unit, head) into its own two-slot ring and serves the T tiles of the head, so
-// the K ring holds 32 KB stages only (4 in flight instead of 3 stages of K and
-// Q).  A thread keeps the running maxima over heads of its token's O last-row
-// group sums in registers, so the groups never synchronise; it adds its rows in
-// the same order as window_kernel, and the results are the same bits.
+// Tile-owning variant for O of 8 or 16 and a window that is a multiple of 8 (query
+// tiles ordered by query head, Geometry::jm).
+//
+// A unit is T consecutive candidate tiles of one sequence and one head group, and
+// the NA = T * P epilogue groups (one TMEM accumulator each) split it: group a owns
+// tile a / P for the heads a % P, a % P + P, ... of the head group.  The query block
+// Q_h is loaded once per (unit, head) into its own two-slot ring and serves the T
+// tiles of the head, so the K ring holds 32 KB stages only.  A thread keeps the
+// running maxima over its heads of its token's O last-row group sums in registers;
+// with P > 1 the P groups of a tile meet in shared memory at the unit's end (the
+// maximum does not depend on the order).  CTAs claim units from a per-launch
+// counter.
+//
+// Each row sum adds its positions in ascending order, as window_kernel does.
 // ---------------------------------------------------------------------------
 constexpr int kTileOMax = 16;     // largest O of the tile-owning variant (register maxima)
 constexpr int kMaxKStages = 6;
+constexpr int kUnitSlots = 4;     // claimed units in flight inside a CTA
 
 struct TileArgs {
+    CUtensorMap kmap[kMaxGroup], qmap[kMaxGroup];
     Geometry G;
-    Scratch sc;
-    Slot sl;
+    int* err;
+    int* claim;                     // the launch's unit counter, zero before the launch
+    Slot sl[kMaxGroup];
     const int* cu;
-    int Npad, kst, nacc, units, fault;
+    int upl;                        // units of a layer
+    int Npad, kst, nacc, T, units, fault;
 };
 
 struct __align__(8) TileBars {
     uint64_t k_full[kMaxKStages], k_empty[kMaxKStages], q_full[2], q_empty[2], acc_full[4], acc_empty[4];
+    uint64_t u_full[kUnitSlots], u_empty[kUnitSlots];
+    uint64_t m_full[4], m_empty[4];  // per tile, P > 1: the other groups' maxima are there / have been read
     uint64_t mma_done;
     uint32_t tmem_base;
     volatile int abort_flag;
-    volatile int gok[4][2];     // per group: the outcome of its accumulator wait, by item parity
+    volatile int unit[kUnitSlots];   // claimed unit (-1: no more work)
 };
 
-__host__ __device__ inline size_t tile_smem_bytes(int Npad, int kst) {
-    return 1024 + (size_t)kst * kKTileBytes + 2 * (size_t)Npad * 256 + 4 * 2 * 256 * sizeof(float) + sizeof(TileBars);
+// Shared memory: K stages | query slots [2] | normalisers [4 groups][2][256] | maxima [3][O][128] (P > 1) | barriers.
+__host__ __device__ inline size_t tile_smem_bytes(int Npad, int kst, bool shared_tiles) {
+    return 1024 + (size_t)kst * kKTileBytes + 2 * (size_t)Npad * 256 + 4 * 2 * 256 * sizeof(float) +
+           (shared_tiles ? 3 * kTileOMax * kTileT * sizeof(float) : 0) + sizeof(TileBars);
 }
 
-// Unit u -> sequence s, first candidate tile j0 of the unit, its tile count nt,
+// Unit u of a layer -> sequence s, first candidate tile j0 of the unit, its tile count nt,
 // head group ng, global candidate tile of j0.
 struct TileUnit {
     int s, j0, nt, ng, tg0, L, Lc, row0;
@@ -498,87 +516,70 @@ __device__ __forceinline__ bool decode_tile_unit(const Geometry& G, const int* c
     return false;
 }
 
-// One head of this thread's token: rows [qOe, qO) add to poe only, rows [qO, w)
-// to po, to poe when q >= qOe, and to the running maxima mx[q - qO] (ascending q
-// in both parts, as head_rows).
+// Group sums G_h[q] of eight window positions q0 .. q0 + 7 of this thread's token:
+// sum over the query heads j of 2^(s * scale * log2 e - normaliser), columns
+// j * w + q.  nrs: the normalisers.  GG > 0: the group size g, known at compile
+// time (the columns of up to four query heads are loaded together).
 template <int GG>
-__device__ __forceinline__ void head_rows_tile(uint32_t taddr, const float* __restrict__ rsb, int w, int qmin,
-                                               float sl2, int qO, int qOe, float* mx, float& po, float& poe) {
-    constexpr int QPC = 32 / GG, CW = QPC * GG;
-    for (int qb = qOe; qb < qO; qb += QPC) {
-        const int c0 = qb * GG;
-        float v[32];
-        ptx::tmem_ld32(taddr + (uint32_t)c0, v);
-        ptx::tmem_wait_ld();
-        float pr[CW];
+__device__ __forceinline__ void group_sums8(uint32_t taddr, const float* __restrict__ nrs, int g, int w, int q0, float sl2,
+                                            float* gs) {
+    auto add_head = [&](const float* v, int j, bool first) {
+        const float4* n4 = reinterpret_cast<const float4*>(nrs + j * w + q0);
+        const float4 na = n4[0], nb = n4[1];
+        const float n[8] = {na.x, na.y, na.z, na.w, nb.x, nb.y, nb.z, nb.w};
 #pragma unroll
-        for (int i = 0; i < CW; ++i) pr[i] = ptx::ex2(fmaf(v[i], sl2, -rsb[c0 + i]));
-#pragma unroll
-        for (int k = 0; k < QPC; ++k) {
-            float gs = 0.f;
-#pragma unroll
-            for (int j = 0; j < GG; ++j) gs += pr[k * GG + j];
-            const int q = qb + k;
-            gs = q >= qmin ? gs : 0.f;
-            if (q < qO) poe += gs;
+        for (int k = 0; k < 8; ++k) {
+            const float e = ptx::ex2(fmaf(v[k], sl2, -n[k]));
+            gs[k] = first ? e : gs[k] + e;
         }
-    }
+    };
+    if constexpr (GG > 0) {
 #pragma unroll
-    for (int c = 0; c < (kTileOMax + QPC - 1) / QPC; ++c) {
-        const int qb = qO + c * QPC;
-        if (qb >= w) break;
-        const int c0 = qb * GG;
-        float v[32];
-        ptx::tmem_ld32(taddr + (uint32_t)c0, v);
-        ptx::tmem_wait_ld();
-        float pr[CW];
+        for (int j0 = 0; j0 < GG; j0 += 4) {
+            float v[4][8];
 #pragma unroll
-        for (int i = 0; i < CW; ++i) pr[i] = ptx::ex2(fmaf(v[i], sl2, -rsb[c0 + i]));
+            for (int jj = 0; jj < 4; ++jj)
+                if (j0 + jj < GG) ptx::tmem_ld8(taddr + (uint32_t)((j0 + jj) * w + q0), v[jj]);
+            ptx::tmem_wait_ld();
 #pragma unroll
-        for (int k = 0; k < QPC; ++k) {
-            const int idx = c * QPC + k;
-            if (idx < kTileOMax) {
-                float gs = 0.f;
+            for (int jj = 0; jj < 4; ++jj)
+                if (j0 + jj < GG) add_head(v[jj], j0 + jj, j0 + jj == 0);
+        }
+    } else {
 #pragma unroll
-                for (int j = 0; j < GG; ++j) gs += pr[k * GG + j];
-                const int q = qb + k;
-                gs = q >= qmin ? gs : 0.f;
-                if (q < w) {
-                    if (q >= qOe) poe += gs;
-                    po += gs;
-                    mx[idx] = fmaxf(mx[idx], gs);
-                }
-            }
+        for (int k = 0; k < 8; ++k) gs[k] = 0.f;   // 0 + x is x: the sums start at +0 or above
+        for (int j = 0; j < g; ++j) {
+            float v[8];
+            ptx::tmem_ld8(taddr + (uint32_t)(j * w + q0), v);
+            ptx::tmem_wait_ld();
+            add_head(v, j, false);
         }
     }
 }
 
 template <int GG>
-__global__ void __launch_bounds__(kWinThreads, 1)
-    window_tiles_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap qmap,
-                        const __grid_constant__ TileArgs A) {
+__global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __grid_constant__ TileArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if (threadIdx.x == 0) {
-        ptx::prefetch_tensormap(&kmap);
-        ptx::prefetch_tensormap(&qmap);
-        // The next launch on this stream (the next layer's row statistics) reads
+        ptx::prefetch_tensormap(&A.kmap[0]);
+        ptx::prefetch_tensormap(&A.qmap[0]);
+        // The next launch on this stream (the next group's row statistics) reads
         // nothing this grid writes and does not wait for it: let it be scheduled.
         asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     }
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const Geometry G = A.G;
-    const Scratch sc = A.sc;
-    const Slot sl = A.sl;
+    int* const err = A.err;
+    const int upl = A.upl;
     const int* const cu_dev = A.cu;
-    const int kst = A.kst, NA = A.nacc, units = A.units, fault = A.fault;
-    const int Npad = A.Npad, R = G.R;
-    const int T = NA;                                        // tiles per unit = epilogue groups
+    const int kst = A.kst, NA = A.nacc, T = A.T, units = A.units, fault = A.fault;
+    const int Npad = A.Npad, R = G.R, P = NA / T;
     uint8_t* sK = smem;                                      // kst x 32 KB
     uint8_t* sQ = sK + (size_t)kst * kKTileBytes;            // 2 slots x Npad x 256 B
     float* rsm = reinterpret_cast<float*>(sQ + 2 * (size_t)Npad * 256);   // [4][2][256]
-    TileBars* bars = reinterpret_cast<TileBars*>(rsm + 4 * 2 * 256);
+    float* mbuf = rsm + 4 * 2 * 256;                         // [3][O][128], P > 1 only
+    TileBars* bars = reinterpret_cast<TileBars*>(mbuf + (P > 1 ? 3 * kTileOMax * kTileT : 0));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int u0 = blockIdx.x, ustep = gridDim.x;
 
     if (threadIdx.x == 32) {
         for (int i = 0; i < kst; ++i) {
@@ -593,6 +594,14 @@ __global__ void __launch_bounds__(kWinThreads, 1)
             ptx::mbar_init(&bars->acc_full[i], 1);
             ptx::mbar_init(&bars->acc_empty[i], 4);   // one arrival per warp of the group
         }
+        for (int i = 0; i < T; ++i) {
+            ptx::mbar_init(&bars->m_full[i], 4 * (P > 1 ? P - 1 : 1));
+            ptx::mbar_init(&bars->m_empty[i], 4);
+        }
+        for (int i = 0; i < kUnitSlots; ++i) {
+            ptx::mbar_init(&bars->u_full[i], 1);
+            ptx::mbar_init(&bars->u_empty[i], 1 + 4 * NA);   // the MMA issuer and every epilogue warp
+        }
         ptx::mbar_init(&bars->mma_done, 1);
         bars->abort_flag = 0;
         ptx::fence_barrier_init();
@@ -605,200 +614,308 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
+    auto give_up = [&]() {
+        bars->abort_flag = 1;
+        atomicExch(err, 3);
+    };
+    // The next claimed unit for a warp of the MMA issuer or the epilogue; -1: no more
+    // work, -2: gave up.
+    auto take_unit = [&](int di) {
+        const int ds = di % kUnitSlots;
+        if (!ptx::warp_wait(&bars->u_full[ds], (di / kUnitSlots) & 1, &bars->abort_flag)) {
+            if (lane == 0) give_up();
+            return -2;
+        }
+        const int u = ptx::warp_uniform(bars->unit[ds]);
+        if (lane == 0) ptx::mbar_arrive(&bars->u_empty[ds]);
+        return u;
+    };
+    auto uniform_unit = [&](int u, TileUnit& tu) {
+        const int lay = u / upl;
+        decode_tile_unit(G, cu_dev, T, u - lay * upl, tu);
+        tu.s = ptx::warp_uniform(tu.s);
+        tu.nt = ptx::warp_uniform(tu.nt);
+        tu.ng = ptx::warp_uniform(tu.ng);
+        tu.row0 = ptx::warp_uniform(tu.row0);
+        return lay;
+    };
 
+    // The producer and the MMA issuer run as whole warps and elect a lane for the
+    // instructions that one thread issues (see score_kernel).
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            const uint64_t policy = ptx::policy_evict_first();   // the K tiles' last use
-            int qi = 0, ki = 0;
-            int kfills[kMaxKStages] = {0, 0, 0, 0, 0, 0};
-            int qfills[2] = {0, 0};
-            bool stop = false;
-            for (int u = u0; u < units && !stop; u += ustep) {
-                TileUnit tu;
-                decode_tile_unit(G, cu_dev, T, u, tu);
-                const int h0 = tu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
-                for (int hh = 0; hh < nh && !stop; ++hh) {
-                    const int h = h0 + hh;
-                    const int qs = qi & 1, nq = qi >> 1;
-                    if (nq > 0 && !ptx::mbar_wait_abortable(&bars->q_empty[qs], (nq - 1) & 1, &bars->abort_flag)) {
-                        bars->abort_flag = 1;
-                        atomicExch(sc.err, 3);
-                        stop = true;
-                        break;
-                    }
-                    if (bars->abort_flag) {
-                        stop = true;
-                        break;
-                    }
-                    uint8_t* q = sQ + (size_t)qs * Npad * 256;
+        const uint64_t policy = ptx::policy_evict_first();   // the K tiles' last use
+        int qi = 0, ki = 0, st = 0;
+        uint32_t kphase = 0u;   // bit st: the stage has been filled an odd number of times
+        bool stop = false;
+        int next = 0;
+        if (lane == 0) next = atomicAdd(A.claim, 1);
+        for (int di = 0; !stop; ++di) {
+            const int ds = di % kUnitSlots, nd = di / kUnitSlots;
+            if (nd > 0 && !ptx::warp_wait(&bars->u_empty[ds], (nd - 1) & 1, &bars->abort_flag)) {
+                stop = true;
+                break;
+            }
+            const int u = ptx::warp_uniform(bars->abort_flag ? units : next);
+            if (lane == 0) {
+                bars->unit[ds] = u < units ? u : -1;
+                ptx::mbar_arrive(&bars->u_full[ds]);
+            }
+            if (u >= units) break;
+            if (lane == 0) next = atomicAdd(A.claim, 1);   // arrives while this unit is loaded
+            TileUnit tu;
+            const int lay = uniform_unit(u, tu);
+            const int h0 = tu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
+            for (int hh = 0; hh < nh && !stop; ++hh) {
+                const int h = h0 + hh;
+                const int qs = qi & 1, nq = qi >> 1;
+                if (nq > 0 && !ptx::warp_wait(&bars->q_empty[qs], (nq - 1) & 1, &bars->abort_flag)) {
+                    stop = true;
+                    break;
+                }
+                if (ptx::elect_one()) {
                     ptx::mbar_arrive_expect_tx(&bars->q_full[qs], 2u * (uint32_t)R * 128u);
-                    ptx::tma_load_4d(q, &qmap, &bars->q_full[qs], 0, h * G.g, 0, tu.s);
-                    ptx::tma_load_4d(q + Npad * 128, &qmap, &bars->q_full[qs], 64, h * G.g, 0, tu.s);
-                    ++qfills[qs];
-                    ++qi;
-                    for (int j = 0; j < tu.nt; ++j) {
-                        const int st = ki % kst, nk = ki / kst;
-                        if (nk > 0 && !ptx::mbar_wait_abortable(&bars->k_empty[st], (nk - 1) & 1, &bars->abort_flag)) {
-                            bars->abort_flag = 1;
-                            atomicExch(sc.err, 3);
-                            stop = true;
-                            break;
-                        }
+                    load_queries(sQ + (size_t)qs * Npad * 256, (uint32_t)Npad * 128u, &A.qmap[lay], &bars->q_full[qs], G, h,
+                                 tu.s);
+                }
+                __syncwarp();
+                ++qi;
+                for (int j = 0; j < tu.nt; ++j) {
+                    if (ki >= kst && !ptx::warp_wait(&bars->k_empty[st], ((kphase >> st) & 1u) ^ 1u, &bars->abort_flag)) {
+                        stop = true;
+                        break;
+                    }
+                    if (ptx::elect_one()) {
                         uint8_t* sk = sK + (size_t)st * kKTileBytes;
                         const int row = tu.row0 + j * kTileT;
                         ptx::mbar_arrive_expect_tx(&bars->k_full[st], (uint32_t)kKTileBytes);
-                        ptx::tma_load_3d(sk, &kmap, &bars->k_full[st], 0, h, row, policy);
-                        ptx::tma_load_3d(sk + kKTileBytes / 2, &kmap, &bars->k_full[st], 64, h, row, policy);
-                        ++kfills[st];
-                        ++ki;
+                        ptx::tma_load_3d(sk, &A.kmap[lay], &bars->k_full[st], 0, h, row, policy);
+                        ptx::tma_load_3d(sk + kKTileBytes / 2, &A.kmap[lay], &bars->k_full[st], 64, h, row, policy);
                     }
+                    __syncwarp();
+                    kphase ^= 1u << st;
+                    ++ki;
+                    st = st + 1 == kst ? 0 : st + 1;
                 }
             }
-            // Drain: every issued copy lands before the CTA may exit.
-            for (int st = 0; st < kst; ++st)
-                if (kfills[st] > 0) ptx::mbar_wait(&bars->k_full[st], (kfills[st] - 1) & 1, 50000000ull);
-            for (int qs = 0; qs < 2; ++qs)
-                if (qfills[qs] > 0) ptx::mbar_wait(&bars->q_full[qs], (qfills[qs] - 1) & 1, 50000000ull);
         }
+        if (stop && lane == 0) give_up();
+        // Drain: every issued copy lands before the CTA may exit.
+        for (int b = 0; b < kst && b < ki; ++b)
+            ptx::mbar_wait(&bars->k_full[b], ((ki - b + kst - 1) / kst - 1) & 1, 50000000ull);
+        for (int b = 0; b < 2 && b < qi; ++b)
+            ptx::mbar_wait(&bars->q_full[b], ((qi - b + 1) / 2 - 1) & 1, 50000000ull);
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = ptx::idesc_bf16_f32(128, Npad);
-            int qi = 0, ki = 0, first = 1;
-            int cnt[4] = {0, 0, 0, 0};
-            bool stop = false;
-            for (int u = u0; u < units && !stop; u += ustep) {
-                TileUnit tu;
-                decode_tile_unit(G, cu_dev, T, u, tu);
-                const int nh = min(G.HG, G.Hkv - tu.ng * G.HG);
-                for (int hh = 0; hh < nh && !stop; ++hh) {
-                    const int qs = qi & 1;
-                    if (bars->abort_flag ||
-                        !ptx::mbar_wait_abortable(&bars->q_full[qs], (qi >> 1) & 1, &bars->abort_flag)) {
-                        bars->abort_flag = 1;
-                        atomicExch(sc.err, 3);
+        const uint32_t idesc = ptx::idesc_bf16_f32(128, Npad);
+        const uint64_t qdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sQ)), kdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sK));
+        const uint32_t qhalf = (uint32_t)Npad * 128u;
+        int qi = 0, st = 0, first = 1;
+        uint32_t kphase = 0u, used = 0u, aphase = 0u;   // per stage / accumulator
+        bool stop = false;
+        for (int di = 0; !stop; ++di) {
+            const int u = take_unit(di);
+            if (u < 0) break;
+            TileUnit tu;
+            uniform_unit(u, tu);
+            const int nh = min(G.HG, G.Hkv - tu.ng * G.HG);
+            for (int hh = 0, hp = 0; hh < nh && !stop; ++hh, hp = hp + 1 == P ? 0 : hp + 1) {
+                const int qs = qi & 1;
+                if (!ptx::warp_wait(&bars->q_full[qs], (qi >> 1) & 1, &bars->abort_flag)) {
+                    stop = true;
+                    break;
+                }
+                for (int j = 0; j < tu.nt; ++j) {
+                    const int b = j * P + hp;
+                    // Giving up on a stage in flight is safe: the producer drains its own loads.
+                    if (!ptx::warp_wait(&bars->k_full[st], (kphase >> st) & 1u, &bars->abort_flag) ||
+                        (((used >> b) & 1u) != 0u &&
+                         !ptx::warp_wait(&bars->acc_empty[b], ((aphase >> b) & 1u) ^ 1u, &bars->abort_flag))) {
                         stop = true;
                         break;
                     }
-                    const uint32_t sq = ptx::smem_u32(sQ + (size_t)qs * Npad * 256);
-                    for (int j = 0; j < tu.nt; ++j) {
-                        const int st = ki % kst;
-                        // Giving up on a stage in flight is safe: the producer drains its own loads.
-                        if (!ptx::mbar_wait_abortable(&bars->k_full[st], (ki / kst) & 1, &bars->abort_flag) ||
-                            (cnt[j] > 0 &&
-                             !ptx::mbar_wait_abortable(&bars->acc_empty[j], (cnt[j] - 1) & 1, &bars->abort_flag))) {
-                            bars->abort_flag = 1;
-                            atomicExch(sc.err, 3);
-                            stop = true;
-                            break;
-                        }
-                        ptx::tc_fence_after();
-                        const uint32_t sk = ptx::smem_u32(sK + (size_t)st * kKTileBytes);
-                        const uint32_t d = tmem + (uint32_t)(j * Npad);
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one()) {
+                        const uint64_t kd = kdesc + (uint32_t)(st * (kKTileBytes >> 4)), qd = qdesc + (uint32_t)qs * (qhalf >> 3);
+                        const uint32_t d = tmem + (uint32_t)(b * Npad);
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk) {
-                            const int half = kk >> 2, kin = kk & 3;
-                            const uint64_t ad = ptx::smem_desc_k_sw128(sk + half * (kKTileBytes / 2) + kin * 32);
-                            const uint64_t bd = ptx::smem_desc_k_sw128(sq + half * Npad * 128 + kin * 32);
-                            ptx::mma_bf16(d, ad, bd, idesc, kk > 0 ? 1u : 0u);
+                            const uint32_t half = kk >> 2, kin = kk & 3;
+                            ptx::mma_bf16(d, kd + half * (kKTileBytes >> 5) + kin * 2, qd + half * (qhalf >> 4) + kin * 2, idesc,
+                                          kk > 0 ? 1u : 0u);
                         }
                         ptx::mma_commit(&bars->k_empty[st]);
-                        if (!(fault && first)) ptx::mma_commit(&bars->acc_full[j]);
-                        first = 0;
-                        ++ki;
-                        ++cnt[j];
+                        if (!(fault && first)) ptx::mma_commit(&bars->acc_full[b]);
+                        if (j + 1 == tu.nt) ptx::mma_commit(&bars->q_empty[qs]);
                     }
-                    ptx::mma_commit(&bars->q_empty[qs]);
-                    ++qi;
+                    __syncwarp();
+                    first = 0;
+                    kphase ^= 1u << st;
+                    used |= 1u << b;
+                    aphase ^= 1u << b;
+                    st = st + 1 == kst ? 0 : st + 1;
                 }
+                ++qi;
             }
-            ptx::mma_commit(&bars->mma_done);
         }
+        if (stop && lane == 0) give_up();
+        if (ptx::elect_one()) ptx::mma_commit(&bars->mma_done);
+        __syncwarp();
     } else if (warp < 2 + 4 * NA) {
         // ------------------------------------------------------------ epilogue
-        const int grp = (warp - 2) >> 2;                  // the tile of the unit this group owns
+        const int grp = (warp - 2) >> 2;                  // accumulator
+        const int tile = grp / P, par = grp - tile * P;   // tile of the unit, heads par, par + P, ...
         const int gtid = threadIdx.x - 64 - grp * 128;
         const int quad = warp & 3;
         const int tok = quad * 32 + lane;
-        const int bar_id = 1 + grp;
-        const int qO = G.w - G.O, qOe = G.w - G.Oe;
-        const float invO = 1.f / (float)G.O, invOe = 1.f / (float)G.Oe;
+        const int w = G.w, g = G.g, O = G.O;
+        const int qO = w - O, qOe = w - G.Oe;
+        const float invO = 1.f / (float)O, invOe = 1.f / (float)G.Oe;
+        const float sl2 = G.sl2;
         const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(grp * Npad);
         float* rs_g = rsm + grp * 2 * 256;
+        // This thread's columns of an item, gtid and gtid + 128: their rows in the statistics.
+        const int r0 = gtid % w * g + gtid / w, r1 = (gtid + 128) % w * g + (gtid + 128) / w;
         asm volatile("griddepcontrol.wait;\n" ::: "memory");
-        auto fetch = [&](int s, int h, float& a, float& b) {
-            const float2* src = sc.rowstat + ((size_t)s * G.Hkv + h) * R;
+        auto fetch = [&](const float2* rowstat, int s, int h, float& a, float& b) {
+            const float2* src = rowstat + ((size_t)s * G.Hkv + h) * R;
             a = b = 0.f;
             if (gtid < R) {
-                const float2 m = __ldcg(src + gtid);
+                const float2 m = __ldcg(src + r0);
                 a = m.x + __log2f(m.y);
             }
             if (gtid + 128 < R) {
-                const float2 m = __ldcg(src + gtid + 128);
+                const float2 m = __ldcg(src + r1);
                 b = m.x + __log2f(m.y);
             }
         };
-        int k = 0;
-        bool failed = false;
-        for (int u = u0; u < units && !failed; u += ustep) {
+        uint32_t k = 0u, meets = 0u;   // items of this group and meetings of its tile's groups so far
+        bool failed = false;           // this warp gave up on a wait
+        for (int di = 0;; ++di) {
+            const int u = failed ? -2 : take_unit(di);
+            // The group's warps leave together: whoever gave up says so at the next
+            // group barrier, where all of them hear it.
+            if (ptx::named_bar_or(1 + grp, 128, u == -2) || u < 0) break;
+            const int lay = u / upl;
             TileUnit tu;
-            decode_tile_unit(G, cu_dev, T, u, tu);
-            if (grp >= tu.nt) continue;   // this group's tile is past the sequence's last
+            decode_tile_unit(G, cu_dev, T, u - lay * upl, tu);
+            if (tile >= tu.nt) continue;   // this group's tile is past the sequence's last
+            const Slot& sl = A.sl[lay];
+            const float2* rowstat = sl.rowstat;
             const int h0 = tu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
-            const int t = (tu.j0 + grp) * kTileT + tok;
-            const int qmin = t - (tu.L - G.w);
+            const int t0 = (tu.j0 + tile) * kTileT, t = t0 + tok;
+            // Rows q < qmin come before the token (it lies in the window part, a candidate
+            // only when every position is one): their attention to it is 0.
+            const int qmin = t - (tu.L - w);
+            const bool masked = G.wk == 0 && t0 + kTileT - 1 > tu.L - w;
             float mx[kTileOMax];
 #pragma unroll
             for (int i = 0; i < kTileOMax; ++i) mx[i] = 0.f;
-            float pa, pb;
-            fetch(tu.s, h0, pa, pb);
-            for (int hh = 0; hh < nh; ++hh, ++k) {
-                if (gtid == 0) {
-                    const bool ok = !bars->abort_flag &&
-                                    ptx::mbar_wait_abortable(&bars->acc_full[grp], k & 1, &bars->abort_flag,
-                                                             fault && k == 0 && grp == 0 ? kFaultWaitNs
-                                                                                         : 200000000ull);
-                    if (!ok) {
-                        bars->abort_flag = 1;
-                        atomicExch(sc.err, 3);
-                    }
-                    bars->gok[grp][k & 1] = ok ? 1 : 0;
+            float pa = 0.f, pb = 0.f;
+            if (par < nh) fetch(rowstat, tu.s, h0 + par, pa, pb);
+            for (int hh = par; hh < nh; hh += P, ++k) {
+                // The group's threads exchange the normalisers while the accumulator fills.
+                float* nrs = rs_g + (k & 1u) * 256;
+                nrs[gtid] = pa;
+                nrs[gtid + 128] = pb;
+                // One warp of the group polls, the others wait in the barrier (a polling
+                // warp takes issue slots from those that compute).
+                bool ok = true;
+                if (gtid < 32) {
+                    ok = ptx::warp_wait(&bars->acc_full[grp], k & 1u, &bars->abort_flag,
+                                        fault && k == 0u && grp == 0 ? kFaultWaitNs : 200000000ull);
+                    if (!ok && lane == 0) give_up();
                 }
-                float* rsb = rs_g + (k & 1) * 256;
-                rsb[gtid] = pa;
-                rsb[gtid + 128] = pb;
-                ptx::named_bar_sync(bar_id, 128);
-                if (!bars->gok[grp][k & 1]) {
-                    failed = true;
-                    break;
-                }
-                if (hh + 1 < nh) fetch(tu.s, h0 + hh + 1, pa, pb);   // the next head's rows, in flight
+                failed = ptx::named_bar_or(1 + grp, 128, !ok);
+                if (failed) break;
+                if (hh + P < nh) fetch(rowstat, tu.s, h0 + hh + P, pa, pb);   // the next head's rows, in flight
                 ptx::tc_fence_after();
                 float po = 0.f, poe = 0.f;
-                head_rows_tile<GG>(tbase, rsb, G.w, qmin, G.sl2, qO, qOe, mx, po, poe);
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bars->acc_empty[grp]);
+                float gs[8];
+                auto sums = [&](int q0) {
+                    group_sums8<GG>(tbase, nrs, g, w, q0, sl2, gs);
+                    if (masked) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) gs[i] = q0 + i < qmin ? 0.f : gs[i];
+                    }
+                };
+                for (int q0 = qOe & ~7; q0 < qO; q0 += 8) {
+                    sums(q0);
+                    if (q0 >= qOe) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) poe += gs[i];
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (q0 + i >= qOe) poe += gs[i];
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < kTileOMax / 8; ++c) {
+                    const int q0 = qO + 8 * c;
+                    if (q0 >= w) break;
+                    sums(q0);
+                    if (q0 + 8 >= w) {   // the accumulator is in registers
+                        ptx::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive(&bars->acc_empty[grp]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float x = gs[i];
+                        if (q0 + i >= qOe) poe += x;
+                        po += x;
+                        mx[8 * c + i] = fmaxf(mx[8 * c + i], x);
+                    }
+                }
                 if (t < tu.Lc) {
                     const size_t row = (size_t)tu.s * G.Hkv + h0 + hh;
                     sl.rawO[row * G.ML + t] = po * invO;
                     sl.rawOe[row * G.ML + t] = poe * invOe;
                 }
             }
-            if (failed) break;
+            if (failed) continue;
+            if (P > 1) {
+                // The P groups of the tile: their maxima meet in the first one's registers.
+                float* mb = mbuf + (size_t)(tile * (P - 1)) * kTileOMax * kTileT + tok;
+                int ok = 1;
+                if (lane == 0) {
+                    if (par > 0)
+                        ok = meets == 0u || ptx::mbar_wait_abortable(&bars->m_empty[tile], (meets - 1u) & 1u, &bars->abort_flag);
+                    else
+                        ok = ptx::mbar_wait_abortable(&bars->m_full[tile], meets & 1u, &bars->abort_flag);
+                    if (!ok) give_up();
+                }
+                ++meets;
+                if (!__shfl_sync(0xffffffffu, ok, 0)) {
+                    failed = true;
+                    continue;
+                }
+                __syncwarp();   // what lane 0 waited for is there for every lane
+                if (par > 0) {
+#pragma unroll
+                    for (int i = 0; i < kTileOMax; ++i) mb[((par - 1) * kTileOMax + i) * kTileT] = mx[i];
+                } else {
+                    for (int o = 0; o < P - 1; ++o)
+#pragma unroll
+                        for (int i = 0; i < kTileOMax; ++i) mx[i] = fmaxf(mx[i], mb[(o * kTileOMax + i) * kTileT]);
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(par > 0 ? &bars->m_full[tile] : &bars->m_empty[tile]);
+            }
+            if (par > 0) continue;
             // I[t] = (1/O) sum over the last O rows of the maxima over the heads (or
             // this head group's maxima, combined by the heads kernel).
             if (G.NG > 1) {
-                float* wp = sl.wpart + ((size_t)(tu.tg0 + grp) * G.NG + tu.ng) * G.O * kTileT;
+                float* wp = sl.wpart + ((size_t)(tu.tg0 + tile) * G.NG + tu.ng) * O * kTileT;
 #pragma unroll
                 for (int i = 0; i < kTileOMax; ++i)
-                    if (i < G.O) wp[i * kTileT + tok] = mx[i];
+                    if (i < O) wp[i * kTileT + tok] = mx[i];
             } else if (t < tu.Lc) {
                 float ip = 0.f;
 #pragma unroll
                 for (int i = 0; i < kTileOMax; ++i)
-                    if (i < G.O) ip += mx[i];
+                    if (i < O) ip += mx[i];
                 sl.rawI[(size_t)tu.s * G.ML + t] = ip * invO;
             }
         }
@@ -820,7 +937,7 @@ int kst_for(int Npad, int O) {
     return k;
 }
 
-// Units of a launch: (sequence, candidate tile, head group).
+// Units of a layer: (sequence, candidate tile, head group).
 int units_of(const Geometry& g) { return g.win_tiles * g.NG; }
 
 }  // namespace
@@ -838,46 +955,25 @@ cudaError_t configure_window(const Geometry& g) {
     for (auto fn : {window_kernel<0>, window_kernel<1>, window_kernel<2>, window_kernel<4>, window_kernel<7>,
                     window_kernel<8>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemWin);
-    for (auto fn : {window_tiles_kernel<1>, window_tiles_kernel<2>, window_tiles_kernel<4>, window_tiles_kernel<7>,
-                    window_tiles_kernel<8>})
+    for (auto fn : {window_tiles_kernel<0>, window_tiles_kernel<1>, window_tiles_kernel<2>, window_tiles_kernel<4>,
+                    window_tiles_kernel<7>, window_tiles_kernel<8>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemWin);
     return e;
 }
 
 namespace {
 
-int tile_kst_for(int Npad) {
+// SMs of a window grid: a few are left to the selection chain and the other
+// layers' kernels.
+int usable_sms(int num_sms) { return num_sms > 2 * kWinReserveSms ? num_sms - kWinReserveSms : num_sms; }
+
+int tile_kst_for(int Npad, bool shared_tiles) {
     int k = kMaxKStages;
-    while (k > 1 && tile_smem_bytes(Npad, k) > (size_t)kMaxSmemWin) --k;
+    while (k > 1 && tile_smem_bytes(Npad, k, shared_tiles) > (size_t)kMaxSmemWin) --k;
     return k;
 }
 
-// The tile variant applies to O <= 16 with a straight-line group size, when every
-// 32-column TMEM load of its epilogue (chunks starting at rows w - O' and w - O)
-// stays inside the 512 allocated columns.
-bool tile_variant_fits(const Geometry& g) {
-    if (g.O > kTileOMax || !(g.g == 1 || g.g == 2 || g.g == 4 || g.g == 7 || g.g == 8)) return false;
-    const int qpc = 32 / g.g, qO = g.w - g.O, qOe = g.w - g.Oe;
-    const int Npad = npad_of(g.R), nacc = Npad <= 128 ? 4 : 2;
-    int maxcol = 0;
-    for (int qb = qOe; qb < qO; qb += qpc) maxcol = maxcol > qb * g.g + 32 ? maxcol : qb * g.g + 32;
-    for (int c = 0; c < (kTileOMax + qpc - 1) / qpc; ++c) {
-        const int qb = qO + c * qpc;
-        if (qb >= g.w) break;
-        maxcol = maxcol > qb * g.g + 32 ? maxcol : qb * g.g + 32;
-    }
-    return (nacc - 1) * Npad + maxcol <= 512;
-}
-
-// Candidate tiles per unit of the tile-owning variant: one TMEM accumulator and
-// epilogue group each (nacc * Npad <= 512 columns).  With the caller's
-// log-sum-exp no score grid runs beside the window grids, and units of three
-// tiles (more units, a shorter tail) were faster than four there (ragged batch
-// of 8: 2.09 -> 1.90 ms per step), while beside the score grids they were
-// slower (3.02 -> 3.06 ms); two tiles were slower in both.
-int tile_unit_tiles(const Geometry& g, bool lse) { return npad_of(g.R) <= 128 ? (lse ? 3 : 4) : 2; }
-
-// Units of the tile-owning variant: groups of T candidate tiles per sequence and head group.
+// A layer's units of the tile-owning variant: groups of T candidate tiles per sequence and head group.
 int tile_units_of(const Geometry& g, const int* cu_host, int T) {
     int units = 0;
     for (int b = 0; b < g.batch; ++b) {
@@ -888,20 +984,41 @@ int tile_units_of(const Geometry& g, const int* cu_host, int T) {
     return units;
 }
 
-cudaError_t launch_window_tiles(const ScorePlan& sp, const Geometry& g, const LayerIO& io, const Scratch& sc,
-                                const Slot& sl, cudaStream_t st, bool after_own_launch) {
+// Candidate tiles per unit: with more of them the query blocks are loaded less
+// often (32 KB for every T tiles of 32 KB), with fewer there are more units; the
+// most that still give every usable SM a unit.
+int tile_unit_tiles(const Geometry& g, int nl, int usable) {
+    int T = npad_of(g.R) <= 128 ? 4 : 2;
+    while (T > 1 && tile_units_of(g, g.cu_host, T) * nl < usable) T /= 2;
+    return T;
+}
+
+template <class Args>
+void set_layers(Args* a, const ScorePlan& sp, const Geometry& g, const Group& gr, const Scratch& sc) {
+    for (int l = 0; l < gr.nl; ++l) {
+        a->kmap[l] = sp.kmap[l];
+        a->qmap[l] = sp.qmap[l];
+        a->sl[l] = gr.sl[l];
+    }
+    a->G = g;
+    a->err = sc.err;
+    a->cu = gr.io[0].cu;
+}
+
+cudaError_t launch_window_tiles(const ScorePlan& sp, const Geometry& g, const Group& gr, const Scratch& sc,
+                                int* claim, cudaStream_t st, bool after_own_launch) {
     TileArgs a{};
-    a.G = g;
-    a.sc = sc;
-    a.sl = sl;
-    a.cu = io.cu;
+    set_layers(&a, sp, g, gr, sc);
+    const int usable = usable_sms(sp.num_sms);
+    a.claim = claim + 1;
     a.Npad = npad_of(g.R);
-    a.nacc = tile_unit_tiles(g, io.lse != nullptr);
-    a.kst = tile_kst_for(a.Npad);
-    a.units = tile_units_of(g, g.cu_host, a.nacc);
+    a.nacc = a.Npad <= 128 ? 4 : 2;   // nacc * Npad <= 512 TMEM columns
+    a.T = tile_unit_tiles(g, gr.nl, usable);
+    a.kst = tile_kst_for(a.Npad, a.T < a.nacc);
+    a.upl = tile_units_of(g, g.cu_host, a.T);
+    a.units = gr.nl * a.upl;
     a.fault = test_fault() == 1 ? 1 : 0;
-    const size_t smem = tile_smem_bytes(a.Npad, a.kst);
-    const int usable = sp.num_sms > 2 * kWinReserveSms ? sp.num_sms - kWinReserveSms : sp.num_sms;
+    const size_t smem = tile_smem_bytes(a.Npad, a.kst, a.T < a.nacc);
     const int grid = a.units < usable ? a.units : usable;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -914,49 +1031,42 @@ cudaError_t launch_window_tiles(const ScorePlan& sp, const Geometry& g, const La
     cfg.attrs = attr;
     cfg.numAttrs = after_own_launch ? 1 : 0;
     switch (g.g) {
-        case 1: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<1>, sp.kmap, sp.qmap, a);
-        case 2: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<2>, sp.kmap, sp.qmap, a);
-        case 4: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<4>, sp.kmap, sp.qmap, a);
-        case 7: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<7>, sp.kmap, sp.qmap, a);
-        default: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<8>, sp.kmap, sp.qmap, a);
+        case 1: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<1>, a);
+        case 2: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<2>, a);
+        case 4: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<4>, a);
+        case 7: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<7>, a);
+        case 8: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<8>, a);
+        default: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<0>, a);
     }
 }
 
 }  // namespace
 
-int window_grid_size(const ScorePlan& sp, const Geometry& g, bool lse) {
+bool tile_variant_fits(const Geometry& g) { return g.w % 8 == 0 && (g.O == 8 || g.O == kTileOMax); }
+
+int window_grid_size(const ScorePlan& sp, const Geometry& g, int nl) {
     if (g.win_tiles == 0) return 0;
-    const int usable = sp.num_sms > 2 * kWinReserveSms ? sp.num_sms - kWinReserveSms : sp.num_sms;
-    if (tile_variant_fits(g) && tile_units_of(g, g.cu_host, tile_unit_tiles(g, lse)) >= usable) return usable;
-    return units_of(g) < usable ? units_of(g) : usable;
+    const int usable = usable_sms(sp.num_sms);
+    const int units = g.jm ? tile_units_of(g, g.cu_host, tile_unit_tiles(g, nl, usable)) : units_of(g);
+    return units * nl < usable ? units * nl : usable;
 }
 
-cudaError_t launch_window(const ScorePlan& sp, const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl,
+cudaError_t launch_window(const ScorePlan& sp, const Geometry& g, const Group& gr, const Scratch& sc, int* claim,
                           cudaStream_t st, bool after_own_launch) {
     if (g.win_tiles == 0) return cudaSuccess;
-    // The tile-owning variant where it applies and its units still give every
-    // usable SM one (it has T times fewer units than the per-tile kernel, whose
-    // CTAs finish sooner when there are few tiles).
-    if (tile_variant_fits(g)) {
-        const int T = tile_unit_tiles(g, io.lse != nullptr);
-        const int usable = sp.num_sms > 2 * kWinReserveSms ? sp.num_sms - kWinReserveSms : sp.num_sms;
-        if (tile_units_of(g, g.cu_host, T) >= usable) return launch_window_tiles(sp, g, io, sc, sl, st, after_own_launch);
-    }
+    if (g.jm) return launch_window_tiles(sp, g, gr, sc, claim, st, after_own_launch);
     WinArgs a{};
-    a.G = g;
-    a.sc = sc;
-    a.sl = sl;
-    a.cu = io.cu;
+    set_layers(&a, sp, g, gr, sc);
     a.Npad = npad_of(g.R);
     a.kst = kst_for(a.Npad, g.O);
     a.nacc = a.Npad <= 128 ? 4 : 2;   // nacc * Npad <= 512 TMEM columns
-    a.units = units_of(g);
+    a.upl = units_of(g);
+    a.units = gr.nl * a.upl;
     a.fault = test_fault() == 1 ? 1 : 0;
     a.tmem_cols = 512;   // one CTA per SM; a 32-column load past the last group's columns stays inside
     const size_t smem = win_smem_bytes(a.Npad, g.O, a.kst);
-    // Persistent: at most one CTA per SM, leaving a few SMs to the selection
-    // chain and the other layers' kernels.
-    const int usable = sp.num_sms > 2 * kWinReserveSms ? sp.num_sms - kWinReserveSms : sp.num_sms;
+    // Persistent: at most one CTA per SM.
+    const int usable = usable_sms(sp.num_sms);
     const int grid = a.units < usable ? a.units : usable;
     // after_own_launch: the previous kernel on the stream is this layer's
     // row-statistics launch and no event wait stands between them; the launch is
@@ -973,12 +1083,12 @@ cudaError_t launch_window(const ScorePlan& sp, const Geometry& g, const LayerIO&
     cfg.attrs = attr;
     cfg.numAttrs = after_own_launch ? 1 : 0;
     switch (g.g) {
-        case 1: return cudaLaunchKernelEx(&cfg, window_kernel<1>, sp.kmap, sp.qmap, a);
-        case 2: return cudaLaunchKernelEx(&cfg, window_kernel<2>, sp.kmap, sp.qmap, a);
-        case 4: return cudaLaunchKernelEx(&cfg, window_kernel<4>, sp.kmap, sp.qmap, a);
-        case 7: return cudaLaunchKernelEx(&cfg, window_kernel<7>, sp.kmap, sp.qmap, a);
-        case 8: return cudaLaunchKernelEx(&cfg, window_kernel<8>, sp.kmap, sp.qmap, a);
-        default: return cudaLaunchKernelEx(&cfg, window_kernel<0>, sp.kmap, sp.qmap, a);
+        case 1: return cudaLaunchKernelEx(&cfg, window_kernel<1>, a);
+        case 2: return cudaLaunchKernelEx(&cfg, window_kernel<2>, a);
+        case 4: return cudaLaunchKernelEx(&cfg, window_kernel<4>, a);
+        case 7: return cudaLaunchKernelEx(&cfg, window_kernel<7>, a);
+        case 8: return cudaLaunchKernelEx(&cfg, window_kernel<8>, a);
+        default: return cudaLaunchKernelEx(&cfg, window_kernel<0>, a);
     }
 }
 
