@@ -20,6 +20,21 @@ namespace {
 
 namespace cg = cooperative_groups;
 
+// Whether a row's importances are staged in shared memory beside its scores.
+__host__ __device__ constexpr bool chain_stages_i(int nt, int kpt) { return nt * kpt <= 16384; }
+__host__ __device__ constexpr int chain_smem_bytes(int nt, int kpt) {
+    return nt * kpt * (int)sizeof(float) * (chain_stages_i(nt, kpt) ? 2 : 1);
+}
+
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+}
+
 struct ChainArgs {
     Geometry G;
     const int* cu;
@@ -200,10 +215,20 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
     __shared__ HistSelectShared sm;
     __shared__ __align__(16) uint32_t bits[2][HS::kWords];   // this head's kept positions, by layer parity
     __shared__ __align__(16) uint32_t uni[HS::kWords];       // the last layer's union
+    __shared__ uint32_t spres[HS::kWords];                   // the layer's preserved bits
     __shared__ JointShared js[1];
+    // [KPT / 4][NT]: each thread's scores of the layer; then its importances, where
+    // both fit.
+    extern __shared__ __align__(16) float4 sP[];
+    constexpr bool kStageI = chain_stages_i(NT, KPT);
+    float4* const sI = sP + NT * KPT / 4;
     cg::cluster_group cluster = cg::this_cluster();
     const int h = (int)cluster.block_rank(), s = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    HS::clear(sm);
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    // The scores and the state come from the kernels before this one.
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int Hkv = A.G.Hkv, words = A.G.words, budget = A.G.budget;
     const int L = __ldg(&A.cu[s + 1]) - __ldg(&A.cu[s]);
     const int Lc = L - A.G.wk;
@@ -227,29 +252,43 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         const int t = HS::position(4 * g);
         n4[g] = t < L ? __ldcg(reinterpret_cast<const uint32_t*>(nst + t)) : 0u;
     }
-    HS::clear(sm);
-    // Sixteen values of a thread at a time: its scores, and the preserved bits.
-    float4 p[4], im[4];
-    uint32_t pw[4];
-    auto load = [&](int l, int part) {
+    uint32_t top = 0u;   // bit l: the head takes O' in layer l
+    for (int l = 0; l < A.nl; ++l) top |= (__ldg(&A.sl[l].htop[row]) != 0 ? 1u : 0u) << l;
+    // A layer's scores P, importance I and preserved bits come by asynchronous copies
+    // into shared memory, issued once the layer before has its keys: beside the score
+    // and window grids an L2 round trip takes 2 us and more, a third of the layer.
+    // (Rows of more than 16384 positions leave no room for I: it comes into registers
+    // under the cluster barrier.  A thread reads only the scores that it copied.)
+    auto stage = [&](int l) {
         const Slot& sl = A.sl[l];
-        const float* P = (__ldg(&sl.htop[row]) ? sl.POe : sl.PO) + row * A.G.ML;
-        const float* I = sl.I + (size_t)s * A.G.ML;
-        const uint32_t* pres = sl.pres + row * words;
+        const float* P = (((top >> l) & 1u) ? sl.POe : sl.PO) + row * A.G.ML;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const int t = HS::position(16 * part + 4 * g);
+        for (int g = 0; g < KPT / 4; ++g) {
+            const int t = HS::position(4 * g);
             if (t < Lc) {
-                p[g] = __ldg(reinterpret_cast<const float4*>(P + t));
-                im[g] = __ldg(reinterpret_cast<const float4*>(I + t));
-                pw[g] = __ldg(&pres[t >> 5]) >> (t & 31);
+                copy_async<16>(&sP[g * NT + tid], P + t);
+                if constexpr (kStageI) copy_async<16>(&sI[g * NT + tid], A.sl[l].I + (size_t)s * A.G.ML + t);
             }
         }
+        if (tid < HS::kWords && tid < wordsL) copy_async<4>(&spres[tid], sl.pres + row * words + tid);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    // With 64 registers a thread (NT = 1024) there is no room for the next layer's
-    // scores while this one's are ranked.
-    constexpr bool kAhead = NT < 1024;
-    if (kAhead && select) load(0, 0);
+    float4 im[kStageI ? 1 : KPT / 4];
+    auto load_i = [&](int l) {
+        if constexpr (kStageI) return;
+        const float* I = A.sl[l].I + (size_t)s * A.G.ML;
+#pragma unroll
+        for (int g = 0; g < KPT / 4; ++g) {
+            const int t = HS::position(4 * g);
+            if constexpr (!kStageI)
+                im[g] = t < Lc ? __ldg(reinterpret_cast<const float4*>(I + t)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    if (select) {
+        stage(0);
+        load_i(0);
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
     for (int l = 0; l < A.nl; ++l) {
         uint32_t* b = bits[l & 1];
@@ -260,33 +299,39 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
             float* Pp = A.l0 + l + 1 == A.ncall ? A.sl[l].Pprime + row * A.G.ML : nullptr;
             uint32_t key[KPT];
 #pragma unroll
-            for (int part = 0; part < KPT / 16; ++part) {
-                if (!kAhead || part > 0) load(l, part);
+            for (int g = 0; g < KPT / 4; ++g) {
+                const int t0 = HS::position(4 * g);
+                const float4 p = t0 < Lc ? sP[g * NT + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const uint32_t pres = t0 < Lc ? (spres[t0 >> 5] >> (t0 & 31)) & 15u : 0u;
+                // Positions that do not compete: preserved ones, and from Lc on.
+                const int lim = Lc - t0;
+                const uint32_t out4 = lim >= 4 ? pres : lim > 0 ? pres | (15u << lim) : 15u;
+                keep |= pres << (4 * g);
+                if (lim < 4 && t0 < L)   // the kept tail [Lc, L)
+                    keep |= ((15u << max(lim, 0)) & (t0 + 4 <= L ? 15u : (1u << (L - t0)) - 1u) & 15u) << (4 * g);
+                const float p4[4] = {p.x, p.y, p.z, p.w};
+                float4 iv;
+                if constexpr (kStageI)
+                    iv = t0 < Lc ? sI[g * NT + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+                else
+                    iv = im[g];
+                const float i4[4] = {iv.x, iv.y, iv.z, iv.w};
+                float out[4];
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const int i0 = 16 * part + 4 * g, t0 = HS::position(i0);
-                    const float p4[4] = {p[g].x, p[g].y, p[g].z, p[g].w};
-                    const float i4[4] = {im[g].x, im[g].y, im[g].z, im[g].w};
-                    float out[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int t = t0 + e;
-                        key[i0 + e] = 0u;
-                        if (t < Lc) {
-                            // coverage = n_t / (l + 1), by the rounded reciprocal
-                            const float coverage = (float)((n4[i0 / 4] >> (8 * e)) & 255u) * inv_l1;
-                            const float pp = p4[e] + A.G.lambda * (i4[e] * (1.f - coverage));
-                            out[e] = pp;
-                            const uint32_t kept = (pw[g] >> e) & 1u;
-                            keep |= kept << (i0 + e);
-                            if (!kept) key[i0 + e] = float_order_key(pp);
-                        } else {
-                            out[e] = 0.f;
-                            keep |= (t < L ? 1u : 0u) << (i0 + e);
-                        }
-                    }
-                    if (Pp && t0 < Lc) *reinterpret_cast<float4*>(Pp + t0) = make_float4(out[0], out[1], out[2], out[3]);
+                for (int e = 0; e < 4; ++e) {
+                    // coverage = n_t / (l + 1), by the rounded reciprocal; the byte n_t in
+                    // the mantissa of 2^23 + n_t gives its float without a conversion.
+                    const float n = __uint_as_float(__byte_perm(n4[g], 0x4b000000u, 0x7650u + e)) - 8388608.f;
+                    const float coverage = n * inv_l1;
+                    const float pp = p4[e] + A.G.lambda * (i4[e] * (1.f - coverage));
+                    out[e] = pp;
+                    key[4 * g + e] = (out4 >> e) & 1u ? 0u : float_order_key(pp);
                 }
+                if (Pp && t0 < Lc) *reinterpret_cast<float4*>(Pp + t0) = make_float4(out[0], out[1], out[2], out[3]);
+            }
+            if (l + 1 < A.nl) {
+                __syncthreads();   // the preserved bits have been read
+                stage(l + 1);
             }
             if (A.G.f0 > 0) {
                 HS hs{sm, A.G.f0};
@@ -321,8 +366,9 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         // The heads' kept bits: written above, read below by every CTA of the
         // cluster.  A buffer is written again two layers on, after the next
         // barrier, which every reader passes first.
+        asm volatile("cp.async.wait_all;\n" ::: "memory");   // the next layer's preserved bits, read by other threads
         auto token = cluster.barrier_arrive();
-        if (kAhead && select && l + 1 < A.nl) load(l + 1, 0);
+        if (select && l + 1 < A.nl) load_i(l + 1);
         cluster.barrier_wait(std::move(token));
         // A warp's union words: lane (4 hh + c) takes four words of head hh.
 #pragma unroll
@@ -380,37 +426,58 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
 }
 
 template <int NT, int KPT, bool ADA>
-cudaError_t launch_one(const ChainArgs& a, cudaStream_t st, int priority) {
+cudaError_t launch_one(const ChainArgs& a, cudaStream_t st, int priority, bool programmatic) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.G.Hkv, a.G.batch);
     cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = chain_smem_bytes(NT, KPT);
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = a.G.Hkv;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributePriority;
     attr[1].val.priority = priority;
+    attr[2].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[2].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = programmatic ? 3 : 2;
     return cudaLaunchKernelEx(&cfg, chain_kernel<NT, KPT, ADA>, a);
 }
 
 template <bool ADA>
-cudaError_t launch_for(const Geometry& g, const ChainArgs& a, cudaStream_t st, int priority) {
-    if (g.max_len <= 256 * 16) return launch_one<256, 16, ADA>(a, st, priority);
-    if (g.max_len <= 512 * 16) return launch_one<512, 16, ADA>(a, st, priority);
-    if (g.max_len <= 512 * 32) return launch_one<512, 32, ADA>(a, st, priority);
-    return launch_one<1024, 32, ADA>(a, st, priority);
+cudaError_t launch_for(const Geometry& g, const ChainArgs& a, cudaStream_t st, int priority, bool pdl) {
+    if (g.max_len <= 256 * 16) return launch_one<256, 16, ADA>(a, st, priority, pdl);
+    if (g.max_len <= 512 * 16) return launch_one<512, 16, ADA>(a, st, priority, pdl);
+    if (g.max_len <= 512 * 32) return launch_one<512, 32, ADA>(a, st, priority, pdl);
+    return launch_one<1024, 32, ADA>(a, st, priority, pdl);
+}
+
+template <int NT, int KPT>
+cudaError_t configure_one() {
+    for (auto fn : {chain_kernel<NT, KPT, false>, chain_kernel<NT, KPT, true>}) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, chain_smem_bytes(NT, KPT));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
 
+cudaError_t configure_chain() {
+    cudaError_t e = configure_one<256, 16>();
+    if (e == cudaSuccess) e = configure_one<512, 16>();
+    if (e == cudaSuccess) e = configure_one<512, 32>();
+    if (e == cudaSuccess) e = configure_one<1024, 32>();
+    return e;
+}
+
 bool chain_fits(const Geometry& g) { return g.Hkv <= kMaxClusterHeads && g.max_len <= kMaxRegisterRow; }
 
 cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, int l0, int ncall, cudaStream_t st,
-                         int priority) {
+                         int priority, bool programmatic) {
     ChainArgs a{};
     a.G = g;
     a.cu = gr.io[0].cu;
@@ -421,7 +488,7 @@ cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, 
     a.nl = gr.nl;
     a.ncall = ncall;
     for (int l = 0; l < gr.nl; ++l) a.sl[l] = gr.sl[l];
-    return g.ada ? launch_for<true>(g, a, st, priority) : launch_for<false>(g, a, st, priority);
+    return g.ada ? launch_for<true>(g, a, st, priority, programmatic) : launch_for<false>(g, a, st, priority, programmatic);
 }
 
 }  // namespace kvec

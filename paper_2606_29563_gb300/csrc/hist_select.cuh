@@ -124,23 +124,27 @@ struct HistSelect {
                 }
             }
             __syncthreads();
-            const uint32_t bin = (uint32_t)sm.bin;
             kk -= sm.above;
             m = sm.count;
+            // The bucket holds the keys [first, first + 2^shift).
+            const uint32_t first = lo + ((uint32_t)sm.bin << shift), width = 1u << shift;
             match = 0u;
+            uint32_t over = 0u;
 #pragma unroll
             for (int i = 0; i < KPT; ++i) {
-                const uint32_t on = (active >> i) & 1u, d = (key[i] - lo) >> shift;
-                sure |= (on & (d > bin ? 1u : 0u)) << i;
-                match |= (on & (d == bin ? 1u : 0u)) << i;
+                const uint32_t d = key[i] - first;   // wraps below the bucket
+                if (d < width) match |= 1u << i;
+                if (key[i] >= first) over |= 1u << i;
             }
+            match &= active;
+            sure |= over & active & ~match;
             if (m == kk) {   // the bucket is taken whole
                 sure |= match;
                 match = 0u;
             }
             if (m == kk || m <= kSelList || shift == 0) return sure;
             active = match;
-            lo += bin << shift;
+            lo = first;
             shift = max(shift - kSelBits, 0);
         }
     }

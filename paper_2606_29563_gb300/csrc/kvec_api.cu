@@ -287,7 +287,11 @@ Geometry make_geometry(const kvec_handle* h, int batch, int budget, int tiles, i
     return G;
 }
 
-// One layer, every kernel on one stream with one slot (used without a handle).
+// One layer, every kernel on the caller's stream: with nothing to overlap it with,
+// the streams of the pipeline only add event waits between dependent kernels.  Each
+// kernel is a programmatic dependent of the one before it, so that its launch and
+// set-up run beside that one's end; all of them wait for their predecessor before
+// they read what it wrote, so that each has seen everything before it.
 kvec_status run_layer_sequential(kvec_handle* h, const Geometry& G, const LayerIO& io, cudaStream_t st) {
     ScorePlan plan;
     Group gr{};
@@ -297,24 +301,33 @@ kvec_status run_layer_sequential(kvec_handle* h, const Geometry& G, const LayerI
     gr.segpart[0] = h->segpart[0];
     cudaError_t se = plan_score(G, gr, h->num_sms, &plan);
     if (se != cudaSuccess) return cuda_fail(se, "score kernel tensor maps");
-    se = launch_score(plan, G, gr, h->sc, h->claims, st, false);
-    if (se != cudaSuccess) return cuda_fail(se, "score kernel launch");
-    se = launch_rowstat(plan, G, gr, h->claims, st, /*programmatic=*/true, /*after_score=*/true);
-    if (se != cudaSuccess) return cuda_fail(se, "row statistics launch");
-    se = launch_window(plan, G, gr, h->sc, h->claims, st, false);
-    if (se != cudaSuccess) return cuda_fail(se, "window kernel launch");
-    se = launch_heads(G, gr, h->sc, h->claims, st, h->prio_hi);
-    if (se != cudaSuccess) return cuda_fail(se, "heads kernel launch");
-    if (chain_fits(G)) {
-        se = launch_chain(G, gr, h->sc, 0, 1, st, h->prio_hi);
-        if (se != cudaSuccess) return cuda_fail(se, "chain kernel launch");
+    if (io.lse) {
+        se = launch_rowstat_lse(G, gr, st, /*programmatic=*/false);
     } else {
-        se = launch_select(G, io, h->sc, h->slots[0], nullptr, st, h->prio_hi, 0, 1, /*programmatic=*/false);
-        if (se != cudaSuccess) return cuda_fail(se, "select kernel launch");
+        timed_launch(h, 0, st, [&] { se = launch_score(plan, G, gr, h->sc, h->claims, st, false); });
+        if (se != cudaSuccess) return cuda_fail(se, "score kernel launch");
+        se = launch_rowstat(plan, G, gr, h->claims, st, /*programmatic=*/!h->profiling, /*after_score=*/true);
     }
-    se = launch_gather(G, gr, st);
+    if (se != cudaSuccess) return cuda_fail(se, "row statistics launch");
+    timed_launch(h, 1, st, [&] { se = launch_window(plan, G, gr, h->sc, h->claims, st, !h->profiling); });
+    if (se != cudaSuccess) return cuda_fail(se, "window kernel launch");
+    timed_launch(h, 2, st, [&] { se = launch_heads(G, gr, h->sc, h->claims, st, h->prio_hi, G.win_tiles > 0 && !h->profiling); });
+    if (se != cudaSuccess) return cuda_fail(se, "heads kernel launch");
+    const bool chain = chain_fits(G);
+    timed_launch(h, 3, st, [&] {
+        if (chain)
+            se = launch_chain(G, gr, h->sc, 0, 1, st, h->prio_hi, !h->profiling);
+        else
+            se = launch_select(G, io, h->sc, h->slots[0], nullptr, st, h->prio_hi, 0, 1, /*programmatic=*/false);
+    });
+    if (se != cudaSuccess) return cuda_fail(se, "selection kernel launch");
+    if (!chain && G.ada) {
+        se = launch_ada(G, io, h->sc, h->slots[0], st, h->prio_hi, 1);
+        if (se != cudaSuccess) return cuda_fail(se, "adaptive fill launch");
+    }
+    timed_launch(h, 4, st, [&] { se = launch_gather(G, gr, st, h->prio_hi, chain && !h->profiling); });
     if (se != cudaSuccess) return cuda_fail(se, "gather kernel launch");
-    if (!chain_fits(G)) {
+    if (!chain) {
         se = launch_finalize(G, io, h->sc, h->slots[0], st, h->prio_hi, 1);
         if (se != cudaSuccess) return cuda_fail(se, "finalize kernel launch");
     }
@@ -465,13 +478,13 @@ kvec_status launch_pipeline(kvec_handle* h, const Geometry& G, const LayerIO* io
         // (Rows beyond kMaxRegisterRow rank in key rows that every layer shares: one stream.)
         cudaStream_t s_h = (k & 1) && G.max_len <= kMaxRegisterRow ? h->s_heads2 : h->s_heads;
         KV_CHECK(cudaStreamWaitEvent(s_h, h->ev_win[k], 0));
-        timed_launch(h, 2, s_h, [&] { se = launch_heads(G, gr, h->sc, h->claims + 2 * k, s_h, h->prio_hi); });
+        timed_launch(h, 2, s_h, [&] { se = launch_heads(G, gr, h->sc, h->claims + 2 * k, s_h, h->prio_hi, false); });
         if (se != cudaSuccess) return cuda_fail(se, "heads kernel launch");
         KV_CHECK(cudaEventRecord(h->ev_heads[k], s_h));
         KV_CHECK(cudaStreamWaitEvent(h->s_chain, h->ev_heads[k], 0));
         if (last >= h->nsel) KV_CHECK(cudaStreamWaitEvent(h->s_chain, h->ev_gather[group_of[last - h->nsel]], 0));
         if (chain) {
-            timed_launch(h, 3, h->s_chain, [&] { se = launch_chain(G, gr, h->sc, l0, n, h->s_chain, h->prio_hi); });
+            timed_launch(h, 3, h->s_chain, [&] { se = launch_chain(G, gr, h->sc, l0, n, h->s_chain, h->prio_hi, false); });
             if (se != cudaSuccess) return cuda_fail(se, "chain kernel launch");
         }
         for (int l = l0; !chain && l < l0 + gr.nl; ++l) {
@@ -502,7 +515,7 @@ kvec_status launch_pipeline(kvec_handle* h, const Geometry& G, const LayerIO* io
         }
         KV_CHECK(cudaEventRecord(h->ev_sel[k], h->s_chain));
         KV_CHECK(cudaStreamWaitEvent(h->s_gather, h->ev_sel[k], 0));
-        timed_launch(h, 4, h->s_gather, [&] { se = launch_gather(G, gr, h->s_gather); });
+        timed_launch(h, 4, h->s_gather, [&] { se = launch_gather(G, gr, h->s_gather, h->prio_lo, false); });
         if (se != cudaSuccess) return cuda_fail(se, "gather kernel launch");
         KV_CHECK(cudaEventRecord(h->ev_gather[k], h->s_gather));
     }
@@ -665,6 +678,7 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
     if (e == cudaSuccess) e = configure_score(G);
     if (e == cudaSuccess) e = configure_window(G);
     if (e == cudaSuccess) e = configure_select();
+    if (e == cudaSuccess) e = configure_chain();
     if (e == cudaSuccess) e = configure_decode();
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&h->prio_lo, &h->prio_hi);
     for (cudaStream_t* st : {&h->s_score, &h->s_gather, &h->s_cap})
@@ -828,7 +842,13 @@ kvec_status select_layers_impl(kvec_handle* h, int num_layers, int batch, const 
         if (h->seen_keys.size() == kGraphCache) h->seen_keys.erase(h->seen_keys.begin());
         h->seen_keys.push_back(key);
     }
-    s = launch_pipeline(h, G, ios.data(), num_layers, st);
+    if (num_layers == 1) {
+        h->slots[0].sel = h->sel[0];
+        s = run_layer_sequential(h, G, ios[0], st);
+        h->last_slot = 0;
+    } else {
+        s = launch_pipeline(h, G, ios.data(), num_layers, st);
+    }
     if (s != KVEC_OK) return s;
     h->last_batch = batch;
     return KVEC_OK;
@@ -905,6 +925,7 @@ kvec_status noalloc_setup(int dev, void** base, const Geometry& G) {
         e = configure_score(G);
         if (e == cudaSuccess) e = configure_window(G);
         if (e == cudaSuccess) e = configure_select();
+        if (e == cudaSuccess) e = configure_chain();
         if (e != cudaSuccess) return cuda_fail(e, "kernel attributes");
         // The error word (the array's first bytes) starts at zero; calls leave it
         // set until kvec_noalloc_sync_status reads and clears it.

@@ -113,8 +113,8 @@ struct DecodeIO {
 
 __device__ __forceinline__ uint32_t float_order_key(float f) {
     // Monotone map of IEEE floats onto unsigned integers (larger float -> larger key).
-    uint32_t u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    const uint32_t u = __float_as_uint(f);
+    return u ^ ((uint32_t)((int)u >> 31) | 0x80000000u);   // ~u for negative floats, else the sign bit set
 }
 
 // Finds (sequence, local index) of global item `gi` where sequence s owns
@@ -197,8 +197,10 @@ cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t 
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// programmatic (here and below): a programmatic dependent of the stream's previous
+// kernel, which it waits for before it reads anything.
 cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, int* claim, cudaStream_t st,
-                         int priority);
+                         int priority, bool programmatic);
 // lcall: the layer's index within a call of ncall layers (0 for the first);
 // prev: the previous layer's slot (null for lcall = 0), whose kept-position
 // bits give that layer's union.  The coverage counts alternate between the
@@ -215,7 +217,7 @@ cudaError_t launch_select(const Geometry& g, const LayerIO& io, const Scratch& s
 // launch, state and header included; needs chain_fits(g).
 bool chain_fits(const Geometry& g);
 cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, int l0, int ncall, cudaStream_t st,
-                         int priority);
+                         int priority, bool programmatic);
 cudaError_t launch_finalize(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& last, cudaStream_t st,
                             int priority, int ncall);
 // Adaptive fill: the layer's extra fill slots over every head of a sequence,
@@ -225,7 +227,7 @@ cudaError_t launch_ada(const Geometry& g, const LayerIO& io, const Scratch& sc, 
                        int priority, int ncall);
 cudaError_t launch_decode(const DecodeIO& io, int num_sms, cudaStream_t st);
 // out_idx from the slot's kept-position bits, then the K/V rows.
-cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st);
+cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st, int priority, bool programmatic);
 
 // Fault injected by kvec_set_test_fault (0: none), read when a kernel is launched.
 int test_fault();
@@ -237,6 +239,7 @@ size_t window_smem_bytes(const Geometry& g);
 cudaError_t configure_score(const Geometry& g);
 cudaError_t configure_window(const Geometry& g);
 cudaError_t configure_select();
+cudaError_t configure_chain();
 cudaError_t configure_decode();
 
 }  // namespace kvec

@@ -10,9 +10,14 @@
 // delaying the launch:
 //   warp 0      TMA producer: the KV head's g*w query rows (once per (s,h) of a
 //               chunk, two buffers) and a ring of 128-token K tiles, both
-//               128-byte swizzled;
-//   warp 1      one thread issues tcgen05.mma (M = 128 query rows per M-block,
-//               N = 128 tokens, K = 128 = d) into TMEM accumulators;
+//               128-byte swizzled; warp 19 loads the K tiles of the second issuer;
+//   warps 1, 18 issue tcgen05.mma (M = 128 query rows per M-block, N = 128 tokens,
+//               K = 128 = d) into TMEM accumulators, the even ones and the odd ones:
+//               an issuer's waits and commits take as long as the products, which
+//               run meanwhile for the other one's item.  Each has its own part of
+//               the K ring (a ring with two readers that skip each other's stages
+//               would let one of them take a phase for another two further on);
+//               with fewer than four stages there is one issuer;
 //   warps 2..17 epilogue: groups of warps, one per TMEM accumulator, each
 //               taking every NB-th item of a chunk; one thread per query row and
 //               all 128 columns of the item: tcgen05.ld of its logits, their sum
@@ -93,6 +98,12 @@ constexpr int kChunkLarge = 12;          // (sequence, head, tile) items per cla
 constexpr int kChunkSmall = 8;           // items per claim otherwise
 constexpr int kChunkSlots = 4;           // claimed chunks in flight inside a CTA
 
+// MMA issuers of a ring of kst K stages, and the first stage and number of stages
+// of an issuer's part.
+__host__ __device__ constexpr int issuers(int kst) { return kst >= 4 ? 2 : 1; }
+__device__ __forceinline__ int ring_first(int kst, int c) { return c == 0 ? 0 : (kst + 1) / 2; }
+__device__ __forceinline__ int ring_end(int kst, int c) { return c == 0 && issuers(kst) == 2 ? (kst + 1) / 2 : kst; }
+
 struct ScoreArgs {
     CUtensorMap kmap[kMaxGroup], qmap[kMaxGroup];
     Geometry G;
@@ -108,7 +119,9 @@ struct ScoreArgs {
 
 constexpr int kEpiWarps = 16;
 constexpr int kEpiThreads = 32 * kEpiWarps;
-constexpr int kScoreThreads = 64 + kEpiThreads;
+constexpr int kScoreThreads = 64 + kEpiThreads + 64;
+constexpr int kMmaWarp1 = 2 + kEpiWarps;   // the second issuer
+constexpr int kTmaWarp1 = 3 + kEpiWarps;   // its producer
 
 struct __align__(8) Barriers {
     uint64_t k_full[kKStages], k_empty[kKStages];
@@ -153,6 +166,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
     const int per_layer = (W + chunk_items - 1) / chunk_items;   // chunks of a layer
     const int nchunks = A.nl * per_layer;
     int* const claim = A.claim;
+    const int ni = issuers(kst);   // MMA issuers
     const int R = G.R;
     const uint32_t qhalf = (uint32_t)R * 128u;            // bytes of a query buffer's half (64 columns)
     uint8_t* sQ = smem;                                   // 2 buffers x 2 halves x R rows x 128 B
@@ -176,7 +190,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(&bars->q_full[b], 1);
-            ptx::mbar_init(&bars->q_empty[b], 1);
+            ptx::mbar_init(&bars->q_empty[b], ni);
         }
         for (int b = 0; b < 4; ++b) {
             ptx::mbar_init(&bars->acc_full[b], 1);
@@ -184,9 +198,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
         }
         for (int c = 0; c < kChunkSlots; ++c) {
             ptx::mbar_init(&bars->c_full[c], 1);
-            ptx::mbar_init(&bars->c_empty[c], 1 + kEpiWarps);   // the MMA issuer and every epilogue warp
+            ptx::mbar_init(&bars->c_empty[c], 2 * ni - 1 + kEpiWarps);   // issuers, second producer, epilogue warps
         }
-        ptx::mbar_init(&bars->mma_done, 1);
+        ptx::mbar_init(&bars->mma_done, ni);
         bars->abort_flag = 0;
         ptx::fence_barrier_init();
     }
@@ -233,37 +247,49 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
             p.row0 = ptx::warp_uniform(p.row0);
         }
     };
-    if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer
+    if (warp == 0 || warp == kTmaWarp1) {
+        // ------------------------------------------------------------ TMA producers
+        const int me = warp == kTmaWarp1 ? 1 : 0;
         const uint64_t policy = ptx::policy_evict_normal();   // the window kernel reads K again
-        int qloads = 0, issued = 0, st = 0, di = 0;
-        uint32_t kphase = 0u;   // bit st: the stage has been filled an odd number of times
+        int qloads = 0, st = ring_first(kst, me), di = 0;
+        uint32_t kphase = 0u, filled = 0u;   // bit st: filled an odd number of times; filled at all
         int next = 0;
-        if (lane == 0) next = atomicAdd(claim, 1);
+        if (me == 0 && lane == 0) next = atomicAdd(claim, 1);
         bool stop = false;
-        while (!stop) {
-            // Hand the claimed chunk to the MMA issuer and the epilogue, and claim
-            // the next one: its number arrives while this one is loaded.
+        while (!stop && me < ni) {
             const int ds = di % kChunkSlots, nd = di / kChunkSlots;
-            if (nd > 0 && !ptx::warp_wait(&bars->c_empty[ds], (nd - 1) & 1, &bars->abort_flag)) {
-                if (lane == 0) raise_abort(bars, err);
-                break;
-            }
-            const int c = ptx::warp_uniform(bars->abort_flag ? nchunks : next);
-            if (lane == 0) {
-                bars->chunk[ds] = c < nchunks ? c : -1;
-                ptx::mbar_arrive(&bars->c_full[ds]);
+            int c;
+            if (me == 0) {
+                // Hand the claimed chunk to the other roles, and claim the next one: its
+                // number arrives while this one is loaded.
+                if (nd > 0 && !ptx::warp_wait(&bars->c_empty[ds], (nd - 1) & 1, &bars->abort_flag)) {
+                    stop = true;
+                    break;
+                }
+                c = ptx::warp_uniform(bars->abort_flag ? nchunks : next);
+                if (lane == 0) {
+                    bars->chunk[ds] = c < nchunks ? c : -1;
+                    ptx::mbar_arrive(&bars->c_full[ds]);
+                }
+                if (c >= nchunks) break;
+                if (lane == 0) next = atomicAdd(claim, 1);
+            } else {
+                if (!ptx::warp_wait(&bars->c_full[ds], nd & 1, &bars->abort_flag)) {
+                    stop = true;
+                    break;
+                }
+                c = ptx::warp_uniform(bars->chunk[ds]);
+                if (lane == 0) ptx::mbar_arrive(&bars->c_empty[ds]);
+                if (c < 0) break;
             }
             ++di;
-            if (c >= nchunks) break;
-            if (lane == 0) next = atomicAdd(claim, 1);
             const int lay = c / per_layer, i0 = (c - lay * per_layer) * chunk_items, i1 = min(W, i0 + chunk_items);
             const CUtensorMap* kmap = &A.kmap[lay];
             const CUtensorMap* qmap = &A.qmap[lay];
             int prev_sh = -1;   // the query rows are loaded again at every chunk's start
             uniform_init(i0);
             for (int i = i0; i < i1; ++i) {
-                if (p.head() != prev_sh) {
+                if (me == 0 && p.head() != prev_sh) {
                     const int qs = qloads & 1, nq = qloads >> 1;
                     if (nq > 0 && !ptx::warp_wait(&bars->q_empty[qs], (nq - 1) & 1, &bars->abort_flag)) {
                         stop = true;
@@ -277,39 +303,43 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
                     ++qloads;
                     prev_sh = p.head();
                 }
-                if (issued >= kst && !ptx::warp_wait(&bars->k_empty[st], ((kphase >> st) & 1u) ^ 1u, &bars->abort_flag)) {
-                    stop = true;
-                    break;
+                if (ni == 1 || ((i - i0) & 1) == me) {   // the item's issuer (NB is even)
+                    if (((filled >> st) & 1u) != 0u &&
+                        !ptx::warp_wait(&bars->k_empty[st], ((kphase >> st) & 1u) ^ 1u, &bars->abort_flag)) {
+                        stop = true;
+                        break;
+                    }
+                    if (ptx::elect_one()) {
+                        uint8_t* dst = sK + st * kKStageBytes;
+                        const int row = p.row0 + p.j * kTileT;
+                        ptx::mbar_arrive_expect_tx(&bars->k_full[st], (uint32_t)kKStageBytes);
+                        ptx::tma_load_3d(dst, kmap, &bars->k_full[st], 0, p.h, row, policy);
+                        ptx::tma_load_3d(dst + kKHalfBytes, kmap, &bars->k_full[st], 64, p.h, row, policy);
+                    }
+                    __syncwarp();
+                    kphase ^= 1u << st;
+                    filled |= 1u << st;
+                    st = st + 1 == ring_end(kst, me) ? ring_first(kst, me) : st + 1;
                 }
-                if (ptx::elect_one()) {
-                    uint8_t* dst = sK + st * kKStageBytes;
-                    const int row = p.row0 + p.j * kTileT;
-                    ptx::mbar_arrive_expect_tx(&bars->k_full[st], (uint32_t)kKStageBytes);
-                    ptx::tma_load_3d(dst, kmap, &bars->k_full[st], 0, p.h, row, policy);
-                    ptx::tma_load_3d(dst + kKHalfBytes, kmap, &bars->k_full[st], 64, p.h, row, policy);
-                }
-                __syncwarp();
-                kphase ^= 1u << st;
-                ++issued;
-                st = st + 1 == kst ? 0 : st + 1;
                 uniform_next();
             }
-            if (stop && lane == 0) raise_abort(bars, err);
         }
-        // Drain: every issued copy lands before the CTA may exit (stage b was
-        // filled ceil((issued - b) / kst) times, query buffer b ceil((qloads - b) / 2)).
-        for (int b = 0; b < kst && b < issued; ++b)
-            ptx::mbar_wait(&bars->k_full[b], ((issued - b + kst - 1) / kst - 1) & 1, 50000000ull);
+        if (stop && lane == 0) raise_abort(bars, err);
+        // Drain: every issued copy lands before the CTA may exit (query buffer b was
+        // filled ceil((qloads - b) / 2) times).
+        for (int b = 0; b < kst; ++b)
+            if ((filled >> b) & 1u) ptx::mbar_wait(&bars->k_full[b], ((kphase >> b) & 1u) ^ 1u, 50000000ull);
         for (int b = 0; b < 2 && b < qloads; ++b)
             ptx::mbar_wait(&bars->q_full[b], ((qloads - b + 1) / 2 - 1) & 1, 50000000ull);
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
+    } else if (warp == 1 || warp == kMmaWarp1) {
+        // ------------------------------------------------------------ MMA issuers
+        const int me = warp == kMmaWarp1 ? 1 : 0;
         const uint32_t idesc = ptx::idesc_bf16_f32(128, kTileT);
         const uint64_t qdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sQ)), kdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sK));
-        int qk = 0, st = 0, di = 0;
+        int qk = 0, st = ring_first(kst, me), di = 0;
         uint32_t kphase = 0u, used = 0u, aphase = 0u;   // per stage / accumulator
         bool stop = false;
-        while (!stop) {
+        while (!stop && me < ni) {
             const int ds = di % kChunkSlots;
             if (!ptx::warp_wait(&bars->c_full[ds], (di / kChunkSlots) & 1, &bars->abort_flag)) {
                 stop = true;
@@ -332,42 +362,47 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
                     ++qk;
                     prev_sh = p.head();
                 }
-                // Giving up on a stage in flight is safe: the producer drains its own loads.
-                if (!ptx::warp_wait(&bars->k_full[st], (kphase >> st) & 1u, &bars->abort_flag) ||
-                    (((used >> buf) & 1u) != 0u &&
-                     !ptx::warp_wait(&bars->acc_empty[buf], ((aphase >> buf) & 1u) ^ 1u, &bars->abort_flag))) {
-                    stop = true;
-                    break;
-                }
-                ptx::tc_fence_after();
                 const bool seg_end = i + 1 >= i1 || p.last_of_head();
-                if (ptx::elect_one()) {
-                    const uint64_t kd = kdesc + (uint32_t)(st * (kKStageBytes >> 4)), qd = qdesc + (uint32_t)qs * (qhalf >> 3);
-#pragma unroll
-                    for (int m = 0; m < MB; ++m) {
-                        const uint32_t d = tmem + (uint32_t)(buf * 128 * MB + m * 128);
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {
-                            const uint32_t half = kk >> 2, kin = kk & 3;
-                            ptx::mma_bf16(d, qd + half * (qhalf >> 4) + m * 1024 + kin * 2,
-                                          kd + half * (kKHalfBytes >> 4) + kin * 2, idesc, kk > 0 ? 1u : 0u);
-                        }
+                if (ni == 1 || (buf & 1) == me) {
+                    // Giving up on a stage in flight is safe: the producer drains its own loads.
+                    if (!ptx::warp_wait(&bars->k_full[st], (kphase >> st) & 1u, &bars->abort_flag) ||
+                        (((used >> buf) & 1u) != 0u &&
+                         !ptx::warp_wait(&bars->acc_empty[buf], ((aphase >> buf) & 1u) ^ 1u, &bars->abort_flag))) {
+                        stop = true;
+                        break;
                     }
-                    ptx::mma_commit(&bars->k_empty[st]);
-                    ptx::mma_commit(&bars->acc_full[buf]);
-                    if (seg_end) ptx::mma_commit(&bars->q_empty[qs]);
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one()) {
+                        const uint64_t kd = kdesc + (uint32_t)(st * (kKStageBytes >> 4)), qd = qdesc + (uint32_t)qs * (qhalf >> 3);
+#pragma unroll
+                        for (int m = 0; m < MB; ++m) {
+                            const uint32_t d = tmem + (uint32_t)(buf * 128 * MB + m * 128);
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk) {
+                                const uint32_t half = kk >> 2, kin = kk & 3;
+                                ptx::mma_bf16(d, qd + half * (qhalf >> 4) + m * 1024 + kin * 2,
+                                              kd + half * (kKHalfBytes >> 4) + kin * 2, idesc, kk > 0 ? 1u : 0u);
+                            }
+                        }
+                        ptx::mma_commit(&bars->k_empty[st]);
+                        ptx::mma_commit(&bars->acc_full[buf]);
+                    }
+                    __syncwarp();
+                    kphase ^= 1u << st;
+                    used |= 1u << buf;
+                    aphase ^= 1u << buf;
+                    st = st + 1 == ring_end(kst, me) ? ring_first(kst, me) : st + 1;
                 }
-                __syncwarp();
-                kphase ^= 1u << st;
-                used |= 1u << buf;
-                aphase ^= 1u << buf;
-                st = st + 1 == kst ? 0 : st + 1;
+                if (seg_end) {   // this issuer's products of the segment, if any, are the last of its query rows
+                    if (ptx::elect_one()) ptx::mma_commit(&bars->q_empty[qs]);
+                    __syncwarp();
+                }
                 buf = buf + 1 == NB ? 0 : buf + 1;
                 uniform_next();
             }
         }
         if (stop && lane == 0) raise_abort(bars, err);
-        if (ptx::elect_one()) ptx::mma_commit(&bars->mma_done);
+        if (me < ni && ptx::elect_one()) ptx::mma_commit(&bars->mma_done);
         __syncwarp();
     } else {
         // ------------------------------------------------------------ epilogue

@@ -858,6 +858,7 @@ __device__ Moments block_moments(Moments v, float3* red) {
 // normalised over the candidates, sum(x ln x)/S - ln S with S = sum(x).
 __global__ void __launch_bounds__(kSelectThreads) heads_pool_kernel(const __grid_constant__ Geometry G,
                                                                      const __grid_constant__ Group A, int* claim) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     // The window grid has completed: its work counter is free for the next launch.
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) claim[1] = 0;
     const LayerIO& io = A.io[blockIdx.z];
@@ -1058,6 +1059,7 @@ __global__ void __launch_bounds__(NT) heads_topk_reg_kernel(const __grid_constan
     const int Lc = L - G.wk;
     const size_t row = (size_t)s * G.Hkv + h;
     HS::clear(sm);
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     // Programmatic dependent of the pooling kernel: its sigmas and pooled rows are
     // read only after that grid has completed.
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -1416,6 +1418,7 @@ __global__ void __launch_bounds__(kSelectThreads) finalize_kernel(Geometry G, La
 __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A) {
     __shared__ int wsum[32];
     __shared__ int spos[16];
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int s = blockIdx.z % G.batch, h = blockIdx.y;
     const LayerIO& io = A.io[blockIdx.z / G.batch];
     const Slot& sl = A.sl[blockIdx.z / G.batch];
@@ -1493,10 +1496,10 @@ cudaError_t configure_select() {
 }
 
 cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, int* claim, cudaStream_t st,
-                         int priority) {
+                         int priority, bool programmatic) {
     const dim3 grid(g.Hkv, g.batch, gr.nl);
     cudaError_t e = launch_prio(heads_pool_kernel, grid, dim3(kSelectThreads), g.NG > 1 ? (size_t)kPoolSmemBytes : 0, st,
-                                priority, false, g, gr, claim);
+                                priority, programmatic, g, gr, claim);
     if (e != cudaSuccess) return e;
     // Sixteen positions a thread while a block can hold the longest row so.
     const auto reg = [&](auto kernel, int threads) {
@@ -1531,9 +1534,9 @@ cudaError_t launch_ada(const Geometry& g, const LayerIO& io, const Scratch& sc, 
                        io, sc, sl, ncall);
 }
 
-cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st) {
-    gather_kernel<<<dim3((g.cap + 15) / 16, g.Hkv, gr.nl * g.batch), 256, 0, st>>>(g, gr);
-    return cudaGetLastError();
+cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st, int priority, bool programmatic) {
+    return launch_prio(gather_kernel, dim3((g.cap + 15) / 16, g.Hkv, gr.nl * g.batch), dim3(256), 0, st, priority,
+                       programmatic, g, gr);
 }
 
 }  // namespace kvec

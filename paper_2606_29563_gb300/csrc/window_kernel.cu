@@ -454,8 +454,14 @@ __global__ void __launch_bounds__(kWinThreads, 1)
 // Each row sum adds its positions in ascending order, as window_kernel does.
 // ---------------------------------------------------------------------------
 constexpr int kTileOMax = 16;     // largest O of the tile-owning variant (register maxima)
+// The paper's windows (w = O' = 32, O = 16): known at compile time, the epilogue's
+// addresses are constants and no position is compared with a window's start, which
+// takes 40 % of its instructions away (it bounds the kernel).
+constexpr int kDefWindow = 32, kDefObs = 16;
 constexpr int kMaxKStages = 6;
 constexpr int kUnitSlots = 4;     // claimed units in flight inside a CTA
+constexpr int kTileThreads = kWinThreads + 64;   // warps 18 and 19: a second MMA issuer and its producer
+constexpr int kTileMmaWarp1 = 18, kTileTmaWarp1 = 19;
 
 struct TileArgs {
     CUtensorMap kmap[kMaxGroup], qmap[kMaxGroup];
@@ -557,8 +563,8 @@ __device__ __forceinline__ void group_sums8(uint32_t taddr, const float* __restr
     }
 }
 
-template <int GG>
-__global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __grid_constant__ TileArgs A) {
+template <int GG, bool DW>
+__global__ void __launch_bounds__(kTileThreads, 1) window_tiles_kernel(const __grid_constant__ TileArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if (threadIdx.x == 0) {
         ptx::prefetch_tensormap(&A.kmap[0]);
@@ -574,6 +580,12 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
     const int* const cu_dev = A.cu;
     const int kst = A.kst, NA = A.nacc, T = A.T, units = A.units, fault = A.fault;
     const int Npad = A.Npad, R = G.R, P = NA / T;
+    // MMA issuers, each with its own part of the K ring (see score_kernel), and the
+    // item's: by accumulator j * P + hh % P, even or odd.
+    const int ni = kst >= 4 ? 2 : 1, half_ring = (kst + 1) / 2;
+    auto ring_first = [&](int c) { return c == 0 ? 0 : half_ring; };
+    auto ring_end = [&](int c) { return c == 0 && ni == 2 ? half_ring : kst; };
+    auto issuer = [&](int j, int hh) { return ni == 1 ? 0 : (P == 1 ? j : hh) & 1; };
     uint8_t* sK = smem;                                      // kst x 32 KB
     uint8_t* sQ = sK + (size_t)kst * kKTileBytes;            // 2 slots x Npad x 256 B
     float* rsm = reinterpret_cast<float*>(sQ + 2 * (size_t)Npad * 256);   // [4][2][256]
@@ -588,7 +600,7 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
         }
         for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(&bars->q_full[i], 1);
-            ptx::mbar_init(&bars->q_empty[i], 1);
+            ptx::mbar_init(&bars->q_empty[i], ni);
         }
         for (int i = 0; i < 4; ++i) {
             ptx::mbar_init(&bars->acc_full[i], 1);
@@ -600,9 +612,9 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
         }
         for (int i = 0; i < kUnitSlots; ++i) {
             ptx::mbar_init(&bars->u_full[i], 1);
-            ptx::mbar_init(&bars->u_empty[i], 1 + 4 * NA);   // the MMA issuer and every epilogue warp
+            ptx::mbar_init(&bars->u_empty[i], 2 * ni - 1 + 4 * NA);   // issuers, second producer, epilogue warps
         }
-        ptx::mbar_init(&bars->mma_done, 1);
+        ptx::mbar_init(&bars->mma_done, ni);
         bars->abort_flag = 0;
         ptx::fence_barrier_init();
     }
@@ -642,46 +654,57 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
 
     // The producer and the MMA issuer run as whole warps and elect a lane for the
     // instructions that one thread issues (see score_kernel).
-    if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer
+    if (warp == 0 || warp == kTileTmaWarp1) {
+        // ------------------------------------------------------------ TMA producers
+        const int me = warp == kTileTmaWarp1 ? 1 : 0;
         const uint64_t policy = ptx::policy_evict_first();   // the K tiles' last use
-        int qi = 0, ki = 0, st = 0;
-        uint32_t kphase = 0u;   // bit st: the stage has been filled an odd number of times
+        int qi = 0, st = ring_first(me);
+        uint32_t kphase = 0u, filled = 0u;   // bit st: filled an odd number of times; filled at all
         bool stop = false;
         int next = 0;
-        if (lane == 0) next = atomicAdd(A.claim, 1);
-        for (int di = 0; !stop; ++di) {
-            const int ds = di % kUnitSlots, nd = di / kUnitSlots;
-            if (nd > 0 && !ptx::warp_wait(&bars->u_empty[ds], (nd - 1) & 1, &bars->abort_flag)) {
-                stop = true;
-                break;
+        if (me == 0 && lane == 0) next = atomicAdd(A.claim, 1);
+        for (int di = 0; !stop && me < ni; ++di) {
+            int u;
+            if (me == 0) {
+                const int ds = di % kUnitSlots, nd = di / kUnitSlots;
+                if (nd > 0 && !ptx::warp_wait(&bars->u_empty[ds], (nd - 1) & 1, &bars->abort_flag)) {
+                    stop = true;
+                    break;
+                }
+                u = ptx::warp_uniform(bars->abort_flag ? units : next);
+                if (lane == 0) {
+                    bars->unit[ds] = u < units ? u : -1;
+                    ptx::mbar_arrive(&bars->u_full[ds]);
+                }
+                if (u >= units) break;
+                if (lane == 0) next = atomicAdd(A.claim, 1);   // arrives while this unit is loaded
+            } else {
+                u = take_unit(di);
+                if (u < 0) break;
             }
-            const int u = ptx::warp_uniform(bars->abort_flag ? units : next);
-            if (lane == 0) {
-                bars->unit[ds] = u < units ? u : -1;
-                ptx::mbar_arrive(&bars->u_full[ds]);
-            }
-            if (u >= units) break;
-            if (lane == 0) next = atomicAdd(A.claim, 1);   // arrives while this unit is loaded
             TileUnit tu;
             const int lay = uniform_unit(u, tu);
             const int h0 = tu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
             for (int hh = 0; hh < nh && !stop; ++hh) {
                 const int h = h0 + hh;
-                const int qs = qi & 1, nq = qi >> 1;
-                if (nq > 0 && !ptx::warp_wait(&bars->q_empty[qs], (nq - 1) & 1, &bars->abort_flag)) {
-                    stop = true;
-                    break;
+                if (me == 0) {
+                    const int qs = qi & 1, nq = qi >> 1;
+                    if (nq > 0 && !ptx::warp_wait(&bars->q_empty[qs], (nq - 1) & 1, &bars->abort_flag)) {
+                        stop = true;
+                        break;
+                    }
+                    if (ptx::elect_one()) {
+                        ptx::mbar_arrive_expect_tx(&bars->q_full[qs], 2u * (uint32_t)R * 128u);
+                        load_queries(sQ + (size_t)qs * Npad * 256, (uint32_t)Npad * 128u, &A.qmap[lay], &bars->q_full[qs], G, h,
+                                     tu.s);
+                    }
+                    __syncwarp();
+                    ++qi;
                 }
-                if (ptx::elect_one()) {
-                    ptx::mbar_arrive_expect_tx(&bars->q_full[qs], 2u * (uint32_t)R * 128u);
-                    load_queries(sQ + (size_t)qs * Npad * 256, (uint32_t)Npad * 128u, &A.qmap[lay], &bars->q_full[qs], G, h,
-                                 tu.s);
-                }
-                __syncwarp();
-                ++qi;
                 for (int j = 0; j < tu.nt; ++j) {
-                    if (ki >= kst && !ptx::warp_wait(&bars->k_empty[st], ((kphase >> st) & 1u) ^ 1u, &bars->abort_flag)) {
+                    if (issuer(j, hh) != me) continue;
+                    if (((filled >> st) & 1u) != 0u &&
+                        !ptx::warp_wait(&bars->k_empty[st], ((kphase >> st) & 1u) ^ 1u, &bars->abort_flag)) {
                         stop = true;
                         break;
                     }
@@ -694,26 +717,27 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
                     }
                     __syncwarp();
                     kphase ^= 1u << st;
-                    ++ki;
-                    st = st + 1 == kst ? 0 : st + 1;
+                    filled |= 1u << st;
+                    st = st + 1 == ring_end(me) ? ring_first(me) : st + 1;
                 }
             }
         }
         if (stop && lane == 0) give_up();
         // Drain: every issued copy lands before the CTA may exit.
-        for (int b = 0; b < kst && b < ki; ++b)
-            ptx::mbar_wait(&bars->k_full[b], ((ki - b + kst - 1) / kst - 1) & 1, 50000000ull);
+        for (int b = 0; b < kst; ++b)
+            if ((filled >> b) & 1u) ptx::mbar_wait(&bars->k_full[b], ((kphase >> b) & 1u) ^ 1u, 50000000ull);
         for (int b = 0; b < 2 && b < qi; ++b)
             ptx::mbar_wait(&bars->q_full[b], ((qi - b + 1) / 2 - 1) & 1, 50000000ull);
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
+    } else if (warp == 1 || warp == kTileMmaWarp1) {
+        // ------------------------------------------------------------ MMA issuers
+        const int me = warp == kTileMmaWarp1 ? 1 : 0;
         const uint32_t idesc = ptx::idesc_bf16_f32(128, Npad);
         const uint64_t qdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sQ)), kdesc = ptx::smem_desc_k_sw128(ptx::smem_u32(sK));
         const uint32_t qhalf = (uint32_t)Npad * 128u;
-        int qi = 0, st = 0, first = 1;
+        int qi = 0, st = ring_first(me), first = 1;
         uint32_t kphase = 0u, used = 0u, aphase = 0u;   // per stage / accumulator
         bool stop = false;
-        for (int di = 0; !stop; ++di) {
+        for (int di = 0; !stop && me < ni; ++di) {
             const int u = take_unit(di);
             if (u < 0) break;
             TileUnit tu;
@@ -727,39 +751,42 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
                 }
                 for (int j = 0; j < tu.nt; ++j) {
                     const int b = j * P + hp;
-                    // Giving up on a stage in flight is safe: the producer drains its own loads.
-                    if (!ptx::warp_wait(&bars->k_full[st], (kphase >> st) & 1u, &bars->abort_flag) ||
-                        (((used >> b) & 1u) != 0u &&
-                         !ptx::warp_wait(&bars->acc_empty[b], ((aphase >> b) & 1u) ^ 1u, &bars->abort_flag))) {
-                        stop = true;
-                        break;
-                    }
-                    ptx::tc_fence_after();
-                    if (ptx::elect_one()) {
-                        const uint64_t kd = kdesc + (uint32_t)(st * (kKTileBytes >> 4)), qd = qdesc + (uint32_t)qs * (qhalf >> 3);
-                        const uint32_t d = tmem + (uint32_t)(b * Npad);
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {
-                            const uint32_t half = kk >> 2, kin = kk & 3;
-                            ptx::mma_bf16(d, kd + half * (kKTileBytes >> 5) + kin * 2, qd + half * (qhalf >> 4) + kin * 2, idesc,
-                                          kk > 0 ? 1u : 0u);
+                    if (issuer(j, hh) == me) {
+                        // Giving up on a stage in flight is safe: the producer drains its own loads.
+                        if (!ptx::warp_wait(&bars->k_full[st], (kphase >> st) & 1u, &bars->abort_flag) ||
+                            (((used >> b) & 1u) != 0u &&
+                             !ptx::warp_wait(&bars->acc_empty[b], ((aphase >> b) & 1u) ^ 1u, &bars->abort_flag))) {
+                            stop = true;
+                            break;
                         }
-                        ptx::mma_commit(&bars->k_empty[st]);
-                        if (!(fault && first)) ptx::mma_commit(&bars->acc_full[b]);
-                        if (j + 1 == tu.nt) ptx::mma_commit(&bars->q_empty[qs]);
+                        ptx::tc_fence_after();
+                        if (ptx::elect_one()) {
+                            const uint64_t kd = kdesc + (uint32_t)(st * (kKTileBytes >> 4)), qd = qdesc + (uint32_t)qs * (qhalf >> 3);
+                            const uint32_t d = tmem + (uint32_t)(b * Npad);
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk) {
+                                const uint32_t half = kk >> 2, kin = kk & 3;
+                                ptx::mma_bf16(d, kd + half * (kKTileBytes >> 5) + kin * 2, qd + half * (qhalf >> 4) + kin * 2,
+                                              idesc, kk > 0 ? 1u : 0u);
+                            }
+                            ptx::mma_commit(&bars->k_empty[st]);
+                            if (!(fault && first)) ptx::mma_commit(&bars->acc_full[b]);
+                        }
+                        __syncwarp();
+                        kphase ^= 1u << st;
+                        used |= 1u << b;
+                        aphase ^= 1u << b;
+                        st = st + 1 == ring_end(me) ? ring_first(me) : st + 1;
                     }
-                    __syncwarp();
                     first = 0;
-                    kphase ^= 1u << st;
-                    used |= 1u << b;
-                    aphase ^= 1u << b;
-                    st = st + 1 == kst ? 0 : st + 1;
                 }
+                if (ptx::elect_one()) ptx::mma_commit(&bars->q_empty[qs]);   // this issuer's products of the head
+                __syncwarp();
                 ++qi;
             }
         }
         if (stop && lane == 0) give_up();
-        if (ptx::elect_one()) ptx::mma_commit(&bars->mma_done);
+        if (me < ni && ptx::elect_one()) ptx::mma_commit(&bars->mma_done);
         __syncwarp();
     } else if (warp < 2 + 4 * NA) {
         // ------------------------------------------------------------ epilogue
@@ -768,9 +795,9 @@ __global__ void __launch_bounds__(kWinThreads, 1) window_tiles_kernel(const __gr
         const int gtid = threadIdx.x - 64 - grp * 128;
         const int quad = warp & 3;
         const int tok = quad * 32 + lane;
-        const int w = G.w, g = G.g, O = G.O;
-        const int qO = w - O, qOe = w - G.Oe;
-        const float invO = 1.f / (float)O, invOe = 1.f / (float)G.Oe;
+        const int w = DW ? kDefWindow : G.w, g = GG > 0 ? GG : G.g, O = DW ? kDefObs : G.O, Oe = DW ? kDefWindow : G.Oe;
+        const int qO = w - O, qOe = w - Oe;
+        const float invO = 1.f / (float)O, invOe = 1.f / (float)Oe;
         const float sl2 = G.sl2;
         const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(grp * Npad);
         float* rs_g = rsm + grp * 2 * 256;
@@ -955,8 +982,10 @@ cudaError_t configure_window(const Geometry& g) {
     for (auto fn : {window_kernel<0>, window_kernel<1>, window_kernel<2>, window_kernel<4>, window_kernel<7>,
                     window_kernel<8>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemWin);
-    for (auto fn : {window_tiles_kernel<0>, window_tiles_kernel<1>, window_tiles_kernel<2>, window_tiles_kernel<4>,
-                    window_tiles_kernel<7>, window_tiles_kernel<8>})
+    for (auto fn : {window_tiles_kernel<0, true>, window_tiles_kernel<1, true>, window_tiles_kernel<2, true>,
+                    window_tiles_kernel<4, true>, window_tiles_kernel<7, true>, window_tiles_kernel<8, true>,
+                    window_tiles_kernel<0, false>, window_tiles_kernel<1, false>, window_tiles_kernel<2, false>,
+                    window_tiles_kernel<4, false>, window_tiles_kernel<8, false>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemWin);
     return e;
 }
@@ -1022,7 +1051,7 @@ cudaError_t launch_window_tiles(const ScorePlan& sp, const Geometry& g, const Gr
     const int grid = a.units < usable ? a.units : usable;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kWinThreads);
+    cfg.blockDim = dim3(kTileThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -1030,13 +1059,17 @@ cudaError_t launch_window_tiles(const ScorePlan& sp, const Geometry& g, const Gr
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = after_own_launch ? 1 : 0;
+    const bool dw = g.w == kDefWindow && g.Oe == kDefWindow && g.O == kDefObs;
+    const auto launch = [&](auto with_dw, auto without) {
+        return dw ? cudaLaunchKernelEx(&cfg, with_dw, a) : cudaLaunchKernelEx(&cfg, without, a);
+    };
     switch (g.g) {
-        case 1: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<1>, a);
-        case 2: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<2>, a);
-        case 4: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<4>, a);
-        case 7: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<7>, a);
-        case 8: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<8>, a);
-        default: return cudaLaunchKernelEx(&cfg, window_tiles_kernel<0>, a);
+        case 1: return launch(window_tiles_kernel<1, true>, window_tiles_kernel<1, false>);
+        case 2: return launch(window_tiles_kernel<2, true>, window_tiles_kernel<2, false>);
+        case 4: return launch(window_tiles_kernel<4, true>, window_tiles_kernel<4, false>);
+        case 7: return launch(window_tiles_kernel<7, true>, window_tiles_kernel<0, false>);
+        case 8: return launch(window_tiles_kernel<8, true>, window_tiles_kernel<8, false>);
+        default: return launch(window_tiles_kernel<0, true>, window_tiles_kernel<0, false>);
     }
 }
 
