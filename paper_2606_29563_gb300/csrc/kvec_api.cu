@@ -63,7 +63,7 @@ struct TimedLaunch {
 int kvec::test_fault() { return g_test_fault.load(std::memory_order_relaxed); }
 
 constexpr int kSlots = 4 * kMaxGroup;   // per-layer score arrays in flight between the score and select stages
-constexpr int kPartials = 2 * kMaxGroup;   // layers whose segment partials are in flight
+constexpr int kPartials = 4 * kMaxGroup;   // layers whose segment partials are in flight
 constexpr int kSelRing = 32;               // layers whose kept-position bits are in flight to the gather
 constexpr size_t kSlotBytes = size_t(8) << 30;
 constexpr size_t kPartialsBytes = size_t(128) << 20;   // for the segment partials of the layers in flight
@@ -382,16 +382,26 @@ cudaError_t restore_full_edges(cudaGraph_t graph, const std::vector<std::pair<cu
         if (e_ != cudaSuccess) return cuda_fail(e_, #call);   \
     } while (0)
 
-// Layers that share a launch: the persistent grids' start and end (about 10 us)
-// weigh less on more layers, so as many as the ring of slots and partials leaves
-// room for two groups of, and four groups or more of a long call.  The last groups
-// halve, as nothing overlaps the last one's selection.  (32 layers in us with 1 / 2
-// / 4 / 8 layers a launch: ragged batch of 8 prompts 2896 / 2624 / 2436 / 2327, one
-// prompt of 8192 tokens 816 / 571 / 452 / 421.)
+// Layers that share a launch, from layer l0 on.  The persistent grids' start and end
+// (about 10 us) weigh less on more layers, so as many as fit (32 layers in us with
+// 1 / 2 / 4 / 8 layers a launch: ragged batch of 8 prompts 2896 / 2624 / 2436 / 2327,
+// one prompt of 8192 tokens 816 / 571 / 452 / 421).  Where one prompt makes up most
+// of the call, its selection takes about as long as its scores and starts sooner
+// behind a first group of four (first group of 8 / 4: 8192 tokens 402 / 393, 32768
+// 1286 / 1211, Qwen shape 515 / 487; but 16 short prompts 985 / 1029, two prompts of
+// 8192 and 6000 tokens 510 / 524).
 int group_layers(const kvec_handle* h, const Geometry& G, int n, int l0) {
     if (G.max_len > kMaxRegisterRow) return 1;   // the heads kernels' key rows are one layer's
-    const int left = n - l0;
-    int gs = std::min({kMaxGroup, h->nslots / 2, h->nsegpart / 2, (n + 3) / 4, std::max((left + 1) / 2, 2), left});
+    int gs = std::min(kMaxGroup, n - l0);
+    // Without the chain kernel a layer's selection is a launch of its own (two with the
+    // adaptive fill) and the longest stage: it starts early behind small groups, which
+    // double as it falls behind (16 KV heads, 1 / 2 / 8 layers a launch / doubling: 32
+    // layers of 4200 and 3000 tokens 894 / 725 / 606 / 624 us, 8 layers of 16000 tokens
+    // 387 / 329 / 361 / 329; adaptive, 8 layers of 3000 tokens 569 / 577 / 608 / 578).
+    if (!chain_fits(G)) gs = std::min(gs, G.ada ? 1 : std::max({1, std::min(2, n / 4), l0}));
+    if (n > h->nslots) gs = std::min(gs, h->nslots / 2);       // a group selects while the next one's
+    if (n > h->nsegpart) gs = std::min(gs, std::max(h->nsegpart / 2, 1));   // scores are computed
+    if (l0 == 0 && 2 * (long long)G.total_tokens < 3 * (long long)G.max_len) gs = std::min(gs, kMaxGroup / 2);
     return std::max(1, std::min(gs, 65535 / G.batch));
 }
 
@@ -655,6 +665,7 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
             {(void**)&sl.pres, MB * Hkv * W * sizeof(uint32_t)}, {(void**)&sl.Pprime, MB * Hkv * ML * sizeof(float)},
             {(void**)&sl.wpart, max_tiles * NGmax * p.obs_window * kTileT * sizeof(float)},
             {(void**)&sl.rowstat, MB * Hkv * R * sizeof(float2)},
+            {(void**)&sl.mom, MB * Hkv * pool_chunks((int)ML) * sizeof(float4)},
         };
         parts.insert(parts.end(), sp.begin(), sp.end());
     }
@@ -842,7 +853,7 @@ kvec_status select_layers_impl(kvec_handle* h, int num_layers, int batch, const 
         if (h->seen_keys.size() == kGraphCache) h->seen_keys.erase(h->seen_keys.begin());
         h->seen_keys.push_back(key);
     }
-    if (num_layers == 1) {
+    if (num_layers == 1 && chain_fits(G)) {
         h->slots[0].sel = h->sel[0];
         s = run_layer_sequential(h, G, ios[0], st);
         h->last_slot = 0;
@@ -982,7 +993,6 @@ kvec_status kvec_select_layer_noalloc(const kvec_params* params, int batch, cons
     Part parts[] = {
         {(void**)&tmp.sc.err, sizeof(int)},                   // error word, first: see noalloc_setup
         {(void**)&tmp.claims, 2 * sizeof(int)},
-        {(void**)&tmp.sc.refused, nb * sizeof(int)},
         {(void**)&tmp.sc.nbuf, nb * round_up((size_t)params->max_seqlen, 16)},
         {(void**)&tmp.segpart[0], score_partial_bytes(make_geometry(&tmp, batch, budget, tiles, chunks, cu_seqlens_host[batch], max_len), nt)},
         {(void**)&tmp.slots[0].wpart, nt * NGv * (size_t)params->obs_window * kTileT * sizeof(float)},
@@ -1025,6 +1035,10 @@ kvec_status kvec_select_layer_noalloc(const kvec_params* params, int batch, cons
         *pt.dst = static_cast<char*>(base) + off;
         off += round_up(pt.bytes, 256);
     }
+    // In parts that nothing uses while these are: the selection's keys come after the
+    // pooled moments are read, and the chain kernel leaves the counts' copy alone.
+    tmp.slots[0].mom = reinterpret_cast<float4*>(tmp.sc.keys_sel);   // 16 bytes a row and 2048 positions
+    tmp.sc.refused = reinterpret_cast<int*>(tmp.sc.nbuf);            // 4 of a sequence's 16 bytes and more
     cudaStream_t st = (cudaStream_t)stream;
     // The rest of the array keeps the previous call's contents: every part below
     // the error word is written before it is read within the call.

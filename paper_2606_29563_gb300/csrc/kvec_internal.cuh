@@ -15,6 +15,8 @@ constexpr int kMaxPool = 15;       // largest pool kernel (halo 7)
 constexpr int kSelectThreads = 512;
 constexpr int kMaxObsWindow = 64;  // largest O: the window kernel keeps O x 128 head maxima in shared memory
 constexpr int kWinHeadsPerCta = 8; // KV heads one window CTA processes
+constexpr int kPoolChunk = 2048;   // positions of a row that one CTA pools
+__host__ __device__ inline int pool_chunks(int n) { return (n + kPoolChunk - 1) / kPoolChunk; }
 constexpr int kMaxGroup = 8;       // consecutive layers one launch may serve
 constexpr int kMaxClusterHeads = 8;      // KV heads of a sequence that one (portable) cluster serves
 constexpr int kMaxRegisterRow = 32768;   // positions whose keys a block's registers hold
@@ -64,6 +66,7 @@ struct Slot {
     float* wpart;         // [win_tiles][NG][O][kTileT] per-group head maxima of G_h[q][t] (NG > 1)
     uint32_t* sel;        // [max_batch][Hkv][words]  kept positions of the layer, one bit each
     float2* rowstat;      // [max_batch][Hkv][R]    (row max in log2 units, softmax denominator)
+    float4* mom;          // [max_batch][Hkv][pool_chunks(ML)] per chunk of pooled P_O (pool_rows_kernel)
 };
 
 struct Scratch {
@@ -95,7 +98,7 @@ struct Group {
     int nl;
     LayerIO io[kMaxGroup];
     Slot sl[kMaxGroup];
-    float2* segpart[kMaxGroup];   // score kernel's partials: [segments][accumulators][R] (max, sum)
+    float2* segpart[kMaxGroup];   // score kernel's partials: [segments][accumulators][R] or [items][R] (max, sum)
 };
 
 // One decoding step over a compacted cache (decode_kernel.cu).
@@ -145,6 +148,7 @@ struct ScorePlan {
     int grid, threads, mb;   // mb: 128-row M-blocks per KV head
     int items;               // (sequence, head, tile) work items of a layer
     int chunk;               // work items per claim of the score kernel (segment boundaries of its partials)
+    int by_item;             // layout of the partials: one slot an item instead of one a segment and group
     size_t smem;
     int num_sms;             // SMs of the device (persistent grids are sized from it)
 };

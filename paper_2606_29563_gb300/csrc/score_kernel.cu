@@ -34,6 +34,8 @@
 // The window kernel recomputes the logits with these statistics.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "kvec_internal.cuh"
 #include "sm100_ptx.cuh"
 #include "tile_loads.cuh"
@@ -114,6 +116,7 @@ struct ScoreArgs {
     int kst;      // K ring depth
     int* claim;   // the launch's chunk counter, zero before the launch
     int chunk;    // items per claim
+    int by_item;  // layout of the partials (partials_by_item)
     float2* segpart[kMaxGroup];
 };
 
@@ -490,6 +493,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
             // the two grows from a segment to the next.
             float2* const segpart = A.segpart[lay];
             p.init(i0);
+            int f = i0;   // the segment's first item
             for (int i = i0; i < i1; ++i) {
                 if ((i - i0) % NB == grp) {
                     // One warp of the group polls, the others wait in the barrier (a
@@ -551,7 +555,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
                     if (lane == 0) ptx::mbar_arrive(&bars->acc_empty[grp]);
                 }
                 if (i + 1 >= i1 || p.last_of_head()) {   // the segment ends
-                    if (vrow) segpart[((size_t)(cl + p.head()) * NB + grp) * R + row] = make_float2(seg_m, seg_z);
+                    // By item: the group's first item of the segment, if it has one (a
+                    // chunk starts at a multiple of NB).
+                    const int slot = A.by_item ? f + ((grp - f) & (NB - 1)) : (cl + p.head()) * NB + grp;
+                    if (vrow && (!A.by_item || slot <= i)) segpart[(size_t)slot * R + row] = make_float2(seg_m, seg_z);
+                    f = i + 1;
                     seg_m = -INFINITY;
                     seg_z = 0.f;
                 }
@@ -574,7 +582,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
 // layers), one thread per row, as the score kernel orders them.
 template <int NB>
 __global__ void __launch_bounds__(256) rowstat_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A,
-                                                      int chunk, int* claim, int wait_prev) {
+                                                      int chunk, int by_item, int* claim, int wait_prev) {
     // The window launch that follows may start; it waits for this grid.
     if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     // wait_prev: a programmatic dependent of the score launch right before it on
@@ -601,8 +609,12 @@ __global__ void __launch_bounds__(256) rowstat_kernel(const __grid_constant__ Ge
 #pragma unroll
         for (int k = 0; k < kSegs; ++k)
 #pragma unroll
-            for (int a = 0; a < NB; ++a)
-                pz[k][a] = g0 + k <= seg1 ? __ldcg(&src[((size_t)(g0 + k) * NB + a) * G.R]) : make_float2(-INFINITY, 0.f);
+            for (int a = 0; a < NB; ++a) {
+                const int c0 = (g0 + k - sh) * chunk, f = max(c0, ib), f1 = min(c0 + chunk, ib + nt);
+                const int slot = by_item ? f + ((a - f) & (NB - 1)) : (g0 + k) * NB + a;
+                pz[k][a] = g0 + k <= seg1 && (!by_item || slot < f1) ? __ldcg(&src[(size_t)slot * G.R])
+                                                                     : make_float2(-INFINITY, 0.f);
+            }
 #pragma unroll
         for (int k = 0; k < kSegs; ++k) {
             float ms = pz[k][0].x, zs = pz[k][0].y;
@@ -656,6 +668,15 @@ int kstages_for(const Geometry& g) {
     return kst;
 }
 
+// A layer's partials lie by segment and group (slot segment * NB + group, every one
+// written), or by item where that takes less room, i.e. with fewer than about eight
+// tiles a head: in the slot of the group's first item of the segment.
+size_t partial_slots(const Geometry& g, size_t tiles) {
+    return (tiles * g.Hkv / kChunkSmall + 1 + (size_t)g.batch * g.Hkv) * (4 / mblocks(g));
+}
+
+int partials_by_item(const Geometry& g, size_t tiles) { return tiles * g.Hkv < partial_slots(g, tiles); }
+
 size_t smem_bytes_for(const Geometry& g) { return smem_bytes_with(g, kstages_for(g)); }
 
 }  // namespace
@@ -663,7 +684,7 @@ size_t smem_bytes_for(const Geometry& g) { return smem_bytes_with(g, kstages_for
 size_t score_smem_bytes(const Geometry& g) { return smem_bytes_for(g); }
 
 size_t score_partial_bytes(const Geometry& g, size_t tiles) {
-    return (tiles * g.Hkv / kChunkSmall + 1 + (size_t)g.batch * g.Hkv) * (4 / mblocks(g)) * g.R * sizeof(float2);
+    return std::min(tiles * g.Hkv, partial_slots(g, tiles)) * g.R * sizeof(float2);
 }
 
 cudaError_t configure_score(const Geometry& g) {
@@ -719,6 +740,7 @@ cudaError_t plan_score(const Geometry& g, const Group& gr, int num_sms, ScorePla
     plan->chunk = plan->items / kChunkLarge >= usable ? kChunkLarge : kChunkSmall;
     const int nchunks = (plan->items + plan->chunk - 1) / plan->chunk * gr.nl;
     plan->grid = nchunks < usable ? nchunks : usable;
+    plan->by_item = partials_by_item(g, g.total_tiles);
     plan->threads = kScoreThreads;
     plan->mb = mblocks(g);
     plan->smem = smem_bytes_for(g);
@@ -748,8 +770,8 @@ cudaError_t launch_rowstat(const ScorePlan& plan, const Geometry& g, const Group
                            bool programmatic, bool after_score) {
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = launch_config(dim3(g.Hkv, g.batch, gr.nl), 256, 0, st, &attr, programmatic);
-    if (plan.mb == 2) return cudaLaunchKernelEx(&cfg, rowstat_kernel<2>, g, gr, plan.chunk, claim, after_score ? 1 : 0);
-    return cudaLaunchKernelEx(&cfg, rowstat_kernel<4>, g, gr, plan.chunk, claim, after_score ? 1 : 0);
+    if (plan.mb == 2) return cudaLaunchKernelEx(&cfg, rowstat_kernel<2>, g, gr, plan.chunk, plan.by_item, claim, after_score ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, rowstat_kernel<4>, g, gr, plan.chunk, plan.by_item, claim, after_score ? 1 : 0);
 }
 
 cudaError_t launch_rowstat_lse(const Geometry& g, const Group& gr, cudaStream_t st, bool programmatic) {
@@ -774,6 +796,7 @@ cudaError_t launch_score(const ScorePlan& plan, const Geometry& g, const Group& 
     a.kst = kstages_for(g);
     a.claim = claim;
     a.chunk = plan.chunk;
+    a.by_item = plan.by_item;
     // after_own_launch: the previous kernel on the stream is the previous
     // group's launch, whose results this grid does not read; the launch is then
     // its programmatic dependent and never executes griddepcontrol.wait.

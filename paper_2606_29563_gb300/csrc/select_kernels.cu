@@ -6,6 +6,8 @@
 // shared by all keys skipped, 4-bit digits counted in registers, one barrier
 // per digit, small threshold buckets compacted and ranked directly).  Ties at
 // the threshold go to the lower position.
+#include <algorithm>
+
 #include "hist_select.cuh"
 #include "kvec_internal.cuh"
 
@@ -729,27 +731,8 @@ struct Pooled4 {
     float v[4];
 };
 
-__device__ __forceinline__ Pooled4 pool4(const float* __restrict__ raw, size_t stride, int parts, int t4, int Lc,
-                                         int halo, bool avg) {
-    float x[20];
-#pragma unroll
-    for (int i = 0; i < 20; ++i) x[i] = 0.f;
-    for (int pt = 0; pt < parts; ++pt) {
-        const float* r = raw + pt * stride;
-        float4 f[5];
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-            const int p = t4 - 8 + 4 * b;
-            f[b] = (p >= 0 && p < Lc) ? __ldcg(reinterpret_cast<const float4*>(r + p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-            x[4 * b] += f[b].x;
-            x[4 * b + 1] += f[b].y;
-            x[4 * b + 2] += f[b].z;
-            x[4 * b + 3] += f[b].w;
-        }
-    }
+// Pools the four positions [t4, t4 + 4) of a row from its values x at [t4 - 8, t4 + 12).
+__device__ __forceinline__ Pooled4 pool_window(float* x, int t4, int Lc, int halo, bool avg) {
     Pooled4 out;
     if (avg) {
         // Average variant: the mean of the in-range neighbours.
@@ -783,6 +766,30 @@ __device__ __forceinline__ Pooled4 pool4(const float* __restrict__ raw, size_t s
         out.v[i] = m;
     }
     return out;
+}
+
+__device__ __forceinline__ Pooled4 pool4(const float* __restrict__ raw, size_t stride, int parts, int t4, int Lc,
+                                         int halo, bool avg) {
+    float x[20];
+#pragma unroll
+    for (int i = 0; i < 20; ++i) x[i] = 0.f;
+    for (int pt = 0; pt < parts; ++pt) {
+        const float* r = raw + pt * stride;
+        float4 f[5];
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            const int p = t4 - 8 + 4 * b;
+            f[b] = (p >= 0 && p < Lc) ? __ldcg(reinterpret_cast<const float4*>(r + p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            x[4 * b] += f[b].x;
+            x[4 * b + 1] += f[b].y;
+            x[4 * b + 2] += f[b].z;
+            x[4 * b + 3] += f[b].w;
+        }
+    }
+    return pool_window(x, t4, Lc, halo, avg);
 }
 
 // Running (count, mean, sum of squared deviations); merge() is Chan et al.'s
@@ -850,7 +857,180 @@ __device__ Moments block_moments(Moments v, float3* red) {
     return t;
 }
 
-// Section 4.1, first half.  One CTA per (KV head, sequence, layer): pool the head's
+// Section 4.1, first half, with one head group (Hkv <= 8): the pooled rows P_O and
+// P_O' of every KV head and the pooled I (max-pool, inherited from SnapKV; or the
+// average variant), and per chunk of a head's pooled P_O what its ranking key is
+// merged from (head_key).  Grid (chunks, Hkv + 1, layers * batch); row Hkv is I.
+//
+// A chunk per CTA: a CTA per row spends its time waiting for one round of loads
+// after another (8192 tokens, one layer: 13.3 us on eight CTAs, 4.5 us here).
+__global__ void __launch_bounds__(256) pool_rows_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A,
+                                                        int* claim) {
+    __shared__ float3 red[8];
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    // The window grid has completed: its work counter is free for the next launch.
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) claim[1] = 0;
+    const int h = blockIdx.y, s = blockIdx.z % G.batch;
+    const LayerIO& io = A.io[blockIdx.z / G.batch];
+    const Slot& sl = A.sl[blockIdx.z / G.batch];
+    const int Lc = io.cu[s + 1] - io.cu[s] - G.wk;
+    const int t_lo = blockIdx.x * kPoolChunk, t_hi = min(t_lo + kPoolChunk, Lc);
+    if (t_lo >= Lc) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int halo = G.pool / 2;
+    const bool avg = G.pool_avg != 0;
+    const size_t row = (size_t)s * G.Hkv + h;
+    // The raw rows of the chunk and eight positions on either side, in one round of
+    // loads (pooling from global memory reads every value five times).
+    __shared__ __align__(16) float buf[2][kPoolChunk + 16];
+    const bool imp = h == G.Hkv;
+    const float* rows[2] = {imp ? sl.rawI + (size_t)s * G.ML : sl.rawO + row * G.ML, sl.rawOe + row * G.ML};
+    float* outs[2] = {imp ? sl.I + (size_t)s * G.ML : sl.PO + row * G.ML, sl.POe + row * G.ML};
+    const int nrows = imp ? 1 : 2;
+    constexpr int kRounds = kPoolChunk / 1024;
+    {
+        float4 v[2][kRounds + 1];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int k = 0; k <= kRounds; ++k) {
+                const int at = 4 * tid + 1024 * k, t = t_lo - 8 + at;   // the last round: the far halo
+                v[r][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (r < nrows && at < kPoolChunk + 16 && t >= 0 && t < Lc)
+                    v[r][k] = __ldcg(reinterpret_cast<const float4*>(rows[r] + t));
+            }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int k = 0; k <= kRounds; ++k) {
+                const int at = 4 * tid + 1024 * k;
+                if (r < nrows && at < kPoolChunk + 16) *reinterpret_cast<float4*>(&buf[r][at]) = v[r][k];
+            }
+    }
+    __syncthreads();
+    auto pooled = [&](int r, int k) {
+        const int at = 4 * tid + 1024 * k;
+        float w[20];
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            const float4 f = *reinterpret_cast<const float4*>(&buf[r][at + 4 * b]);
+            w[4 * b] = f.x;
+            w[4 * b + 1] = f.y;
+            w[4 * b + 2] = f.z;
+            w[4 * b + 3] = f.w;
+        }
+        return pool_window(w, t_lo + at, Lc, halo, avg);
+    };
+    // Count, sum and, in a second step over the registers, squared deviations from
+    // the thread's mean; or, for the entropy criterion, the sums of x and x ln x.
+    float n = 0.f, sum = 0.f, second = 0.f;
+    float x[4 * kRounds];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        if (r >= nrows) break;
+#pragma unroll
+        for (int k = 0; k < kRounds; ++k) {
+            const int t4 = t_lo + 4 * tid + 1024 * k;
+            Pooled4 p;
+            p.v[0] = p.v[1] = p.v[2] = p.v[3] = 0.f;
+            if (t4 < t_hi) {
+                p = pooled(r, k);
+                *reinterpret_cast<float4*>(outs[r] + t4) = make_float4(p.v[0], p.v[1], p.v[2], p.v[3]);
+            }
+            if (r == 0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const bool in = t4 + i < t_hi;
+                    x[4 * k + i] = in ? p.v[i] : 0.f;
+                    n += in ? 1.f : 0.f;
+                    sum += x[4 * k + i];
+                }
+            }
+        }
+    }
+    // The preserved-token kernel may be scheduled now; it waits for this grid.
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (imp) return;
+    const float mean = n > 0.f ? sum / n : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4 * kRounds; ++i) {
+        if (G.head_entropy) {
+            if (x[i] > 0.f) second = fmaf(x[i], logf(x[i]), second);
+        } else if (t_lo + 4 * tid + 1024 * (i >> 2) + (i & 3) < t_hi) {
+            second = fmaf(x[i] - mean, x[i] - mean, second);
+        }
+    }
+    float4* mom = sl.mom + row * pool_chunks(G.ML) + blockIdx.x;
+    if (G.head_entropy) {
+        for (int o = 16; o; o >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            second += __shfl_xor_sync(0xffffffffu, second, o);
+        }
+        if (lane == 0) red[warp] = make_float3(sum, second, 0.f);
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < 8; ++w) {
+                sum += red[w].x;
+                second += red[w].y;
+            }
+            *mom = make_float4(sum, second, 0.f, 0.f);
+        }
+    } else {
+        Moments m{n, mean, second};
+        for (int o = 16; o; o >>= 1)
+            m.merge(__shfl_xor_sync(0xffffffffu, m.n, o), __shfl_xor_sync(0xffffffffu, m.mean, o),
+                    __shfl_xor_sync(0xffffffffu, m.m2, o));
+        if (lane == 0) red[warp] = make_float3(m.n, m.mean, m.m2);
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < 8; ++w) m.merge(red[w].x, red[w].y, red[w].z);
+            *mom = make_float4(m.n, m.mean, m.m2, 0.f);
+        }
+    }
+}
+
+// The ranking key of KV head h of sequence s (lower keys take O' first): the
+// sample standard deviation of its pooled P_O over the Lc candidates, or minus its
+// entropy; merged from pool_rows_kernel's chunks, or as heads_pool_kernel left it.
+__device__ __forceinline__ float head_key(const Geometry& G, const Slot& sl, int s, int h, int Lc) {
+    const size_t row = (size_t)s * G.Hkv + h;
+    if (G.NG > 1) return __ldcg(&sl.sigma[row]);
+    const float4* mom = sl.mom + row * pool_chunks(G.ML);
+    const int nc = pool_chunks(Lc);
+    if (G.head_entropy) {
+        float sum = 0.f, xlx = 0.f;
+        for (int c = 0; c < nc; ++c) {
+            const float4 v = __ldcg(&mom[c]);
+            sum += v.x;
+            xlx += v.y;
+        }
+        return sum > 0.f ? xlx / sum - logf(sum) : 0.f;
+    }
+    Moments m{0.f, 0.f, 0.f};
+    for (int c0 = 0; c0 < nc; c0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            v[c] = c0 + c < nc ? __ldcg(&mom[c0 + c]) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) m.merge(v[c].x, v[c].y, v[c].z);
+    }
+    return Lc >= 2 ? sqrtf(fmaxf(m.m2, 0.f) / (float)(Lc - 1)) : 0.f;
+}
+
+// Whether head h is among the delta heads with the lowest keys; called by a whole
+// warp, every lane the same answer.  Ties to the lower head.  Lane h's key is left
+// in *key.
+__device__ __forceinline__ bool head_takes_ext(const Geometry& G, const Slot& sl, int s, int h, int Lc, float* key) {
+    const int lane = threadIdx.x & 31;
+    const float so = lane < G.Hkv ? head_key(G, sl, s, lane, Lc) : INFINITY;
+    const float sigma = __shfl_sync(0xffffffffu, so, h);
+    const bool before = lane < G.Hkv && (so < sigma || (so == sigma && lane < h));
+    *key = sigma;
+    return __popc(__ballot_sync(0xffffffffu, before)) < G.delta;
+}
+
+// Section 4.1, first half, with several head groups.  One CTA per (KV head, sequence, layer): pool the head's
 // P_O and P_O' rows and a slice of I (max-pool, inherited from SnapKV; or the
 // average variant) and the head's ranking key: sigma_h = sample std of pooled
 // P_O over the candidates (Welford/Chan moments in fp32), or, for the entropy
@@ -898,13 +1078,7 @@ __global__ void __launch_bounds__(kSelectThreads) heads_pool_kernel(const __grid
     {
         const int per = ((Lc + G.Hkv - 1) / G.Hkv + 3) & ~3;
         const int a0 = min(h * per, Lc), b0 = min(a0 + per, Lc);
-        if (G.NG == 1) {
-            const float* rI = sl.rawI + (size_t)s * G.ML;
-            for (int t4 = a0 + 4 * tid; t4 < b0; t4 += 4 * NT) {
-                const Pooled4 c = pool4(rI, 0, 1, t4, Lc, halo, avg);
-                *reinterpret_cast<float4*>(sl.I + (size_t)s * G.ML + t4) = make_float4(c.v[0], c.v[1], c.v[2], c.v[3]);
-            }
-        } else {
+        {
             // The window kernel left, per group of KV heads, the maxima over the
             // group of G_h[q][t] (q >= w - O): raw I is (1/O) times the sum over q of
             // the maxima over the groups.  Built in shared memory chunk by chunk (with
@@ -1003,13 +1177,12 @@ __global__ void __launch_bounds__(kSelectThreads, 2) heads_topk_kernel(const __g
     // read only after that grid has completed.
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     if (tid < 32) {
-        const float sigma = __ldcg(&sl.sigma[row]);
-        const float so = tid < G.Hkv ? __ldcg(&sl.sigma[(size_t)s * G.Hkv + tid]) : INFINITY;
-        const bool before = tid < G.Hkv && (so < sigma || (so == sigma && tid < h));
-        const int rank = __popc(__ballot_sync(0xffffffffu, before));
+        float key;
+        const bool ext = head_takes_ext(G, sl, s, h, Lc, &key);
         if (tid == 0) {
-            top_flag = rank < G.delta;
-            sl.htop[row] = rank < G.delta;
+            top_flag = ext;
+            sl.htop[row] = ext;
+            if (G.NG == 1) sl.sigma[row] = key;
         }
     }
     __syncthreads();
@@ -1054,7 +1227,7 @@ __global__ void __launch_bounds__(NT) heads_topk_reg_kernel(const __grid_constan
     __shared__ HistSelectShared sm;
     __shared__ __align__(16) uint32_t bits[HS::kWords];
     const int h = blockIdx.x, s = blockIdx.y;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x;
     const int L = io.cu[s + 1] - io.cu[s];
     const int Lc = L - G.wk;
     const size_t row = (size_t)s * G.Hkv + h;
@@ -1063,12 +1236,18 @@ __global__ void __launch_bounds__(NT) heads_topk_reg_kernel(const __grid_constan
     // Programmatic dependent of the pooling kernel: its sigmas and pooled rows are
     // read only after that grid has completed.
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    // Every warp ranks the sequence's sigmas the same way.
-    const float sigma = __ldcg(&sl.sigma[row]);
-    const float so = lane < G.Hkv ? __ldcg(&sl.sigma[(size_t)s * G.Hkv + lane]) : INFINITY;
-    const bool before = lane < G.Hkv && (so < sigma || (so == sigma && lane < h));
-    const bool top = __popc(__ballot_sync(0xffffffffu, before)) < G.delta;
-    if (tid == 0) sl.htop[row] = top;
+    __shared__ int ext_flag;
+    if (tid < 32) {
+        float key;
+        const bool ext = head_takes_ext(G, sl, s, h, Lc, &key);
+        if (tid == 0) {
+            ext_flag = ext;
+            sl.htop[row] = ext;
+            if (G.NG == 1) sl.sigma[row] = key;
+        }
+    }
+    __syncthreads();
+    const bool top = ext_flag;
     uint32_t* pres = sl.pres + row * G.words;
     if (L <= G.budget || G.Kp == 0) {
         for (int wd = tid; wd < G.words; wd += NT) pres[wd] = 0u;
@@ -1413,23 +1592,26 @@ __global__ void __launch_bounds__(kSelectThreads) finalize_kernel(Geometry G, La
 // out_idx[s,h,j] = position of the j-th kept bit of (s, h) (-1 past the last),
 // j < cap (the budget, or the head capacity of the adaptive fill);
 // out_k[s,h,j,:] = K[cu[s] + idx, h, :] (zeros for idx = -1); the same for V.
-// Grid (ceil(cap/16), Hkv, layers * batch), 256 threads: the block finds its 16 ranks from
-// a prefix count over the row's bits words, then a half-warp moves one 256-byte row.
+// Grid (ceil(cap/64), Hkv, layers * batch), 256 threads: the block finds its 64
+// ranks from a prefix count over the row's bits words, then each half-warp moves
+// four 256-byte rows of K and of V, all of their loads in flight together (sixteen
+// ranks a block took 1.9 times the SM time: every block counts the whole row).
+constexpr int kGatherRows = 64;
 __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A) {
     __shared__ int wsum[32];
-    __shared__ int spos[16];
+    __shared__ int spos[kGatherRows];
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int s = blockIdx.z % G.batch, h = blockIdx.y;
     const LayerIO& io = A.io[blockIdx.z / G.batch];
     const Slot& sl = A.sl[blockIdx.z / G.batch];
     const int tid = threadIdx.x, NT = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5;
-    const int L = io.cu[s + 1] - io.cu[s];
+    const int c0 = io.cu[s], L = io.cu[s + 1] - c0;
     const int wordsL = (L + 31) >> 5;
     const size_t srow = (size_t)s * G.Hkv + h;
     const uint32_t* sel = sl.sel + srow * G.words;
-    const int r0 = blockIdx.x * 16;
-    if (tid < 16) spos[tid] = -1;
+    const int r0 = blockIdx.x * kGatherRows;
+    if (tid < kGatherRows) spos[tid] = -1;
     // Contiguous runs of words per thread, ranked by an exclusive prefix sum.
     const int wpt = (wordsL + NT - 1) / NT;
     const int w_lo = min(tid * wpt, wordsL), w_hi = min(w_lo + wpt, wordsL);
@@ -1437,10 +1619,10 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geo
     for (int wd = w_lo; wd < w_hi; ++wd) mine += __popc(__ldcg(&sel[wd]));
     int total;
     int rank = block_exclusive_sum(mine, wsum, total);   // its barriers also order spos's initialisation
-    if (rank < r0 + 16 && rank + mine > r0) {
-        for (int wd = w_lo; wd < w_hi && rank < r0 + 16; ++wd) {
+    if (rank < r0 + kGatherRows && rank + mine > r0) {
+        for (int wd = w_lo; wd < w_hi && rank < r0 + kGatherRows; ++wd) {
             uint32_t b = __ldcg(&sel[wd]);
-            while (b && rank < r0 + 16) {
+            while (b && rank < r0 + kGatherRows) {
                 const int bit = __ffs(b) - 1;
                 b &= b - 1u;
                 if (rank >= r0) spos[rank - r0] = wd * 32 + bit;
@@ -1449,20 +1631,29 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geo
         }
     }
     __syncthreads();
-    const int rloc = warp * 2 + (lane >> 4), sub = lane & 15;
-    const int j = r0 + rloc;
-    if (j >= G.cap) return;
-    const size_t orow = srow * G.cap + j;
-    const int idx = spos[rloc];
-    if (sub == 0) io.out_idx[orow] = idx;
-    uint4 kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
-    if (idx >= 0 && idx < L) {
-        const size_t src = (((size_t)io.cu[s] + idx) * G.Hkv + h) * kHeadDim + sub * 8;
-        kv = __ldg(reinterpret_cast<const uint4*>(io.k + src));
-        vv = __ldg(reinterpret_cast<const uint4*>(io.v + src));
+    constexpr int kPer = kGatherRows / 16;   // rows of a half-warp
+    const int hw = warp * 2 + (lane >> 4), sub = lane & 15;
+    uint4 kv[kPer], vv[kPer];
+    int idx[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        idx[i] = spos[hw + 16 * i];
+        kv[i] = vv[i] = make_uint4(0, 0, 0, 0);
+        if (idx[i] >= 0 && idx[i] < L) {
+            const size_t src = (((size_t)c0 + idx[i]) * G.Hkv + h) * kHeadDim + sub * 8;
+            kv[i] = __ldg(reinterpret_cast<const uint4*>(io.k + src));
+            vv[i] = __ldg(reinterpret_cast<const uint4*>(io.v + src));
+        }
     }
-    reinterpret_cast<uint4*>(io.out_k + orow * kHeadDim)[sub] = kv;
-    reinterpret_cast<uint4*>(io.out_v + orow * kHeadDim)[sub] = vv;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int j = r0 + hw + 16 * i;
+        if (j >= G.cap) break;
+        const size_t orow = srow * G.cap + j;
+        if (sub == 0) io.out_idx[orow] = idx[i];
+        reinterpret_cast<uint4*>(io.out_k + orow * kHeadDim)[sub] = kv[i];
+        reinterpret_cast<uint4*>(io.out_v + orow * kHeadDim)[sub] = vv[i];
+    }
 }
 
 }  // namespace
@@ -1498,8 +1689,11 @@ cudaError_t configure_select() {
 cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, int* claim, cudaStream_t st,
                          int priority, bool programmatic) {
     const dim3 grid(g.Hkv, g.batch, gr.nl);
-    cudaError_t e = launch_prio(heads_pool_kernel, grid, dim3(kSelectThreads), g.NG > 1 ? (size_t)kPoolSmemBytes : 0, st,
-                                priority, programmatic, g, gr, claim);
+    cudaError_t e =
+        g.NG == 1 ? launch_prio(pool_rows_kernel, dim3(std::max(1, pool_chunks(g.max_len - g.wk)), g.Hkv + 1, gr.nl * g.batch),
+                                dim3(256), 0, st, priority, programmatic, g, gr, claim)
+                  : launch_prio(heads_pool_kernel, grid, dim3(kSelectThreads), (size_t)kPoolSmemBytes, st, priority,
+                                programmatic, g, gr, claim);
     if (e != cudaSuccess) return e;
     // Sixteen positions a thread while a block can hold the longest row so.
     const auto reg = [&](auto kernel, int threads) {
@@ -1535,7 +1729,8 @@ cudaError_t launch_ada(const Geometry& g, const LayerIO& io, const Scratch& sc, 
 }
 
 cudaError_t launch_gather(const Geometry& g, const Group& gr, cudaStream_t st, int priority, bool programmatic) {
-    return launch_prio(gather_kernel, dim3((g.cap + 15) / 16, g.Hkv, gr.nl * g.batch), dim3(256), 0, st, priority,
+    return launch_prio(gather_kernel, dim3((g.cap + kGatherRows - 1) / kGatherRows, g.Hkv, gr.nl * g.batch),
+                       dim3(256), 0, st, priority,
                        programmatic, g, gr);
 }
 
