@@ -4,15 +4,18 @@
 //
 // Only this step is serial across layers, so one launch walks all the layers
 // whose scores are ready.  A cluster of Hkv CTAs serves a sequence, a CTA per KV
-// head: every thread keeps the counts n_t of its positions in registers, builds
-// their keys in registers, and the heads' kept bits meet over distributed shared
-// memory behind one cluster barrier per layer, under which the next layer's
-// scores are already being loaded.  Per-layer launches instead pass the union
-// and the counts through L2 and stage the keys in shared memory: 14 to 17 us per
-// layer of one 8192-token sequence where this takes about 4.
+// head: every thread keeps the counts n_t of its positions (in shared memory for
+// the longest rows), builds their keys in registers, and the heads' kept bits meet
+// over distributed shared memory behind one cluster barrier per layer, while the
+// next layer's scores are being copied in.  A chain of dependent steps (a histogram
+// between five block barriers, then the cluster's) bounds a layer, not bandwidth.
+// Per-layer launches instead pass the union and the counts through L2 and stage the
+// keys in shared memory: 14 to 17 us per layer of one 8192-token sequence where this
+// takes about 5.5.
 #include <cooperative_groups.h>
 
 #include "hist_select.cuh"
+#include "sm100_ptx.cuh"
 
 namespace kvec {
 
@@ -20,19 +23,15 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-// Whether a row's importances are staged in shared memory beside its scores.
+// Rows of up to 16384 positions have their importances in shared memory beside the
+// scores; longer ones, whose threads need the registers, their counts.
 __host__ __device__ constexpr bool chain_stages_i(int nt, int kpt) { return nt * kpt <= 16384; }
 __host__ __device__ constexpr int chain_smem_bytes(int nt, int kpt) {
-    return nt * kpt * (int)sizeof(float) * (chain_stages_i(nt, kpt) ? 2 : 1);
+    return nt * kpt * (int)sizeof(float) + nt * kpt * (chain_stages_i(nt, kpt) ? (int)sizeof(float) : 1);
 }
 
-template <int BYTES>
-__device__ __forceinline__ void copy_async(void* dst, const void* src) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    if constexpr (BYTES == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+__device__ __forceinline__ void copy_async_word(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(ptx::smem_u32(dst)), "l"(src) : "memory");
 }
 
 struct ChainArgs {
@@ -217,15 +216,21 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
     __shared__ __align__(16) uint32_t uni[HS::kWords];       // the last layer's union
     __shared__ uint32_t spres[HS::kWords];                   // the layer's preserved bits
     __shared__ JointShared js[1];
-    // [KPT / 4][NT]: each thread's scores of the layer; then its importances, where
-    // both fit.
-    extern __shared__ __align__(16) float4 sP[];
+    __shared__ uint64_t staged;   // the layer's scores (and importances) are there
+    // The layer's scores by position, then its importances, or the counts as [KPT / 4][NT]
+    // words of four.
+    extern __shared__ __align__(128) float4 sP[];
     constexpr bool kStageI = chain_stages_i(NT, KPT);
     float4* const sI = sP + NT * KPT / 4;
+    uint32_t* const sN = reinterpret_cast<uint32_t*>(sI);
     cg::cluster_group cluster = cg::this_cluster();
     const int h = (int)cluster.block_rank(), s = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     HS::clear(sm);
+    if (tid == 0) {
+        ptx::mbar_init(&staged, 1);
+        ptx::fence_barrier_init();
+    }
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     // The scores and the state come from the kernels before this one.
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -246,48 +251,39 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         if (tid == 0) atomicExch(A.err, 2);
         return;
     }
-    uint32_t n4[KPT / 4];   // counts of this thread's positions, four bytes a word
+    uint32_t n4[kStageI ? KPT / 4 : 1];   // counts of this thread's positions, four bytes a word
+    auto counts = [&](int g) -> uint32_t& {
+        if constexpr (kStageI) return n4[g];
+        return sN[g * NT + tid];
+    };
 #pragma unroll
     for (int g = 0; g < KPT / 4; ++g) {
         const int t = HS::position(4 * g);
-        n4[g] = t < L ? __ldcg(reinterpret_cast<const uint32_t*>(nst + t)) : 0u;
+        counts(g) = t < L ? __ldcg(reinterpret_cast<const uint32_t*>(nst + t)) : 0u;
     }
     uint32_t top = 0u;   // bit l: the head takes O' in layer l
     for (int l = 0; l < A.nl; ++l) top |= (__ldg(&A.sl[l].htop[row]) != 0 ? 1u : 0u) << l;
-    // A layer's scores P, importance I and preserved bits come by asynchronous copies
-    // into shared memory, issued once the layer before has its keys: beside the score
-    // and window grids an L2 round trip takes 2 us and more, a third of the layer.
-    // (Rows of more than 16384 positions leave no room for I: it comes into registers
-    // under the cluster barrier.  A thread reads only the scores that it copied.)
+    // A layer's scores P and importance I come by bulk copies into shared memory, issued
+    // once the layer before has its keys: beside the score and window grids an L2 round
+    // trip takes 2 us and more.  (Bulk, since cp.async by every thread kept it from its
+    // own work: 32 layers of 8192 tokens 403 -> 390 us, 28 of the Qwen shape at 16384
+    // 498 -> 477.  Rows of more than 16384 positions leave no room for I, which is read
+    // where it is used: 32 layers of 32768 tokens 1086 us; loaded under the cluster
+    // barrier into 32 registers of the 64 that 1024 threads have, 1237.)
     auto stage = [&](int l) {
         const Slot& sl = A.sl[l];
-        const float* P = (((top >> l) & 1u) ? sl.POe : sl.PO) + row * A.G.ML;
-#pragma unroll
-        for (int g = 0; g < KPT / 4; ++g) {
-            const int t = HS::position(4 * g);
-            if (t < Lc) {
-                copy_async<16>(&sP[g * NT + tid], P + t);
-                if constexpr (kStageI) copy_async<16>(&sI[g * NT + tid], A.sl[l].I + (size_t)s * A.G.ML + t);
-            }
+        if (tid == 0) {
+            const float* P = (((top >> l) & 1u) ? sl.POe : sl.PO) + row * A.G.ML;
+            const uint32_t bytes = (uint32_t)((Lc + 3) & ~3) * (uint32_t)sizeof(float);
+            ptx::mbar_arrive_expect_tx(&staged, kStageI ? 2 * bytes : bytes);
+            ptx::bulk_load(sP, P, bytes, &staged);
+            if constexpr (kStageI) ptx::bulk_load(sI, sl.I + (size_t)s * A.G.ML, bytes, &staged);
         }
-        if (tid < HS::kWords && tid < wordsL) copy_async<4>(&spres[tid], sl.pres + row * words + tid);
+        if (tid < HS::kWords && tid < wordsL) copy_async_word(&spres[tid], sl.pres + row * words + tid);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    float4 im[kStageI ? 1 : KPT / 4];
-    auto load_i = [&](int l) {
-        if constexpr (kStageI) return;
-        const float* I = A.sl[l].I + (size_t)s * A.G.ML;
-#pragma unroll
-        for (int g = 0; g < KPT / 4; ++g) {
-            const int t = HS::position(4 * g);
-            if constexpr (!kStageI)
-                im[g] = t < Lc ? __ldg(reinterpret_cast<const float4*>(I + t)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    };
-    if (select) {
-        stage(0);
-        load_i(0);
-    }
+    __syncthreads();   // the barrier is set up
+    if (select) stage(0);
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
     for (int l = 0; l < A.nl; ++l) {
@@ -297,11 +293,13 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
             const float inv_l1 = __frcp_rn((float)(ell0 + (uint32_t)l + 1u));
             // P' of the last layer of a call is kept for inspection (kvec_debug_scores).
             float* Pp = A.l0 + l + 1 == A.ncall ? A.sl[l].Pprime + row * A.G.ML : nullptr;
+            // A copy that never lands is reported; the call's results are then void.
+            if (!ptx::mbar_wait(&staged, l & 1)) atomicExch(A.err, 3);
             uint32_t key[KPT];
 #pragma unroll
             for (int g = 0; g < KPT / 4; ++g) {
                 const int t0 = HS::position(4 * g);
-                const float4 p = t0 < Lc ? sP[g * NT + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 p = t0 < Lc ? sP[t0 >> 2] : make_float4(0.f, 0.f, 0.f, 0.f);
                 const uint32_t pres = t0 < Lc ? (spres[t0 >> 5] >> (t0 & 31)) & 15u : 0u;
                 // Positions that do not compete: preserved ones, and from Lc on.
                 const int lim = Lc - t0;
@@ -312,16 +310,17 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
                 const float p4[4] = {p.x, p.y, p.z, p.w};
                 float4 iv;
                 if constexpr (kStageI)
-                    iv = t0 < Lc ? sI[g * NT + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    iv = t0 < Lc ? sI[t0 >> 2] : make_float4(0.f, 0.f, 0.f, 0.f);
                 else
-                    iv = im[g];
+                    iv = t0 < Lc ? __ldg(reinterpret_cast<const float4*>(A.sl[l].I + (size_t)s * A.G.ML + t0)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 const float i4[4] = {iv.x, iv.y, iv.z, iv.w};
+                const uint32_t nc = counts(g);
                 float out[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     // coverage = n_t / (l + 1), by the rounded reciprocal; the byte n_t in
                     // the mantissa of 2^23 + n_t gives its float without a conversion.
-                    const float n = __uint_as_float(__byte_perm(n4[g], 0x4b000000u, 0x7650u + e)) - 8388608.f;
+                    const float n = __uint_as_float(__byte_perm(nc, 0x4b000000u, 0x7650u + e)) - 8388608.f;
                     const float coverage = n * inv_l1;
                     const float pp = p4[e] + A.G.lambda * (i4[e] * (1.f - coverage));
                     out[e] = pp;
@@ -330,7 +329,7 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
                 if (Pp && t0 < Lc) *reinterpret_cast<float4*>(Pp + t0) = make_float4(out[0], out[1], out[2], out[3]);
             }
             if (l + 1 < A.nl) {
-                __syncthreads();   // the preserved bits have been read
+                __syncthreads();   // the scores and the preserved bits have been read
                 stage(l + 1);
             }
             if (A.G.f0 > 0) {
@@ -367,9 +366,7 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         // cluster.  A buffer is written again two layers on, after the next
         // barrier, which every reader passes first.
         asm volatile("cp.async.wait_all;\n" ::: "memory");   // the next layer's preserved bits, read by other threads
-        auto token = cluster.barrier_arrive();
-        if (select && l + 1 < A.nl) load_i(l + 1);
-        cluster.barrier_wait(std::move(token));
+        cluster.sync();
         // A warp's union words: lane (4 hh + c) takes four words of head hh.
 #pragma unroll
         for (int part = 0; part < KPT / 16; ++part) {
@@ -390,7 +387,7 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 const uint32_t nib = (uni[w0 + g * 4 + (lane >> 3)] >> ((lane & 7) * 4)) & 15u;
-                n4[part * 4 + g] += (nib * 0x00204081u) & 0x01010101u;   // a byte per position: no count passes 255
+                counts(part * 4 + g) += (nib * 0x00204081u) & 0x01010101u;   // a byte per position: no count passes 255
             }
             // The head's kept positions, for the gather.
             if (lane < 16 && w0 + lane < wordsL) A.sl[l].sel[row * words + w0 + lane] = b[w0 + lane];
@@ -405,9 +402,9 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         const int t = HS::position(4 * g);
         if (t < f0 || t >= f1) continue;
         if (t + 4 <= L) {
-            *reinterpret_cast<uint32_t*>(nst + t) = n4[g];
+            *reinterpret_cast<uint32_t*>(nst + t) = counts(g);
         } else {
-            for (int e = 0; t + e < L; ++e) nst[t + e] = (uint8_t)(n4[g] >> (8 * e));
+            for (int e = 0; t + e < L; ++e) nst[t + e] = (uint8_t)(counts(g) >> (8 * e));
         }
     }
     if (h == 0) {
@@ -446,11 +443,15 @@ cudaError_t launch_one(const ChainArgs& a, cudaStream_t st, int priority, bool p
     return cudaLaunchKernelEx(&cfg, chain_kernel<NT, KPT, ADA>, a);
 }
 
+// As few threads as hold the longest row with 16 values each (32 from 16384 on).  One
+// layer of 8192 positions takes longer with 1024 threads and 8 values each (barriers;
+// 32 layers 395 against 387 us) and one of 16384 with 512 and 32 (28 layers of the
+// Qwen shape 477 against 468).
 template <bool ADA>
 cudaError_t launch_for(const Geometry& g, const ChainArgs& a, cudaStream_t st, int priority, bool pdl) {
     if (g.max_len <= 256 * 16) return launch_one<256, 16, ADA>(a, st, priority, pdl);
     if (g.max_len <= 512 * 16) return launch_one<512, 16, ADA>(a, st, priority, pdl);
-    if (g.max_len <= 512 * 32) return launch_one<512, 32, ADA>(a, st, priority, pdl);
+    if (g.max_len <= 1024 * 16) return launch_one<1024, 16, ADA>(a, st, priority, pdl);
     return launch_one<1024, 32, ADA>(a, st, priority, pdl);
 }
 
@@ -469,7 +470,7 @@ cudaError_t configure_one() {
 cudaError_t configure_chain() {
     cudaError_t e = configure_one<256, 16>();
     if (e == cudaSuccess) e = configure_one<512, 16>();
-    if (e == cudaSuccess) e = configure_one<512, 32>();
+    if (e == cudaSuccess) e = configure_one<1024, 16>();
     if (e == cudaSuccess) e = configure_one<1024, 32>();
     return e;
 }
