@@ -123,6 +123,8 @@ struct ScoreArgs {
 constexpr int kEpiWarps = 16;
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kScoreThreads = 64 + kEpiThreads + 64;
+constexpr int kScoreRegThreads = 896;
+static_assert(kScoreThreads <= kScoreRegThreads, "the launch bound");
 constexpr int kMmaWarp1 = 2 + kEpiWarps;   // the second issuer
 constexpr int kTmaWarp1 = 3 + kEpiWarps;   // its producer
 
@@ -155,8 +157,14 @@ __device__ __forceinline__ void merge_partial(float& M, float& Z, float2 o) {
 
 // MB: 128-row M-blocks per KV head (R <= 128 * MB).  The 16 epilogue warps form
 // NB = 4 / MB groups of 4 * MB warps, one group per TMEM accumulator.
+// Compiled for kScoreRegThreads threads, i.e. for 72 registers (nothing spills): of
+// the register file 19456 are left, so that row statistics, pooling and gather CTAs
+// run beside a score CTA that stays for its whole grid, instead of on the few SMs
+// without one.  With the 96 that 640 threads may have: ragged batch of 8 prompts 2217 us
+// (72: 2098), 16 short prompts 1052 (985), 32 layers of 8192 tokens 388 (371), of 32768
+// 1087 (1046).  The window kernel spills below 96 (given log-sum-exps 1277 -> 1308).
 template <int MB>
-__global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_constant__ ScoreArgs A) {
+__global__ void __launch_bounds__(kScoreRegThreads, 1) score_kernel(const __grid_constant__ ScoreArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // 1024-byte alignment for the swizzled operand tiles.
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
