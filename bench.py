@@ -183,7 +183,17 @@ def committed_step_traffic(wl, layers: int):
 
 
 E2E_CHUNK = 8            # layers per kvec_select_layers call in the end-to-end step
-LAUNCHES_PER_LAYER = 7   # score, row statistics, window, heads pooling, heads top-K, select, gather
+
+
+def launches_per_call(sel, step):
+    """Kernel launches of one multi-layer call, counted by the handle (layers share launches in groups):
+    score; row statistics and window; pooling and top-K; selection; gather."""
+    from paper_2606_29563_gb300 import kvec
+    kvec.kvec_set_profiling(sel.handle, True)
+    step()
+    n = [kvec.kvec_kernel_time(sel.handle, k)[1] for k in range(5)]
+    kvec.kvec_set_profiling(sel.handle, False)
+    return n[0] + 2 * n[1] + 2 * n[2] + n[3] + n[4]
 
 
 def workload_bytes(wl):
@@ -419,9 +429,7 @@ def run_ours(args, wl):
     # End to end through the public API: pinned host inputs copied in, indices and state copied out.
     e2e = run_e2e(args, wl, sel, layers, outs, state, cu_host, cu_dev, dev, stream) if args.e2e else None
 
-    # Per layer: score, row statistics, window, heads pooling, heads top-K, select,
-    # gather; per call one finalize launch (the last layer's union into the state).
-    gpu_launches = args.steps * (L_layers * LAUNCHES_PER_LAYER + 1)
+    gpu_launches = args.steps * launches_per_call(sel, step)
     sel.close()
     del layers, qs, ks, vs, outs, state
     torch.cuda.empty_cache()
