@@ -232,8 +232,6 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         ptx::fence_barrier_init();
     }
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    // The scores and the state come from the kernels before this one.
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int Hkv = A.G.Hkv, words = A.G.words, budget = A.G.budget;
     const int L = __ldg(&A.cu[s + 1]) - __ldg(&A.cu[s]);
     const int Lc = L - A.G.wk;
@@ -261,6 +259,9 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         const int t = HS::position(4 * g);
         counts(g) = t < L ? __ldcg(reinterpret_cast<const uint32_t*>(nst + t)) : 0u;
     }
+    // The state is the previous call's, complete before this call's first kernel began;
+    // the scores come from the kernels before this one.
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     uint32_t top = 0u;   // bit l: the head takes O' in layer l
     for (int l = 0; l < A.nl; ++l) top |= (__ldg(&A.sl[l].htop[row]) != 0 ? 1u : 0u) << l;
     // A layer's scores P and importance I come by bulk copies into shared memory, issued

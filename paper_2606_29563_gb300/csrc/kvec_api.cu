@@ -291,7 +291,12 @@ Geometry make_geometry(const kvec_handle* h, int batch, int budget, int tiles, i
 // the streams of the pipeline only add event waits between dependent kernels.  Each
 // kernel is a programmatic dependent of the one before it, so that its launch and
 // set-up run beside that one's end; all of them wait for their predecessor before
-// they read what it wrote, so that each has seen everything before it.
+// they read what it wrote, so that each has seen everything before it.  (The call's
+// inputs and the state, complete before its first kernel began, are read before the
+// wait.)  One layer of 8192 tokens 82 -> 66 us, of 1024 69 -> 50; with the reads before
+// the wait another 1 us of each.  Without the chain kernel the selection and the
+// finalize launch gain nothing here: 16 KV heads, 8000 tokens 91.4 us, by the
+// pipeline's streams 85.0.
 kvec_status run_layer_sequential(kvec_handle* h, const Geometry& G, const LayerIO& io, cudaStream_t st) {
     ScorePlan plan;
     Group gr{};

@@ -597,15 +597,15 @@ __global__ void __launch_bounds__(256) rowstat_kernel(const __grid_constant__ Ge
     // the stream, whose partials are read only after that grid has completed.
     // Otherwise the partials come through a full dependency and the stream's
     // previous kernel (if a programmatic predecessor at all) is not waited for.
-    if (wait_prev) asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int h = blockIdx.x, s = blockIdx.y, lay = blockIdx.z, r = threadIdx.x;
-    // The score grid has completed: its chunk counter is free for the next launch.
-    if (h == 0 && s == 0 && lay == 0 && r == 0) *claim = 0;
-    if (r >= G.R) return;
-    const int* __restrict__ cu = A.io[0].cu;
+    const int* __restrict__ cu = A.io[0].cu;   // an input: read before the wait
     int ib = 0;
     for (int b = 0; b < s; ++b) ib += tiles_of(__ldg(&cu[b + 1]) - __ldg(&cu[b])) * G.Hkv;
     const int nt = tiles_of(__ldg(&cu[s + 1]) - __ldg(&cu[s]));
+    if (wait_prev) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    // The score grid has completed: its chunk counter is free for the next launch.
+    if (h == 0 && s == 0 && lay == 0 && r == 0) *claim = 0;
+    if (r >= G.R) return;
     const int sh = s * G.Hkv + h;
     ib += h * nt;
     const int seg0 = ib / chunk + sh, seg1 = (ib + nt - 1) / chunk + sh;

@@ -867,13 +867,13 @@ __device__ Moments block_moments(Moments v, float3* red) {
 __global__ void __launch_bounds__(256) pool_rows_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A,
                                                         int* claim) {
     __shared__ float3 red[8];
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    // The window grid has completed: its work counter is free for the next launch.
-    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) claim[1] = 0;
     const int h = blockIdx.y, s = blockIdx.z % G.batch;
     const LayerIO& io = A.io[blockIdx.z / G.batch];
     const Slot& sl = A.sl[blockIdx.z / G.batch];
-    const int Lc = io.cu[s + 1] - io.cu[s] - G.wk;
+    const int Lc = io.cu[s + 1] - io.cu[s] - G.wk;   // an input: read before the wait
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    // The window grid has completed: its work counter is free for the next launch.
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) claim[1] = 0;
     const int t_lo = blockIdx.x * kPoolChunk, t_hi = min(t_lo + kPoolChunk, Lc);
     if (t_lo >= Lc) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1600,7 +1600,6 @@ constexpr int kGatherRows = 64;
 __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geometry G, const __grid_constant__ Group A) {
     __shared__ int wsum[32];
     __shared__ int spos[kGatherRows];
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int s = blockIdx.z % G.batch, h = blockIdx.y;
     const LayerIO& io = A.io[blockIdx.z / G.batch];
     const Slot& sl = A.sl[blockIdx.z / G.batch];
@@ -1612,6 +1611,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Geo
     const uint32_t* sel = sl.sel + srow * G.words;
     const int r0 = blockIdx.x * kGatherRows;
     if (tid < kGatherRows) spos[tid] = -1;
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");   // the kept bits come from the kernel before
     // Contiguous runs of words per thread, ranked by an exclusive prefix sum.
     const int wpt = (wordsL + NT - 1) / NT;
     const int w_lo = min(tid * wpt, wordsL), w_hi = min(w_lo + wpt, wordsL);
