@@ -118,3 +118,65 @@ def test_layers_of_one_call_match_layer_by_layer(layers, Hkv, seqlens, over, wit
                 assert torch.equal(p, q)
         assert torch.equal(st1, st2)
     sel.close()
+
+
+# Kernels are programmatic dependents of what precedes them on the stream; in a caller's
+# captured graph that may be a copy, a fill or another stream's kernel, whose results
+# they must still see.
+@pytest.mark.parametrize("before", ["copy", "fill", "other stream"])
+@pytest.mark.parametrize("call", ["decode", "layer"])
+def test_captured_calls_see_the_work_before_them(before, call):
+    gen = torch.Generator().manual_seed(3)
+    rand = lambda *shape: torch.randn(shape, generator=gen).to(torch.bfloat16).cuda()
+    L, Hkv, Hq, batch, cap = 8000, 8, 16, 16, 1024
+    sel = kvec.KvecSelector(kvec.make_params(Hq, Hkv, max_batch=batch, max_seqlen=8192, max_layers=2))
+    if call == "decode":
+        q, shape = rand(batch, Hq, 128), (batch, Hkv, cap, 128)
+        lens = torch.full((batch,), cap, dtype=torch.int32, device="cuda")
+        out = [torch.empty((batch, Hq, 128), device="cuda")]
+        run = lambda k, v: sel.decode_attention(q, k, v, lens, out=out[0])
+    else:
+        q, shape = rand(1, 32, Hq, 128), (L, Hkv, 128)
+        cu = torch.tensor([0, L], dtype=torch.int32).pin_memory()
+        cu_dev, state, out = cu.cuda(), sel.new_state(1), sel.alloc_outputs(1, 256)
+
+        def run(k, v):
+            kvec.kvec_reset(sel.handle, state.data_ptr(), 1, torch.cuda.current_stream().cuda_stream)
+            sel.select_layer(cu, cu_dev, q, k, v, state, 256, outs=out)
+    k, v, ks, vs = (rand(*shape) for _ in range(4))
+
+    def work():
+        if before == "copy":
+            k.copy_(ks)
+            v.copy_(vs)
+        elif before == "fill":
+            v.copy_(vs)
+            k.zero_()
+        else:
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                torch.add(ks, 1.0, out=k)
+                torch.add(vs, 1.0, out=v)
+            torch.cuda.current_stream().wait_stream(side)
+        run(k, v)
+
+    side = torch.cuda.Stream()
+    main = torch.cuda.Stream()
+    with torch.cuda.stream(main):
+        work()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=main):
+            work()
+        for _ in range(3):
+            ks.copy_(rand(*shape))
+            vs.copy_(rand(*shape))
+            work()
+            torch.cuda.synchronize()
+            expect = [o.clone() for o in out]
+            k.fill_(0.25)
+            v.fill_(0.5)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(expect, out))
+    sel.close()
