@@ -389,12 +389,12 @@ cudaError_t restore_full_edges(cudaGraph_t graph, const std::vector<std::pair<cu
 
 // Layers that share a launch, from layer l0 on.  The persistent grids' start and end
 // (about 10 us) weigh less on more layers, so as many as fit (32 layers in us with
-// 1 / 2 / 4 / 8 layers a launch: ragged batch of 8 prompts 2896 / 2624 / 2436 / 2327,
-// one prompt of 8192 tokens 816 / 571 / 452 / 421).  Where one prompt makes up most
+// 1 / 2 / 4 / 8 layers a launch: ragged batch of 8 prompts 2724 / 2412 / 2204 / 2100,
+// one prompt of 8192 tokens 657 / 480 / 400 / 375).  Where one prompt makes up most
 // of the call, its selection takes about as long as its scores and starts sooner
-// behind a first group of four (first group of 8 / 4: 8192 tokens 402 / 393, 32768
-// 1286 / 1211, Qwen shape 515 / 487; but 16 short prompts 985 / 1029, two prompts of
-// 8192 and 6000 tokens 510 / 524).
+// behind a first group of four (first group of 8 / 4: 8192 tokens 375 / 372, 32768
+// 1076 / 1045, Qwen shape 442 / 450; but 16 short prompts 973 / 1006, two prompts of
+// 8192 and 6000 tokens 495 / 503).
 int group_layers(const kvec_handle* h, const Geometry& G, int n, int l0) {
     if (G.max_len > kMaxRegisterRow) return 1;   // the heads kernels' key rows are one layer's
     int gs = std::min(kMaxGroup, n - l0);
