@@ -163,7 +163,9 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
         for (int c = 0; c < 4; ++c) acc[j][c] = 0ull;
     // This lane's logits: row lane / 4 of the block, heads j0 and j0 + 1.
     const int xr = lane >> 2, j0 = 2 * (lane & 3);
-    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+    // Maxima, what the weights refer to (0 while every row so far has a logit of
+    // minus infinity, whose weight is then 0 and not 2^(inf - inf)), and sums.
+    float m[2] = {-INFINITY, -INFINITY}, ref[2] = {0.f, 0.f}, l[2] = {0.f, 0.f};
     int st = 0;
     for (int b = b0; b < b_end; b += kDecWarps) {
         cp_async_wait<ST - 2>();
@@ -194,7 +196,8 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
             float corr[2];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                corr[c] = ptx::ex2(m[c] - mn[c]);   // 0 while m is -inf
+                ref[c] = mn[c] == -INFINITY ? 0.f : mn[c];
+                corr[c] = ptx::ex2(m[c] - ref[c]);   // 0 while m is -inf
                 l[c] *= corr[c];
                 m[c] = mn[c];
             }
@@ -208,7 +211,7 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
         }
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            x[c] = ptx::ex2(x[c] - m[c]);
+            x[c] = ptx::ex2(x[c] - ref[c]);
             l[c] += x[c];
         }
         if (j0 < GP) {
@@ -293,7 +296,8 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
     if (splits == 1) return;
     cluster.sync();
     // CTA r merges query heads r, r + splits, ... over the cluster:
-    // out = sum_c 2^(m_c - M) o_c / sum_c 2^(m_c - M) l_c, zeros for an empty cache.
+    // out = sum_c 2^(m_c - M) o_c / sum_c 2^(m_c - M) l_c, zeros for an empty cache
+    // (and where every logit is minus infinity).
     for (int i = tid; sp + (i / kHeadDim) * splits < g; i += kDecThreads) {
         const int j = sp + (i / kHeadDim) * splits, c = i % kHeadDim;
         float mc[kDecMaxSplits], M = -INFINITY;

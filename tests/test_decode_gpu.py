@@ -114,6 +114,27 @@ def test_batches_over_every_cluster_size(batch, Hq, Hkv):
     _check(_selector(Hq, Hkv, max_batch=batch), q, k.cuda(), v.cuda(), lens)
 
 
+@pytest.mark.parametrize("Hq,Hkv", [(8, 8), (8, 4), (32, 8), (56, 8)])
+@pytest.mark.parametrize("batch,cap", [(1, 40), (4, 530), (80, 130)])
+def test_minus_infinite_logits_have_no_weight(batch, cap, Hq, Hkv):
+    # Keys of minus infinity meet positive queries: the first block of eight rows, every
+    # warp's first blocks, the first half (whole CTAs of a cluster), and all rows but the
+    # last.  A cache with nothing else gives zeros, as an empty one.
+    gen = torch.Generator().manual_seed(cap + Hq)
+    q = _rand((batch, Hq, 128), gen)
+    q[:, :, 0] = q[:, :, 0].abs() + 0.5
+    k = _rand((batch, Hkv, cap, 128), gen)
+    v = _rand((batch, Hkv, cap, 128), gen)
+    sel = _selector(Hq, Hkv, max_batch=batch)
+    for masked in (min(8, cap - 1), min(64, cap - 1), cap // 2, cap - 1):
+        km = k.clone()
+        km[:, :, :masked, 0] = -float("inf")
+        _check(sel, q, km, v, [cap] * batch)
+    km[:, :, :, 0] = -float("inf")
+    lens = torch.full((batch,), cap, dtype=torch.int32, device="cuda")
+    assert not sel.decode_attention(q, km, v, lens).any()
+
+
 def test_peaked_softmax_and_garbage_past_lens():
     gen = torch.Generator().manual_seed(7)
     sel = _selector(8, 2)
