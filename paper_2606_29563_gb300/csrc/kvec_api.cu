@@ -1149,7 +1149,7 @@ kvec_status kvec_sync_status(kvec_handle* h) {
     return KVEC_OK;
 }
 
-void kvec_set_test_fault(int fault) { g_test_fault.store(fault == 1 ? 1 : 0, std::memory_order_relaxed); }
+void kvec_set_test_fault(int fault) { g_test_fault.store(fault == 1 || fault == 2 ? fault : 0, std::memory_order_relaxed); }
 
 kvec_status kvec_set_profiling(kvec_handle* h, int enable) {
     if (!h) return fail(KVEC_ERR_INVALID_ARG, "handle is NULL");

@@ -117,6 +117,7 @@ struct ScoreArgs {
     int* claim;   // the launch's chunk counter, zero before the launch
     int chunk;    // items per claim
     int by_item;  // layout of the partials (partials_by_item)
+    int fault;    // test of the error path (kvec_set_test_fault): one epilogue warp gives up on its first chunk
     float2* segpart[kMaxGroup];
 };
 
@@ -481,11 +482,16 @@ __global__ void __launch_bounds__(kScoreRegThreads, 1) score_kernel(const __grid
         uint32_t nb = 0u;   // items of this group so far
         bool aborted = false;
         while (!aborted) {
-            // Each warp takes the next claimed chunk by itself (-1: no more work).
+            // Each warp takes the next claimed chunk by itself (-1: no more work); the
+            // group's warps go on with it or, when one of them gave up, leave together (the
+            // barrier of an item would wait without a limit for a warp that has left).
             const int ds = di % kChunkSlots;
             int c = -1;
+            bool got = true;
             if (lane == 0) {
-                if (ptx::mbar_wait_abortable(&bars->c_full[ds], (di / kChunkSlots) & 1, &bars->abort_flag)) {
+                got = !(A.fault && ew == 1 && di == 0) &&
+                      ptx::mbar_wait_abortable(&bars->c_full[ds], (di / kChunkSlots) & 1, &bars->abort_flag);
+                if (got) {
                     c = bars->chunk[ds];
                     ptx::mbar_arrive(&bars->c_empty[ds]);
                 } else {
@@ -493,6 +499,7 @@ __global__ void __launch_bounds__(kScoreRegThreads, 1) score_kernel(const __grid
                 }
             }
             c = __shfl_sync(0xffffffffu, c, 0);
+            if (ptx::named_bar_or(1 + grp, 32 * GW, !got)) break;
             ++di;
             if (c < 0) break;
             const int lay = c / per_layer, cl = c - lay * per_layer;
@@ -805,6 +812,7 @@ cudaError_t launch_score(const ScorePlan& plan, const Geometry& g, const Group& 
     a.claim = claim;
     a.chunk = plan.chunk;
     a.by_item = plan.by_item;
+    a.fault = test_fault() == 2 ? 1 : 0;
     // after_own_launch: the previous kernel on the stream is the previous
     // group's launch, whose results this grid does not read; the launch is then
     // its programmatic dependent and never executes griddepcontrol.wait.

@@ -55,3 +55,27 @@ def test_window_wait_timeout_is_reported_and_the_handle_recovers():
     errs = parity.run_parity(wl, sel=sel)
     assert not errs, "\n".join(errs[:25])
     sel.close()
+
+
+# One and two M-blocks of query rows: groups of four and of eight epilogue warps.
+@pytest.mark.parametrize("q_heads", [8, 16])
+def test_a_warp_that_gives_up_takes_its_group_along(q_heads):
+    """kvec_set_test_fault(2): one epilogue warp of every score CTA reports that it gave
+    up while its siblings have work; the group has to leave together (the barrier of an
+    item has no limit), and the call is reported as timed out."""
+    wl = synth.small_workload(seqlens=(700, 333), layers=2, budget=96, num_ext_heads=1, num_q_heads=q_heads)
+    sel = kvec.KvecSelector(kvec.params_from_workload(wl))
+    x = {k: v.cuda() for k, v in synth.make_layer(wl, 0).items()}
+    cu = torch.tensor(wl.cu_seqlens, dtype=torch.int32)
+    st = sel.new_state(wl.batch)
+    try:
+        kvec.kvec_set_test_fault(2)
+        sel.select_layer(cu, cu.cuda(), x["q_obs"], x["k"], x["v"], st, wl.budget)
+        with pytest.raises(kvec.KvecError) as e:
+            kvec.kvec_sync_status(sel.handle)
+        assert e.value.status == kvec.KVEC_ERR_DEVICE_TIMEOUT
+    finally:
+        kvec.kvec_set_test_fault(0)
+    errs = parity.run_parity(wl, sel=sel)
+    assert not errs, "\n".join(errs[:25])
+    sel.close()
