@@ -301,8 +301,9 @@ KVEC_API kvec_status kvec_kernel_time(kvec_handle* h, int kernel, double* total_
  * 20 us: the kernel records KVEC_ERR_DEVICE_TIMEOUT in the error word (read by
  * kvec_sync_status or kvec_noalloc_sync_status), drains its copies and returns,
  * and that call's outputs are invalid.  fault = 2 makes one epilogue warp of
- * every score CTA report that its wait for work gave up, at once; the rest is the
- * same.  fault = 0 (the default) switches it off.  Process-wide; while it is set,
+ * every score CTA report that its wait for work gave up, at once, and one of every
+ * general window kernel's CTA that its wait for a buffer did (at its third unit); the
+ * rest is the same.  fault = 0 (the default) switches it off.  Process-wide; while it is set,
  * multi-layer calls are neither captured into nor replayed from the handle's
  * graph cache. */
 KVEC_API void kvec_set_test_fault(int fault);

@@ -54,8 +54,9 @@ struct WinArgs {
     int nacc;                       // accumulators = epilogue groups (4, or 2 when N > 128)
     int units;                      // (layer, sequence, candidate tile, head group) units of the launch
     uint32_t tmem_cols;
-    int fault;                      // test of the error path (kvec_set_test_fault): the first
-                                    // accumulator is never signalled and its wait gives up early
+    int fault;                      // test of the error path (kvec_set_test_fault).  1: the first
+                                    // accumulator is never signalled and its wait gives up early;
+                                    // 2: a warp gives up on the head maxima buffer of its third unit
 };
 
 // Limit of the epilogue's wait for the withheld accumulator under the injected fault.
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                         ptx::mma_bf16(d, ad, bd, idesc, kk > 0 ? 1u : 0u);
                     }
                     ptx::mma_commit(&bars->empty[st]);
-                    if (!(fault && it == 0)) ptx::mma_commit(&bars->acc_full[b]);
+                    if (!(fault == 1 && it == 0)) ptx::mma_commit(&bars->acc_full[b]);
                 }
             }
             ptx::mma_commit(&bars->mma_done);
@@ -344,23 +345,23 @@ __global__ void __launch_bounds__(kWinThreads, 1)
             const int buf = ul & 1;
             int* mg = maxg + buf * G.O * kTileT;
             // The head maxima buffer of this unit parity is free once the unit two
-            // before has been folded into I (bounded wait on a flag of this CTA).
-            if (!failed && ul >= 2) {
-                int ok = 1;
+            // before has been folded into I (bounded wait on a flag of this CTA).  A warp
+            // that gives up takes its group along: the barriers below have no limit.
+            if (ul >= 2) {
+                bool ok = true;
                 if (lane == 0) {
+                    const bool give_up = fault == 2 && gtid == 32;
                     const long long c0 = clock64();
-                    while (bars->ready[buf] != ul) {
-                        if (bars->abort_flag || clock64() - c0 > 600000000ll) {
-                            ok = 0;
+                    while (give_up || bars->ready[buf] != ul) {
+                        if (give_up || bars->abort_flag || clock64() - c0 > 600000000ll) {
+                            win_abort(bars, err);
+                            ok = false;
                             break;
                         }
                         __nanosleep(64);
                     }
                 }
-                if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                    if (lane == 0) win_abort(bars, err);
-                    failed = true;
-                }
+                if (ptx::named_bar_or(bar_id, 128, !ok)) break;
                 __threadfence_block();
             }
             float pa = 0.f, pb = 0.f;
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                 if (gtid == 0) {
                     const bool ok = !bars->abort_flag &&
                                     ptx::mbar_wait_abortable(&bars->acc_full[grp], k & 1, &bars->abort_flag,
-                                                             fault && it + hh == 0 ? kFaultWaitNs : 200000000ull);
+                                                             fault == 1 && it + hh == 0 ? kFaultWaitNs : 200000000ull);
                     if (!ok) win_abort(bars, err);
                     bars->gok[grp][k & 1] = ok ? 1 : 0;
                 }
@@ -1095,7 +1096,7 @@ cudaError_t launch_window(const ScorePlan& sp, const Geometry& g, const Group& g
     a.nacc = a.Npad <= 128 ? 4 : 2;   // nacc * Npad <= 512 TMEM columns
     a.upl = units_of(g);
     a.units = gr.nl * a.upl;
-    a.fault = test_fault() == 1 ? 1 : 0;
+    a.fault = test_fault();
     a.tmem_cols = 512;   // one CTA per SM; a 32-column load past the last group's columns stays inside
     const size_t smem = win_smem_bytes(a.Npad, g.O, a.kst);
     // Persistent: at most one CTA per SM.

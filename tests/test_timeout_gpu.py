@@ -79,3 +79,30 @@ def test_a_warp_that_gives_up_takes_its_group_along(q_heads):
     errs = parity.run_parity(wl, sel=sel)
     assert not errs, "\n".join(errs[:25])
     sel.close()
+
+
+def test_a_window_warp_that_gives_up_takes_its_group_along():
+    """The same in the general window kernel (a window that is no multiple of 8), whose
+    warps wait by themselves for the head maxima of two units before: more than two units
+    for each of at most 152 CTAs, and the caller's log-sum-exp, so that no score kernel runs."""
+    wl = synth.small_workload(seqlens=(20000, 20100), layers=1, budget=96, num_q_heads=4, num_ext_heads=1,
+                              window=12, obs_window=5, ext_window=9)
+    sel = kvec.KvecSelector(kvec.params_from_workload(wl))
+    x = {k: v.cuda() for k, v in synth.make_layer(wl, 0).items()}
+    lse = torch.full((wl.batch, wl.window, wl.num_q_heads), 9.0, device="cuda")
+    cu = torch.tensor(wl.cu_seqlens, dtype=torch.int32)
+    run = lambda: sel.select_layer(cu, cu.cuda(), x["q_obs"], x["k"], x["v"], sel.new_state(wl.batch), wl.budget, lse=lse)
+    expect = run()
+    kvec.kvec_sync_status(sel.handle)
+    try:
+        kvec.kvec_set_test_fault(2)
+        run()
+        with pytest.raises(kvec.KvecError) as e:
+            kvec.kvec_sync_status(sel.handle)
+        assert e.value.status == kvec.KVEC_ERR_DEVICE_TIMEOUT
+    finally:
+        kvec.kvec_set_test_fault(0)
+    got = run()
+    kvec.kvec_sync_status(sel.handle)
+    assert all(torch.equal(a, b) for a, b in zip(expect, got))
+    sel.close()
