@@ -85,6 +85,32 @@ def test_equal_scores_of_all_heads_go_to_the_lower_head():
     sel.close()
 
 
+def test_a_refused_layer_is_complete_where_its_call_is():
+    """A call whose every sequence is refused (its state counts 255 layers) has done the
+    scores and the heads' choice when its stream reaches the next work, as another call
+    has: they are read back there without a wait in between."""
+    wl = _wl(8, seqlens=(16000, 15000), budget=500, layers=1)
+    x = {k: v.cuda() for k, v in synth.make_layer(wl, 0).items()}
+    cu = torch.tensor(wl.cu_seqlens, dtype=torch.int32)
+    cu_dev = cu.cuda()
+    views = []
+    for layers_done in (0, 255):
+        sel = kvec.KvecSelector(kvec.params_from_workload(wl))
+        state = sel.new_state(wl.batch)
+        state[:, 0] = layers_done
+        before, outs = state.clone(), sel.alloc_outputs(wl.batch, wl.budget)
+        torch.cuda.synchronize()
+        sel.select_layer(cu, cu_dev, x["q_obs"], x["k"], x["v"], state, wl.budget, outs=outs)
+        views.append(sel.debug())
+        if layers_done:
+            with pytest.raises(kvec.KvecError):
+                kvec.kvec_sync_status(sel.handle)
+            assert torch.equal(state, before)
+        sel.close()
+    for name in ("htop", "sigma", "pres_bits"):
+        assert torch.equal(views[0][name], views[1][name]), name
+
+
 # Layers per launch: more layers than score arrays, chunks that cross heads and sequences
 # (partials by item and by segment), more sequences than the walkers cache, no chain
 # kernel (nine heads, long rows), the caller's log-sum-exp, the adaptive fill.
