@@ -491,6 +491,7 @@ cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, 
     a.nl = gr.nl;
     a.ncall = ncall;
     for (int l = 0; l < gr.nl; ++l) a.sl[l] = gr.sl[l];
+    programmatic = programmatic && l0 == 0;   // else the launch before writes the state that this one reads early
     return g.ada ? launch_for<true>(g, a, st, priority, programmatic) : launch_for<false>(g, a, st, priority, programmatic);
 }
 

@@ -202,7 +202,10 @@ cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t 
 }
 
 // programmatic (here and below): a programmatic dependent of the stream's previous
-// kernel, which it waits for before it reads anything.
+// kernel, which it waits for before it reads what that kernel or those before it in
+// the call wrote.  Before the wait it may read the call's inputs and, where nothing of
+// the call has written it yet, the coverage state: both were complete before the
+// call's first kernel began.
 cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, int* claim, cudaStream_t st,
                          int priority, bool programmatic);
 // lcall: the layer's index within a call of ncall layers (0 for the first);
@@ -218,7 +221,8 @@ cudaError_t launch_heads(const Geometry& g, const Group& gr, const Scratch& sc, 
 cudaError_t launch_select(const Geometry& g, const LayerIO& io, const Scratch& sc, const Slot& sl, const Slot* prev,
                           cudaStream_t st, int priority, int lcall, int ncall, bool programmatic);
 // The same for a group whose first layer is layer l0 of a call of ncall, in one
-// launch, state and header included; needs chain_fits(g).
+// launch, state and header included; needs chain_fits(g).  It reads the state before
+// its wait, which the launch of an earlier group writes: programmatic only for l0 = 0.
 bool chain_fits(const Geometry& g);
 cudaError_t launch_chain(const Geometry& g, const Group& gr, const Scratch& sc, int l0, int ncall, cudaStream_t st,
                          int priority, bool programmatic);
