@@ -101,7 +101,16 @@ typedef struct {
 
 /* Creates a handle and allocates its device workspace on the current device.
  * Returns INVALID_ARG / UNSUPPORTED for bad parameters (nothing allocated),
- * OOM or CUDA on allocation failure.  *out is NULL on failure. */
+ * OOM or CUDA on allocation failure.  *out is NULL on failure.
+ * The workspace is one allocation of about
+ *   max_batch * ML * ((12 + 16.2 * S + S / 8) * H_kv + 8 * S + 1) bytes
+ * (ML = max_seqlen + 4 rounded up to a multiple of 32), plus up to 128 MB (or what
+ * two layers take) of softmax partials; with head_budget = 1 another 8.2 * H_kv, and
+ * with more than 8 KV heads 4 * obs_window * ceil(H_kv / 8) * S, times
+ * max_batch * ML.  S = min(max_layers, 32) layers are in flight.  S is halved, down
+ * to 8, while its part takes more than 8 GB or the whole more than a quarter of the
+ * device's free memory, and again while the allocation fails: results are the same,
+ * calls of many layers then overlap less. */
 KVEC_API kvec_status kvec_create(const kvec_params* params, kvec_handle** out);
 
 /* Frees the workspace; waits for the handle's pending work first. */
@@ -303,7 +312,8 @@ KVEC_API kvec_status kvec_kernel_time(kvec_handle* h, int kernel, double* total_
  * and that call's outputs are invalid.  fault = 2 makes one epilogue warp of
  * every score CTA report that its wait for work gave up, at once, and one of every
  * general window kernel's CTA that its wait for a buffer did (at its third unit); the
- * rest is the same.  fault = 0 (the default) switches it off.  Process-wide; while it is set,
+ * rest is the same.  fault = 3 makes kvec_create treat every allocation but the one
+ * of the shortest rings as failed.  fault = 0 (the default) switches it off.  Process-wide; while it is set,
  * multi-layer calls are neither captured into nor replayed from the handle's
  * graph cache. */
 KVEC_API void kvec_set_test_fault(int fault);

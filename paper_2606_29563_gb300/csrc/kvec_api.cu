@@ -9,6 +9,7 @@
 #include <atomic>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "kvec.h"
@@ -587,6 +588,86 @@ void release_handle(kvec_handle* h) {
     delete h;
 }
 
+// Bytes of a layer's partials of the largest call.
+size_t partials_bytes(const kvec_handle* h) {
+    const size_t tiles = (size_t)h->p.max_batch * ((row_stride(h->p.max_seqlen) + kTileT - 1) / kTileT);
+    return score_partial_bytes(make_geometry(h, h->p.max_batch, h->p.window, 1, 1, h->p.window, h->p.window), tiles);
+}
+
+// Places the workspace's arrays for the handle's ring sizes one after another from
+// `base` on (null: only counts) and returns their bytes.
+size_t lay_out_workspace(kvec_handle* h, char* base) {
+    const kvec_params& p = h->p;
+    const size_t MB = p.max_batch, ML = row_stride(p.max_seqlen), Hkv = p.num_kv_heads, R = h->R, W = h->words;
+    const size_t rows = MB * Hkv * ML * sizeof(float);   // a score a head and position
+    const size_t tiles = MB * ((ML + kTileT - 1) / kTileT);
+    const size_t groups = (Hkv + kWinHeadsPerCta - 1) / kWinHeadsPerCta;   // of KV heads
+    const size_t joint = p.head_budget ? MB * (Hkv * ML + 32) : 0;
+    size_t total = 0;
+    const auto place = [&](auto*& dst, size_t bytes) {
+        if (base) dst = reinterpret_cast<std::remove_reference_t<decltype(dst)>>(base + total);
+        total += round_up(bytes, 256);
+    };
+    place(h->sc.keys, rows);
+    place(h->sc.nbuf, MB * round_up((size_t)p.max_seqlen, 16));
+    place(h->sc.err, sizeof(int));
+    place(h->sc.refused, MB * sizeof(int));
+    place(h->sc.keys_sel, rows);
+    place(h->sc.jkeys, joint * sizeof(uint32_t));
+    place(h->sc.jpos, joint * sizeof(int32_t));
+    place(h->sc.jbits, joint / 32 * sizeof(uint32_t));
+    place(h->claims, 2 * (size_t)p.max_layers * sizeof(int));
+    for (int k = 0; k < h->nsel; ++k) place(h->sel[k], MB * Hkv * W * sizeof(uint32_t));
+    for (int k = 0; k < h->nsegpart; ++k) place(h->segpart[k], partials_bytes(h));
+    float* Pprime = nullptr;   // the last layer's of a call only: one for all slots
+    place(Pprime, rows);
+    for (int k = 0; k < h->nslots; ++k) {
+        Slot& sl = h->slots[k];
+        sl.Pprime = Pprime;
+        place(sl.rawO, rows);
+        place(sl.rawOe, rows);
+        place(sl.rawI, MB * ML * sizeof(float));
+        place(sl.PO, rows);
+        place(sl.POe, rows);
+        place(sl.I, MB * ML * sizeof(float));
+        place(sl.sigma, MB * Hkv * sizeof(float));
+        place(sl.htop, MB * Hkv * sizeof(int));
+        place(sl.pres, MB * Hkv * W * sizeof(uint32_t));
+        place(sl.rowstat, MB * Hkv * R * sizeof(float2));
+        place(sl.mom, groups == 1 ? MB * Hkv * pool_chunks((int)ML) * sizeof(float4) : 0);
+        place(sl.wpart, groups > 1 ? tiles * groups * p.obs_window * kTileT * sizeof(float) : 0);
+    }
+    return total;
+}
+
+// The rings of per-layer arrays: as long as a call has layers, up to kSlots slots,
+// kPartials partials and kSelRing kept bits, the slots of at most kSlotBytes and the
+// partials of at most kPartialsBytes.
+constexpr int kMinSlots = kMaxGroup, kMinPartials = 2, kMinSel = kMaxGroup;   // enough for any call
+
+bool rings_are_smallest(const kvec_handle* h) {
+    return h->nslots <= kMinSlots && h->nsegpart <= kMinPartials && h->nsel <= kMinSel;
+}
+
+// Halves the rings that are longer than the smallest; false: none is.
+bool shrink_rings(kvec_handle* h) {
+    if (rings_are_smallest(h)) return false;
+    h->nslots = std::max(h->nslots / 2, std::min(h->nslots, kMinSlots));
+    h->nsegpart = std::max(h->nsegpart / 2, std::min(h->nsegpart, kMinPartials));
+    h->nsel = std::max(h->nsel / 2, std::min(h->nsel, kMinSel));
+    return true;
+}
+
+void size_rings(kvec_handle* h) {
+    const int layers = h->p.max_layers;
+    h->nsel = std::min(layers, kSelRing);
+    h->nsegpart = (int)std::min<size_t>(std::min(layers, kPartials), std::max<size_t>(kMinPartials, kPartialsBytes / partials_bytes(h)));
+    h->nslots = 0;
+    const size_t other = lay_out_workspace(h, nullptr);
+    h->nslots = std::min(layers, kSlots);
+    while (h->nslots > kMinSlots && lay_out_workspace(h, nullptr) - other > kSlotBytes) h->nslots = std::max(h->nslots / 2, kMinSlots);
+}
+
 }  // namespace
 
 extern "C" {
@@ -627,56 +708,22 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
     h->n_off = 16;
     h->union_off = 16 + round_up((size_t)p.max_seqlen, 16);
 
-    const size_t MB = p.max_batch, ML = row_stride(p.max_seqlen), Hkv = p.num_kv_heads, R = h->R,
-                 W = h->words;
-    const size_t max_tiles = MB * ((ML + kTileT - 1) / kTileT);
-    const size_t HGmax = Hkv < (size_t)kWinHeadsPerCta ? Hkv : (size_t)kWinHeadsPerCta;
-    const size_t NGmax = (Hkv + HGmax - 1) / HGmax;
-    struct Part {
-        void** dst;
-        size_t bytes;
-    };
-    std::vector<Part> parts = {
-
-        {(void**)&h->sc.keys, MB * Hkv * ML * sizeof(uint32_t)},
-        {(void**)&h->sc.nbuf, MB * round_up((size_t)p.max_seqlen, 16)},
-        {(void**)&h->sc.err, sizeof(int)},
-        {(void**)&h->sc.refused, MB * sizeof(int)},
-        {(void**)&h->sc.keys_sel, MB * Hkv * ML * sizeof(uint32_t)},
-        {(void**)&h->sc.jkeys, p.head_budget ? MB * (Hkv * ML + 32) * sizeof(uint32_t) : 0},
-        {(void**)&h->sc.jpos, p.head_budget ? MB * (Hkv * ML + 32) * sizeof(int32_t) : 0},
-        {(void**)&h->sc.jbits, p.head_budget ? MB * (Hkv * ML + 32) / 32 * sizeof(uint32_t) : 0},
-        {(void**)&h->claims, 2 * (size_t)p.max_layers * sizeof(int)},
-    };
-    // Partials of as many layers as kPartialsBytes holds, of two at least.
-    Geometry Gmax = make_geometry(h, p.max_batch, p.window, 1, 1, p.window, p.window);
-    const size_t part_bytes = score_partial_bytes(Gmax, max_tiles);
-    h->nsegpart = (int)std::min<size_t>(kPartials, std::max<size_t>(2, kPartialsBytes / part_bytes));
-    h->nsel = std::min(p.max_layers, kSelRing);
-    for (int k = 0; k < h->nsel; ++k) parts.push_back({(void**)&h->sel[k], MB * Hkv * W * sizeof(uint32_t)});
-    for (int k = 0; k < h->nsegpart; ++k) parts.push_back({(void**)&h->segpart[k], part_bytes});
-    // Fewer slots (still a ring of groups) where all of them would take over kSlotBytes,
-    // and no more than a call has layers.
-    const size_t slot_bytes = (5 * MB * Hkv * ML + 2 * MB * ML + max_tiles * NGmax * p.obs_window * kTileT) * sizeof(float);
-    h->nslots = kSlots;
-    while (h->nslots > kMaxGroup && (slot_bytes * h->nslots > kSlotBytes || h->nslots / 2 >= p.max_layers)) h->nslots /= 2;
-    for (int k = 0; k < h->nslots; ++k) {
-        Slot& sl = h->slots[k];
-        std::vector<Part> sp = {
-            {(void**)&sl.rawO, MB * Hkv * ML * sizeof(float)},  {(void**)&sl.rawOe, MB * Hkv * ML * sizeof(float)},
-            {(void**)&sl.rawI, MB * ML * sizeof(float)},        {(void**)&sl.PO, MB * Hkv * ML * sizeof(float)},
-            {(void**)&sl.POe, MB * Hkv * ML * sizeof(float)},   {(void**)&sl.I, MB * ML * sizeof(float)},
-            {(void**)&sl.sigma, MB * Hkv * sizeof(float)},      {(void**)&sl.htop, MB * Hkv * sizeof(int)},
-            {(void**)&sl.pres, MB * Hkv * W * sizeof(uint32_t)}, {(void**)&sl.Pprime, MB * Hkv * ML * sizeof(float)},
-            {(void**)&sl.wpart, max_tiles * NGmax * p.obs_window * kTileT * sizeof(float)},
-            {(void**)&sl.rowstat, MB * Hkv * R * sizeof(float2)},
-            {(void**)&sl.mom, MB * Hkv * pool_chunks((int)ML) * sizeof(float4)},
-        };
-        parts.insert(parts.end(), sp.begin(), sp.end());
+    size_rings(h);
+    // Shorter rings where the device has little room (beside a model's weights and
+    // cache): fewer layers are then in flight and share a launch, down to one.
+    size_t total = lay_out_workspace(h, nullptr), free_bytes = 0, all_bytes = 0;
+    if (cudaMemGetInfo(&free_bytes, &all_bytes) == cudaSuccess) {
+        while (total > free_bytes / 4 && shrink_rings(h)) total = lay_out_workspace(h, nullptr);
+    } else {
+        cudaGetLastError();
     }
-    size_t total = 0;
-    for (auto& pt : parts) total += round_up(pt.bytes, 256);
-    e = cudaMalloc(&h->ws, total);
+    const bool refuse_all_but_smallest = test_fault() == 3;
+    for (;;) {
+        e = refuse_all_but_smallest && !rings_are_smallest(h) ? cudaErrorMemoryAllocation : cudaMalloc(&h->ws, total);
+        if (e == cudaSuccess || !shrink_rings(h)) break;
+        cudaGetLastError();
+        total = lay_out_workspace(h, nullptr);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete h;
@@ -684,11 +731,7 @@ kvec_status kvec_create(const kvec_params* params, kvec_handle** out) {
     }
     h->ws_bytes = total;
     e = cudaMemset(h->ws, 0, total);
-    size_t off = 0;
-    for (auto& pt : parts) {
-        *pt.dst = static_cast<char*>(h->ws) + off;
-        off += round_up(pt.bytes, 256);
-    }
+    lay_out_workspace(h, static_cast<char*>(h->ws));
     Geometry G = make_geometry(h, 1, p.window, 1, 1, p.window, p.window);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess) e = configure_score(G);
@@ -1149,7 +1192,7 @@ kvec_status kvec_sync_status(kvec_handle* h) {
     return KVEC_OK;
 }
 
-void kvec_set_test_fault(int fault) { g_test_fault.store(fault == 1 || fault == 2 ? fault : 0, std::memory_order_relaxed); }
+void kvec_set_test_fault(int fault) { g_test_fault.store(fault >= 1 && fault <= 3 ? fault : 0, std::memory_order_relaxed); }
 
 kvec_status kvec_set_profiling(kvec_handle* h, int enable) {
     if (!h) return fail(KVEC_ERR_INVALID_ARG, "handle is NULL");

@@ -192,7 +192,8 @@ def kvec_output_capacity(params: kvec_params, budget: int) -> int:
 
 def kvec_set_test_fault(fault: int) -> None:
     """Test hook of the error path (1: window kernels give up on a withheld accumulator;
-    2: a warp of the score and general window kernels gives up on a wait; 0: off)."""
+    2: a warp of the score and general window kernels gives up on a wait; 3: kvec_create's larger
+    allocations fail; 0: off)."""
     load().kvec_set_test_fault(int(fault))
 
 

@@ -146,6 +146,45 @@ def test_layers_of_one_call_match_layer_by_layer(layers, Hkv, seqlens, over, wit
     sel.close()
 
 
+# A handle beside a model that leaves little memory: the allocation is tried again with
+# shorter rings (8 layers in flight, partials of 2), down to a launch a layer.
+@pytest.mark.parametrize("layers,Hkv,seqlens,over", [
+    (33, 8, (1500, 700), {}), (32, 2, (9000,), {}), (12, 9, (500, 300), {}), (11, 4, (2100,), dict(head_budget=1, ada_floor=0.25)),
+])
+def test_short_rings_of_a_full_device_give_the_same(layers, Hkv, seqlens, over):
+    wl = _wl(Hkv, 2, seqlens=seqlens, budget=64, layers=layers, **over)
+    xs = [{k: v.cuda() for k, v in x.items()} for x in synth.make_layers(wl, 5)]
+    xs = [xs[l % len(xs)] for l in range(layers)]
+    cu = torch.tensor(wl.cu_seqlens, dtype=torch.int32)
+    cu_dev = cu.cuda()
+    # Room for 16384 positions and more sequences, so that the rings make up the workspace.
+    params = kvec.params_from_workload(wl, max_layers=layers, max_seqlen=16384, max_batch=8)
+    got, used = [], []
+    for fault in (0, 3):
+        free = torch.cuda.mem_get_info()[0]
+        try:
+            kvec.kvec_set_test_fault(fault)
+            sel = kvec.KvecSelector(params)
+        finally:
+            kvec.kvec_set_test_fault(0)
+        used.append(free - torch.cuda.mem_get_info()[0])
+        outs = [sel.alloc_outputs(wl.batch, wl.budget) for _ in xs]
+        for _ in range(3):   # eager, captured, replayed
+            state = sel.new_state(wl.batch)
+            sel.select_layers(cu, cu_dev, [x["q_obs"] for x in xs], [x["k"] for x in xs], [x["v"] for x in xs],
+                              state, wl.budget, outs)
+            torch.cuda.synchronize()
+            got.append([t.clone() for o in outs for t in o] + [state.clone(), sel.debug()["Pprime"][:wl.batch]])
+        sel.close()
+    for other in got[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got[0][:-1], other[:-1]))
+    for s, L in enumerate(wl.seqlens):
+        assert all(torch.equal(got[0][-1][s, :, :L - wl.window], g[-1][s, :, :L - wl.window]) for g in got[1:])
+    rows = 8 * 16416 * Hkv * 4
+    S = min(layers, 32)
+    assert used[0] - used[1] > (S - 8) * 4 * rows   # four score rows a slot less
+
+
 # Kernels are programmatic dependents of what precedes them on the stream; in a caller's
 # captured graph that may be a copy, a fill or another stream's kernel, whose results
 # they must still see.
