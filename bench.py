@@ -31,14 +31,6 @@ if ROOT not in sys.path:
 METRIC = "prefix tokens evicted/sec (all layers, device-timed) and % of HBM roofline"
 DEFAULT_WORKLOAD = "llama8b_ragged8_b256"   # the largest single-GPU configuration
 FALLBACK_HBM_GBS = 6800.0
-KERNEL_SOURCES = {
-    "score": "paper_2606_29563_gb300/csrc/score_kernel.cu",
-    "window": "paper_2606_29563_gb300/csrc/window_kernel.cu",
-    "heads": "paper_2606_29563_gb300/csrc/select_kernels.cu",
-    "select": "paper_2606_29563_gb300/csrc/select_kernels.cu",
-    "gather": "paper_2606_29563_gb300/csrc/select_kernels.cu",
-    "decode": "paper_2606_29563_gb300/csrc/decode_kernel.cu",
-}
 
 
 # ----------------------------------------------------------------------------- distributed plumbing
@@ -151,49 +143,49 @@ def measured_hbm_gbs():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-def committed_traffic(kernel: str, workload: str):
-    """dram read+write bytes per launch from a committed ncu summary, if the kernel is unchanged."""
-    path = os.path.join(ROOT, "profiles", "traffic.json")
+def sources_sha256() -> str:
+    """SHA-256 of everything libkvec is compiled from (kernels, headers, host code and the ABI header)."""
+    csrc = os.path.join(ROOT, "paper_2606_29563_gb300", "csrc")
+    paths = [os.path.join(csrc, name) for name in sorted(os.listdir(csrc)) if name.endswith((".cu", ".cuh"))]
+    sha = hashlib.sha256()
+    for path in paths + [os.path.join(ROOT, "include", "kvec.h")]:
+        with open(path, "rb") as f:
+            sha.update(os.path.basename(path).encode() + b"\0" + f.read())
+    return sha.hexdigest()
+
+
+def committed_traffic(kind: str, workload: str):
+    """The committed ncu record of DRAM traffic (profiles/traffic.json) for `workload`, if it was captured from
+    the current sources; else None."""
     try:
-        with open(path) as f:
+        with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
             data = json.load(f)
-        entry = data[kernel][workload]
-        src = open(os.path.join(ROOT, KERNEL_SOURCES[kernel]), "rb").read()
-        if entry.get("source_sha256") != hashlib.sha256(src).hexdigest():
-            return None
-        return float(entry["bytes_per_launch"])
+        return data[kind][workload] if data["sources_sha256"] == sources_sha256() else None
     except (OSError, ValueError, KeyError, TypeError):
         return None
 
 
-def committed_step_traffic(wl, layers: int):
-    """DRAM bytes (read + written) of one whole step from the committed ncu record of
-    every kernel of a layer (profiles/traffic.json, "step"), if no kernel source has
-    changed since the capture; else None."""
-    path = os.path.join(ROOT, "profiles", "traffic.json")
-    try:
-        with open(path) as f:
-            entry = json.load(f)["step"][wl.name]
-        for rel, sha in entry["sources_sha256"].items():
-            if hashlib.sha256(open(os.path.join(ROOT, rel), "rb").read()).hexdigest() != sha:
-                return None
-        return float(entry["bytes_per_layer"]) * layers
-    except (OSError, ValueError, KeyError, TypeError):
+def committed_step_traffic(wl, layers: int, score_launches: int):
+    """DRAM bytes (read + written) of one whole step from the committed record of every kernel of a layer, if
+    the step's layers share launches as the captured ones did (what a pass finds in L2 depends on it); else None."""
+    entry = committed_traffic("step", wl.name)
+    if entry is None or score_launches * entry["layers_per_launch"] != layers:
         return None
+    return float(entry["bytes_per_layer"]) * layers
 
 
 E2E_CHUNK = 8            # layers per kvec_select_layers call in the end-to-end step
 
 
-def launches_per_call(sel, step):
-    """Kernel launches of one multi-layer call, counted by the handle (layers share launches in groups):
-    score; row statistics and window; pooling and top-K; selection; gather."""
+def launch_counts(sel, step):
+    """Kernel launches of one multi-layer call, counted by the handle (layers share launches in groups): of the
+    score kernel, and of all: score; row statistics and window; pooling and top-K; selection; gather."""
     from paper_2606_29563_gb300 import kvec
     kvec.kvec_set_profiling(sel.handle, True)
     step()
     n = [kvec.kvec_kernel_time(sel.handle, k)[1] for k in range(5)]
     kvec.kvec_set_profiling(sel.handle, False)
-    return n[0] + 2 * n[1] + 2 * n[2] + n[3] + n[4]
+    return n[0], n[0] + 2 * n[1] + 2 * n[2] + n[3] + n[4]
 
 
 def workload_bytes(wl):
@@ -429,7 +421,8 @@ def run_ours(args, wl):
     # End to end through the public API: pinned host inputs copied in, indices and state copied out.
     e2e = run_e2e(args, wl, sel, layers, outs, state, cu_host, cu_dev, dev, stream) if args.e2e else None
 
-    gpu_launches = args.steps * launches_per_call(sel, step)
+    score_launches, call_launches = launch_counts(sel, step)
+    gpu_launches = args.steps * call_launches
     sel.close()
     del layers, qs, ks, vs, outs, state
     torch.cuda.empty_cache()
@@ -445,7 +438,7 @@ def run_ours(args, wl):
                    "precision": "bf16 inputs, fp32 accumulation and scores"},
         "roofline": {"bound": "hbm", "kernel": "whole eviction pass: every kernel of one kvec_select_layers call",
                      "achieved": path_gbs, "peak": peak, "unit": "GB/s", "frac": path_gbs / peak,
-                     "traffic": committed_step_traffic(wl, L_layers), "peak_source": peak_kind,
+                     "traffic": committed_step_traffic(wl, L_layers, score_launches), "peak_source": peak_kind,
                      "bytes_per_step": bytes_step,
                      "bytes": "algorithmic: K read once + q_obs + kept K/V rows read and written + out_idx",
                      "strict_frac": (by["k_read"] + by["gather"] // 2) * L_layers / (ms_per_step / 1e3) / 1e9 / peak},
@@ -583,7 +576,7 @@ def run_decode(args, wl, sel, layers, outs, dev, peak):
             "ms_per_token": ms_token, "us_per_layer_call": us_call, "tokens_per_s": 1e3 / ms_token,
             "gpu_launches_per_token": len(layers), "bytes_per_call": bytes_call,
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                         "traffic": committed_traffic("decode", wl.name)},
+                         "traffic": (committed_traffic("decode", wl.name) or {}).get("bytes_per_launch")},
             "cache_rows_per_head": lens, "cpu_baseline": res_cpu}
 
 
