@@ -22,7 +22,8 @@
  *     first and a rejected call launches nothing.
  *   - Errors are returned as kvec_status; kvec_last_error() gives a message
  *     for the calling thread.  No C++ exception crosses this boundary.
- *   - A handle is used from one host thread at a time.
+ *   - A handle is used from one host thread at a time, and its selection calls
+ *     share one workspace: calls on different streams must not overlap.
  *   - bf16 tensors are raw IEEE bfloat16 (2 bytes per element).
  */
 #ifndef KVEC_H
@@ -262,8 +263,8 @@ KVEC_API kvec_status kvec_noalloc_sync_status(kvec_stream_t stream);
  *   out      device fp32 [batch][H_q][d].
  * 1 <= batch <= max_batch, 1 <= cap <= 2^20, H_q/H_kv <= 8 (else UNSUPPORTED);
  * q, k_cache, v_cache 16-byte aligned, lens 4-byte and out 8-byte aligned.
- * Asynchronous on `stream`; the handle's decode workspace is reused by every
- * call, so calls on different streams must not overlap. */
+ * Asynchronous on `stream`; nothing of the handle is written, so calls on
+ * different streams may overlap. */
 KVEC_API kvec_status kvec_decode_attention(kvec_handle* h, int batch, const void* q,
                                            const void* k_cache, const void* v_cache,
                                            const int32_t* lens, int cap, float* out,
@@ -299,7 +300,7 @@ KVEC_API kvec_status kvec_sync_status(kvec_handle* h);
 
 /* Per-kernel device time recorded since the last kvec_set_profiling(h, 1)
  * call, from CUDA events on the launching stream.  kernel: 0 score (QK^T and
- * softmax statistics), 1 window sums + pooling, 2 cross-head choice +
+ * softmax statistics), 1 window sums, 2 pooling, cross-head choice and
  * preserved tokens, 3 coverage-adjusted selection, 4 gather.  Synchronises. */
 KVEC_API kvec_status kvec_set_profiling(kvec_handle* h, int enable);
 KVEC_API kvec_status kvec_kernel_time(kvec_handle* h, int kernel, double* total_ms, int* launches);

@@ -2,10 +2,13 @@
 // coverage-state update (Section 4.1, Section 4.2, Algorithm 1), plus the K/V
 // gather into the budget-sized cache.
 //
-// Top-k is an exact MSB radix select over order-preserving uint32 keys (bits
-// shared by all keys skipped, 4-bit digits counted in registers, one barrier
-// per digit, small threshold buckets compacted and ranked directly).  Ties at
-// the threshold go to the lower position.
+// The preserved tokens of rows up to kMaxRegisterRow positions come from a histogram
+// over keys in registers (hist_select.cuh), as the coverage-adjusted selection of up to
+// kMaxClusterHeads heads does (chain_kernel.cu).  Longer rows, and the selection with
+// more heads or longer rows (select_kernel, ada_kernel), take an exact MSB radix select
+// over order-preserving uint32 keys (bits shared by all keys skipped, 4-bit digits
+// counted in registers, one barrier per digit, small threshold buckets compacted and
+// ranked directly).  Ties at the threshold go to the lower position in both.
 #include <algorithm>
 
 #include "hist_select.cuh"
@@ -1078,70 +1081,68 @@ __global__ void __launch_bounds__(kSelectThreads) heads_pool_kernel(const __grid
     {
         const int per = ((Lc + G.Hkv - 1) / G.Hkv + 3) & ~3;
         const int a0 = min(h * per, Lc), b0 = min(a0 + per, Lc);
-        {
-            // The window kernel left, per group of KV heads, the maxima over the
-            // group of G_h[q][t] (q >= w - O): raw I is (1/O) times the sum over q of
-            // the maxima over the groups.  Built in shared memory chunk by chunk (with
-            // the pool halo), each (q, t) element loaded by its own thread, then pooled.
-            int tbase = 0;
-            for (int b = 0; b < s; ++b) {
-                const int lb = io.cu[b + 1] - io.cu[b] - G.wk;
-                tbase += lb > 0 ? (lb + kTileT - 1) / kTileT : 0;
-            }
-            const float invO = 1.f / (float)G.O;
-            const size_t n_el = (size_t)G.O * kTileT;
-            const int chunk = ((kPoolSmemBytes / 4) / G.O - 2 * halo) & ~3;
-            for (int c = a0; c < b0; c += chunk) {
-                const int ce = min(c + chunk, b0);
-                const int lo = max(c - halo, 0), hi = min(ce + halo, Lc), span = hi - lo;
-                const int n = G.O * span;   // mbuf[q][span]: element index q * span + (t - lo)
-                for (int base = tid; base < n; base += 8 * NT) {
-                    float m[8];
+        // The window kernel left, per group of KV heads, the maxima over the
+        // group of G_h[q][t] (q >= w - O): raw I is (1/O) times the sum over q of
+        // the maxima over the groups.  Built in shared memory chunk by chunk (with
+        // the pool halo), each (q, t) element loaded by its own thread, then pooled.
+        int tbase = 0;
+        for (int b = 0; b < s; ++b) {
+            const int lb = io.cu[b + 1] - io.cu[b] - G.wk;
+            tbase += lb > 0 ? (lb + kTileT - 1) / kTileT : 0;
+        }
+        const float invO = 1.f / (float)G.O;
+        const size_t n_el = (size_t)G.O * kTileT;
+        const int chunk = ((kPoolSmemBytes / 4) / G.O - 2 * halo) & ~3;
+        for (int c = a0; c < b0; c += chunk) {
+            const int ce = min(c + chunk, b0);
+            const int lo = max(c - halo, 0), hi = min(ce + halo, Lc), span = hi - lo;
+            const int n = G.O * span;   // mbuf[q][span]: element index q * span + (t - lo)
+            for (int base = tid; base < n; base += 8 * NT) {
+                float m[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int idx = base + u * NT;
+                    const int q = idx / span, t = lo + idx - q * span;
+                    m[u] = idx < n ? __ldcg(sl.wpart + (size_t)(tbase + (t >> 7)) * G.NG * n_el + q * kTileT + (t & 127))
+                                   : 0.f;
+                }
+                for (int gg = 1; gg < G.NG; ++gg) {
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         const int idx = base + u * NT;
                         const int q = idx / span, t = lo + idx - q * span;
-                        m[u] = idx < n ? __ldcg(sl.wpart + (size_t)(tbase + (t >> 7)) * G.NG * n_el + q * kTileT + (t & 127))
-                                       : 0.f;
+                        if (idx < n)
+                            m[u] = fmaxf(m[u], __ldcg(sl.wpart + ((size_t)(tbase + (t >> 7)) * G.NG + gg) * n_el +
+                                                       q * kTileT + (t & 127)));
                     }
-                    for (int gg = 1; gg < G.NG; ++gg) {
+                }
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int idx = base + u * NT;
-                            const int q = idx / span, t = lo + idx - q * span;
-                            if (idx < n)
-                                m[u] = fmaxf(m[u], __ldcg(sl.wpart + ((size_t)(tbase + (t >> 7)) * G.NG + gg) * n_el +
-                                                           q * kTileT + (t & 127)));
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (base + u * NT < n) mbuf[base + u * NT] = m[u];
-                }
-                __syncthreads();
-                // Sum over q in place: column tt of row 0 becomes raw I (each thread owns its columns).
-                for (int tt = tid; tt < span; tt += NT) {
-                    float sum = 0.f;
-                    for (int q = 0; q < G.O; ++q) sum += mbuf[q * span + tt];
-                    mbuf[tt] = sum * invO;
-                }
-                __syncthreads();
-                for (int t = c + tid; t < ce; t += NT) {
-                    float m = mbuf[t - lo], cnt = 1.f;
-                    for (int d = 1; d <= halo; ++d) {
-                        if (t - d >= 0) {
-                            m = avg ? m + mbuf[t - d - lo] : fmaxf(m, mbuf[t - d - lo]);
-                            cnt += 1.f;
-                        }
-                        if (t + d < Lc) {
-                            m = avg ? m + mbuf[t + d - lo] : fmaxf(m, mbuf[t + d - lo]);
-                            cnt += 1.f;
-                        }
-                    }
-                    sl.I[(size_t)s * G.ML + t] = avg ? m / cnt : m;
-                }
-                __syncthreads();
+                for (int u = 0; u < 8; ++u)
+                    if (base + u * NT < n) mbuf[base + u * NT] = m[u];
             }
+            __syncthreads();
+            // Sum over q in place: column tt of row 0 becomes raw I (each thread owns its columns).
+            for (int tt = tid; tt < span; tt += NT) {
+                float sum = 0.f;
+                for (int q = 0; q < G.O; ++q) sum += mbuf[q * span + tt];
+                mbuf[tt] = sum * invO;
+            }
+            __syncthreads();
+            for (int t = c + tid; t < ce; t += NT) {
+                float m = mbuf[t - lo], cnt = 1.f;
+                for (int d = 1; d <= halo; ++d) {
+                    if (t - d >= 0) {
+                        m = avg ? m + mbuf[t - d - lo] : fmaxf(m, mbuf[t - d - lo]);
+                        cnt += 1.f;
+                    }
+                    if (t + d < Lc) {
+                        m = avg ? m + mbuf[t + d - lo] : fmaxf(m, mbuf[t + d - lo]);
+                        cnt += 1.f;
+                    }
+                }
+                sl.I[(size_t)s * G.ML + t] = avg ? m / cnt : m;
+            }
+            __syncthreads();
         }
     }
     // The preserved-token kernel may be scheduled now; it waits for this grid before reading sigma.

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
         for (int u = u0, ul = 0; u < units; u += ustep, ++ul) {
             WinUnit wu;
             const int lay = u / upl;
-                decode_unit(G, cu_dev, u - lay * upl, wu);
+            decode_unit(G, cu_dev, u - lay * upl, wu);
             const Slot& sl = A.sl[lay];
             const int h0 = wu.ng * G.HG, nh = min(G.HG, G.Hkv - h0);
             const int t = wu.jt * kTileT + tok;                  // token within the sequence
