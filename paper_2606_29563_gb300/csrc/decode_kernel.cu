@@ -41,6 +41,9 @@ namespace cg = cooperative_groups;
 constexpr int kDecBlock = 8;                          // cached rows per ring stage
 constexpr int kDecStageBytes = 2 * kDecBlock * kHeadDim * 2;   // K rows, then V rows
 constexpr int kDecMaxSplits = 8;                      // CTAs per (sequence, KV head): a portable cluster
+// The maximum before the first logit: the lowest finite value, so that a logit of minus
+// infinity gets the weight 2^-inf = 0 there too, and not 2^(-inf + inf).
+constexpr float kNoLogit = -3.402823466e38f;
 
 struct DecArgs {
     const __nv_bfloat16* q;      // [batch][Hq][d]
@@ -163,9 +166,7 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
         for (int c = 0; c < 4; ++c) acc[j][c] = 0ull;
     // This lane's logits: row lane / 4 of the block, heads j0 and j0 + 1.
     const int xr = lane >> 2, j0 = 2 * (lane & 3);
-    // Maxima, what the weights refer to (0 while every row so far has a logit of
-    // minus infinity, whose weight is then 0 and not 2^(inf - inf)), and sums.
-    float m[2] = {-INFINITY, -INFINITY}, ref[2] = {0.f, 0.f}, l[2] = {0.f, 0.f};
+    float m[2] = {kNoLogit, kNoLogit}, l[2] = {0.f, 0.f};
     int st = 0;
     for (int b = b0; b < b_end; b += kDecWarps) {
         cp_async_wait<ST - 2>();
@@ -196,8 +197,7 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
             float corr[2];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                ref[c] = mn[c] == -INFINITY ? 0.f : mn[c];
-                corr[c] = ptx::ex2(m[c] - ref[c]);   // 0 while m is -inf
+                corr[c] = ptx::ex2(m[c] - mn[c]);   // 0 from kNoLogit on
                 l[c] *= corr[c];
                 m[c] = mn[c];
             }
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
         }
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            x[c] = ptx::ex2(x[c] - ref[c]);
+            x[c] = ptx::ex2(x[c] - m[c]);
             l[c] += x[c];
         }
         if (j0 < GP) {
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
         float L = 0.f, O = 0.f;
 #pragma unroll
         for (int w = 0; w < kDecWarps; ++w) {
-            if (wm[w][j] == -INFINITY) continue;   // no rows
+            if (wm[w][j] == kNoLogit) continue;   // no row with a logit above minus infinity
             const float e = ptx::ex2(wm[w][j] - M);
             L = fmaf(e, wl[w][j], L);
             O = fmaf(e, reinterpret_cast<const float*>(dec_smem)[((size_t)w * GP + j) * kHeadDim + c], O);
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(C::kThreads, C::NC) decode_kernel(const __grid
         float L = 0.f, O = 0.f;
 #pragma unroll
         for (int r = 0; r < kDecMaxSplits; ++r) {
-            if (mc[r] == -INFINITY) continue;
+            if (mc[r] <= kNoLogit) continue;
             const float e = ptx::ex2(mc[r] - M);
             L = fmaf(e, *cluster.map_shared_rank(&cl[j], r), L);
             O = fmaf(e, *cluster.map_shared_rank(&co[j][c], r), O);
