@@ -245,6 +245,12 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
     // refused call leaves the state as it was.
     const bool refuse = A.l0 == 0 ? ell0 + (uint32_t)A.ncall > 255u : __ldcg(&A.refused[s]) != 0;
     if (A.l0 == 0 && h == 0 && tid == 0) A.refused[s] = refuse ? 1 : 0;
+    if (refuse) {   // the same for the whole cluster
+        // What follows on the stream waits for this grid alone, which so waits too.
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
+        if (tid == 0) atomicExch(A.err, 2);
+        return;
+    }
     uint32_t n4[kStageI ? KPT / 4 : 1];   // counts of this thread's positions, four bytes a word
     auto counts = [&](int g) -> uint32_t& {
         if constexpr (kStageI) return n4[g];
@@ -256,13 +262,8 @@ __global__ void __launch_bounds__(NT, 1) chain_kernel(const __grid_constant__ Ch
         counts(g) = t < L ? __ldcg(reinterpret_cast<const uint32_t*>(nst + t)) : 0u;
     }
     // The state is the previous call's, complete before this call's first kernel began;
-    // the scores come from the kernels before this one.  A refused sequence waits for
-    // them too: what follows this grid on the stream waits for this grid alone.
+    // the scores come from the kernels before this one.
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    if (refuse) {   // the same for the whole cluster
-        if (tid == 0) atomicExch(A.err, 2);
-        return;
-    }
     uint32_t top = 0u;   // bit l: the head takes O' in layer l
     for (int l = 0; l < A.nl; ++l) top |= (__ldg(&A.sl[l].htop[row]) != 0 ? 1u : 0u) << l;
     // A layer's scores P and importance I come by bulk copies into shared memory, issued
